@@ -19,12 +19,24 @@
 //   k_cmp_logdet   one thread block per component: sum of log s_k in a fixed
 //                  order.
 //   k_cmp_scatter  the given entries into the dense blocks.
-//   k_cmp_step     one launch per step of the recurrence (the launches are
-//                  captured once into a CUDA graph and replayed); within a step each
-//                  thread owns one later vertex j of one component (all
-//                  components advance together, aligned at their last
-//                  vertex), reads rows N_k of the block at column j
+//   k_cmp_rows     patterns with a full profile (below): every row of the
+//                  completion is a chain of its own, so one launch runs all of
+//                  them side by side.
+//   k_cmp_step     other patterns: one launch per step of the recurrence (the
+//                  launches are captured once into a CUDA graph and replayed);
+//                  within a step each thread owns one later vertex j of one
+//                  component (all components advance together, aligned at
+//                  their last vertex), reads rows N_k of the block at column j
 //                  (coalesced) and writes W[v_k, j] and W[j, v_k].
+//
+// Full profile: for every vertex u, all vertices eliminated between the first
+// one that has u among its later neighbours and u itself have u among theirs
+// (the Cholesky factor has no zeros inside its row envelope; bands and
+// block-arrows in their own order are like that).  Then in
+// W[j, v_k] = W[j, N_k] t_k an element u of N_k eliminated after j has the
+// given entry (u, j), and one eliminated before j was computed by the same
+// row j: row j needs nothing from other rows.  Without that property rows
+// exchange computed entries, and the steps have to stay in order.
 // The dense output holds one row-major n_c x n_c block per component
 // (independent components complete independently; entries between them are
 // zero), vertices of a block in ascending order.
@@ -34,6 +46,7 @@
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "cdsdp_internal.h"
@@ -43,6 +56,11 @@ namespace {
 
 constexpr size_t kCmpAlign = 256;
 constexpr int kStepThreads = 256;
+constexpr int kRowWarps = 2, kRowsPerWarp = 8;  // k_cmp_rows: 8 rows a warp, 4 lanes a row
+constexpr int kRowThreads = 32 * (kRowWarps + 1);  // and one warp that stages the recurrence coefficients
+constexpr int kRowRing = 64;    // latest entries of a row kept in shared memory
+constexpr int kRowFar = 8;      // prefetched older entries per lane
+constexpr int kRowTerms = 1024; // coefficients per stage (at least one step)
 constexpr size_t kMaxWarpSmem = 200 * 1024;  // largest shared block per warp of the factor kernel
 
 inline size_t align_up(size_t x) { return (x + kCmpAlign - 1) / kCmpAlign * kCmpAlign; }
@@ -50,9 +68,12 @@ inline size_t align_up(size_t x) { return (x + kCmpAlign - 1) / kCmpAlign * kCmp
 // Scratch layout (byte offsets, all 256-aligned).  The index section [0, idx_end)
 // is copied from the host image; the rest is written by the kernels.
 struct CmpLayout {
-    size_t lt_ptr, lt_idx, colptr, prow, pcol, comp, loc, posl, peo_cat, peo_off, woff, idx_end;
+    size_t lt_ptr, lt_idx, colptr, prow, pcol, comp, loc, posl, peo_cat, peo_off, woff, lt_pos, lt_loc, first, rowblk,
+        idx_end;
     size_t T, schur, logdet, flag, total;
     int smax = 0, ncomp = 0, maxnc = 0;
+    int nrowblk = 0;       // blocks of k_cmp_rows
+    bool profile = false;  // full profile: rows are independent
     long long welems = 0;
 };
 
@@ -72,6 +93,13 @@ CmpLayout cmp_layout(const HostProblem& hp) {
     L.peo_cat = take(n * 4);
     L.peo_off = take((C + 1) * 4);
     L.woff = take(C * 8);
+    std::vector<int> cnt(C, 0);
+    for (int v = 0; v < hp.n; ++v) ++cnt[hp.comp_of_vertex[v]];
+    for (int nc : cnt) L.nrowblk += (nc + kRowWarps * kRowsPerWarp - 1) / (kRowWarps * kRowsPerWarp);
+    L.lt_pos = take(nl * 4);
+    L.lt_loc = take(nl * 4);
+    L.first = take(n * 4);
+    L.rowblk = take((size_t)L.nrowblk * 8);
     L.idx_end = o;
     L.T = take(nl * 8);
     L.schur = take(n * 8);
@@ -84,7 +112,7 @@ CmpLayout cmp_layout(const HostProblem& hp) {
 }
 
 // Host image of the index section, and the per-component block offsets.
-void cmp_image(const HostProblem& hp, const CmpLayout& L, std::vector<unsigned char>& img,
+void cmp_image(const HostProblem& hp, CmpLayout& L, std::vector<unsigned char>& img,
                std::vector<long long>& woff_out, int& maxnc) {
     const int n = hp.n, C = hp.ncomp;
     img.assign(L.idx_end, 0);
@@ -117,6 +145,37 @@ void cmp_image(const HostProblem& hp, const CmpLayout& L, std::vector<unsigned c
     put(L.peo_cat, peo_cat.data(), n * 4);
     put(L.peo_off, peo_off.data(), (C + 1) * 4);
     put(L.woff, woff_out.data(), C * 8);
+    // k_cmp_rows: elimination position and local index of every later
+    // neighbour; per position, the first position whose list holds it (itself
+    // when none does); the row blocks, longest chains first
+    std::vector<int> lpos(hp.lt_idx.size()), lloc(hp.lt_idx.size()), first(n), seen(n, 0);
+    for (int c = 0; c < C; ++c)
+        for (int q = peo_off[c]; q < peo_off[c + 1]; ++q) first[q] = q - peo_off[c];
+    for (int k = 0; k < n; ++k) {
+        const int v = hp.peo[k], q0 = peo_off[hp.comp_of_vertex[v]];
+        for (int e = hp.lt_ptr[v]; e < hp.lt_ptr[v + 1]; ++e) {
+            const int u = hp.lt_idx[e], qu = q0 + posl[u];
+            lpos[e] = posl[u];
+            lloc[e] = loc[u];
+            first[qu] = std::min(first[qu], posl[v]);
+            ++seen[qu];
+        }
+    }
+    L.profile = true;
+    for (int c = 0; c < C; ++c)
+        for (int q = peo_off[c]; q < peo_off[c + 1]; ++q)
+            if (seen[q] != (q - peo_off[c]) - first[q]) L.profile = false;
+    std::vector<std::pair<int, int>> blk;  // (component, first row position)
+    for (int c = 0; c < C; ++c)
+        for (int r = 0; r < cnt[c]; r += kRowWarps * kRowsPerWarp) blk.emplace_back(c, r);
+    std::stable_sort(blk.begin(), blk.end(),
+                     [](const std::pair<int, int>& a, const std::pair<int, int>& b) { return a.second > b.second; });
+    std::vector<int> flat;
+    for (const auto& b : blk) { flat.push_back(b.first); flat.push_back(b.second); }
+    put(L.lt_pos, lpos.data(), lpos.size() * 4);
+    put(L.lt_loc, lloc.data(), lloc.size() * 4);
+    put(L.first, first.data(), n * 4);
+    put(L.rowblk, flat.data(), flat.size() * 4);
 }
 
 // Pattern value of entry (i, j): binary search of max(i, j) among the rows of
@@ -276,6 +335,181 @@ __global__ void __launch_bounds__(kStepThreads) k_cmp_step(int n, int r, const i
     Wc[lj * ncz + lv] = acc;
 }
 
+// All rows of a full-profile completion (see the top of the file).  A block
+// takes 16 consecutive elimination positions of one component, 8 rows a warp;
+// the rows walk the positions k = (last row) - 1 .. 0 together, so that the
+// coefficients t_k and the indices N_k are the same for all of them and one
+// more warp stages them in shared memory, a stage ahead.  The 4 lanes of a row
+// split the dot product W[j, N_k] t_k: elements of N_k at most 64 positions
+// away come from a ring in shared memory, older ones (or, for rows past the
+// element, given ones) from the dense block, loaded one step ahead; the loads
+// of a step are 8 consecutive entries per element.
+//
+// Bound: the dependent chain of a row (n steps of a few float64 multiply-adds
+// and two shuffles, 0.4 us a step), not bandwidth: 8 n^2 bytes are written
+// once.  4 lanes a row and 16 rows a block put a chain on nearly every SM at
+// n = 2000 (125 blocks).  Banded n = 2000, w = 10, whole call: 8.73 ms as
+// 1999 dependent launches of k_cmp_step, 1.13 ms with this kernel (0.80 ms of
+// it here).  A row past an element's position may read an entry of the dense
+// block that nothing has written: by the profile property it is never used.
+struct RowArgs {
+    const int *lt_ptr, *lt_pos, *lt_loc, *loc, *peo_cat, *peo_off, *first, *rowblk;
+    const long long* woff;
+    const double* T;
+    double* W;
+    int smax, nstep;  // longest later-neighbour list; steps per stage
+};
+
+// A staged coefficient: t_k[a], and where its W[j, u] is: an offset into the
+// ring, or (ring < 0) the local index `far` of u in the dense block.  Unused
+// terms have t = 0 and the offset of the ring's row of zeros.
+struct alignas(16) RowTerm {
+    double t;
+    int ring, far;
+};
+
+// U: terms per lane and step (4 U >= the longest list), 0: smax as given.
+template <int U>
+__global__ void __launch_bounds__(kRowThreads) k_cmp_rows(RowArgs g) {
+    extern __shared__ __align__(16) unsigned char row_smem[];
+    __shared__ double ring[kRowWarps][(kRowRing + 1) * kRowsPerWarp];  // [position & 63][row], then zeros
+    __shared__ int step_loc[2][32], step_far[2][32];  // local index of v_k; some term of the step is far
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int nt = U > 0 ? 4 * U : (g.smax + 3) & ~3, cap = nt * g.nstep;  // terms of a step, of a stage
+    RowTerm* st = reinterpret_cast<RowTerm*>(row_smem);                    // [2][cap]
+    const int c = g.rowblk[2 * blockIdx.x], r0 = g.rowblk[2 * blockIdx.x + 1];
+    const int q0 = g.peo_off[c], nc = g.peo_off[c + 1] - q0;
+    const int kmax = min(r0 + kRowWarps * kRowsPerWarp, nc) - 2;  // highest position any row of the block needs
+    const int nstage = (kmax + g.nstep) / g.nstep;
+    double* Wc = g.W + g.woff[c];
+    // rows of the computing warps
+    const int sub = lane & 3, row = lane >> 2;
+    const int pj = min(r0 + kRowsPerWarp * warp + row, nc - 1);
+    const bool live = warp < kRowWarps && r0 + kRowsPerWarp * warp + row < nc;
+    const size_t lj = g.loc[g.peo_cat[q0 + pj]], ncz = nc;
+    const int fj = g.first[q0 + pj];
+    int fmin = fj;  // below it every row of the warp computes
+    for (int o = 4; o < 32; o <<= 1) fmin = min(fmin, __shfl_xor_sync(0xffffffffu, fmin, o));
+    double* rg = ring[warp < kRowWarps ? warp : 0] + row;
+    if (warp < kRowWarps) {  // ring: the entries at positions kmax + 1 .. kmax + 64 (given ones among them)
+        for (int i = sub; i < kRowRing; i += 4) {
+            const int p = kmax + 1 + i;
+            if (p < nc) rg[(p & (kRowRing - 1)) * kRowsPerWarp] = Wc[(size_t)g.loc[g.peo_cat[q0 + p]] * ncz + lj];
+        }
+        if (sub == 0) rg[kRowRing * kRowsPerWarp] = 0.0;
+    }
+    auto stage = [&](int s) {  // the staging warp: coefficients of stage s into its half
+        const int b = s & 1, k = kmax - s * g.nstep - lane;  // lane i: step i of the stage
+        int beg = 0, sv = 0, any = 0;
+        if (lane < g.nstep && k >= 0) {
+            const int v = g.peo_cat[q0 + k];
+            beg = g.lt_ptr[v];
+            sv = g.lt_ptr[v + 1] - beg;
+            step_loc[b][lane] = g.loc[v];
+        }
+        for (int f0 = 0; f0 < cap; f0 += 8 * 32) {  // eight coefficients a lane in flight
+            double t[8];
+            int p[8], l[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int f = f0 + 32 * u + lane, i = f / nt, a = f - i * nt;
+                const int bi = __shfl_sync(0xffffffffu, beg, i & 31), si = __shfl_sync(0xffffffffu, sv, i & 31);
+                const bool ok = f < cap && a < si;
+                t[u] = ok ? g.T[bi + a] : 0.0;
+                p[u] = ok ? g.lt_pos[bi + a] : -1;
+                l[u] = ok ? g.lt_loc[bi + a] : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int f = f0 + 32 * u + lane, i = f / nt, ki = kmax - s * g.nstep - i;
+                const bool far = p[u] - ki > kRowRing;
+                if (f < cap)
+                    st[b * cap + f] = RowTerm{t[u], far ? -1 : (p[u] < 0 ? kRowRing : p[u] & (kRowRing - 1)) * kRowsPerWarp, l[u]};
+                if (far) any |= 1u << (i & 31);
+            }
+        }
+        any = __reduce_or_sync(0xffffffffu, any);
+        step_far[b][lane] = (any >> lane) & 1;
+    };
+    if (warp == kRowWarps && nstage > 0) stage(0);
+    __syncthreads();
+    constexpr int NF = U > 0 ? U : kRowFar;
+    for (int s = 0; s < nstage; ++s) {
+        if (warp == kRowWarps) {
+            if (s + 1 < nstage) stage(s + 1);
+        } else {
+            const int b = s & 1, k0 = kmax - s * g.nstep, ns = min(g.nstep, k0 + 1);
+            const RowTerm* e0 = st + b * cap + sub;
+            double far[NF];
+            auto load_far = [&](int i) {  // the far entries of step i (older than 64 steps, or given)
+#pragma unroll
+                for (int u = 0; u < NF; ++u) {
+                    if (U == 0 && 4 * u >= nt) break;
+                    const RowTerm e = e0[i * nt + 4 * u];
+                    far[u] = e.ring < 0 ? Wc[(size_t)e.far * ncz + lj] : 0.0;
+                }
+            };
+            if (step_far[b][0]) load_far(0);
+            for (int i = 0; i < ns; ++i) {
+                const int k = k0 - i;
+                const size_t lk = step_loc[b][i];
+                const RowTerm* e = e0 + i * nt;
+                double acc = 0.0;
+                if (step_far[b][i]) {
+#pragma unroll
+                    for (int u = 0; u < NF; ++u) {
+                        if (U == 0 && 4 * u >= nt) break;
+                        acc += (e[4 * u].ring < 0 ? far[u] : rg[max(e[4 * u].ring, 0)]) * e[4 * u].t;
+                    }
+                } else {
+#pragma unroll
+                    for (int u = 0; u < NF; ++u) {
+                        if (U == 0 && 4 * u >= nt) break;
+                        acc += rg[e[4 * u].ring] * e[4 * u].t;
+                    }
+                }
+                if (U == 0)
+                    for (int u = kRowFar; 4 * u < nt; ++u) {
+                        const RowTerm x = e[4 * u];
+                        acc += (x.ring < 0 ? Wc[(size_t)x.far * ncz + lj] : rg[x.ring]) * x.t;
+                    }
+                acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+                acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+                bool given = false;  // (j, v_k) is in the pattern, or v_k is not eliminated before j
+                if (k >= fmin) {
+                    given = k >= fj;
+                    if (given) acc = Wc[lk * ncz + lj];
+                }
+                if (sub == 0) rg[(k & (kRowRing - 1)) * kRowsPerWarp] = acc;
+                if (!given && live) {
+                    if (sub == 0) Wc[lk * ncz + lj] = acc;
+                    if (sub == 1) Wc[lj * ncz + lk] = acc;
+                }
+                __syncwarp();
+                if (i + 1 < ns && step_far[b][i + 1]) load_far(i + 1);
+            }
+        }
+        __syncthreads();
+    }
+}
+
+cudaError_t launch_rows(const RowArgs& a, int blocks, cudaStream_t st) {
+    const int U = (a.smax + 3) / 4;
+    const size_t smem = 2 * sizeof(RowTerm) * (size_t)(4 * U) * a.nstep;  // at most 32 KB
+    switch (U <= kRowFar ? U : 0) {
+        case 1: k_cmp_rows<1><<<blocks, kRowThreads, smem, st>>>(a); break;
+        case 2: k_cmp_rows<2><<<blocks, kRowThreads, smem, st>>>(a); break;
+        case 3: k_cmp_rows<3><<<blocks, kRowThreads, smem, st>>>(a); break;
+        case 4: k_cmp_rows<4><<<blocks, kRowThreads, smem, st>>>(a); break;
+        case 5: k_cmp_rows<5><<<blocks, kRowThreads, smem, st>>>(a); break;
+        case 6: k_cmp_rows<6><<<blocks, kRowThreads, smem, st>>>(a); break;
+        case 7: k_cmp_rows<7><<<blocks, kRowThreads, smem, st>>>(a); break;
+        case 8: k_cmp_rows<8><<<blocks, kRowThreads, smem, st>>>(a); break;
+        default: k_cmp_rows<0><<<blocks, kRowThreads, smem, st>>>(a);
+    }
+    return cudaGetLastError();
+}
+
 int cuda_fail(std::string* err, cudaError_t e, const char* what) {
     if (err) *err = std::string(what) + ": " + cudaGetErrorString(e);
     cudaGetLastError();
@@ -292,7 +526,7 @@ void completion_release(CmpGraph& g) {
 }
 
 int completion_sizes(const HostProblem& hp, size_t* scratch_bytes, long long* w_elems, long long* w_offsets) {
-    const CmpLayout L = cmp_layout(hp);
+    CmpLayout L = cmp_layout(hp);
     std::vector<unsigned char> img;
     std::vector<long long> woff;
     int maxnc = 0;
@@ -307,7 +541,7 @@ int completion_run(const HostProblem& hp, const double* d_X, void* d_scratch, si
                    double* logdet, void* stream, std::string* err, CmpGraph* cache) {
     if (!d_X || !d_scratch) return CDSDP_ERR_ARG;
     if (reinterpret_cast<uintptr_t>(d_scratch) % kCmpAlign) return CDSDP_ERR_ARG;
-    const CmpLayout L = cmp_layout(hp);
+    CmpLayout L = cmp_layout(hp);
     if (scratch_bytes < L.total) return CDSDP_ERR_NOMEM;
     const int ld = std::max(1, L.smax);
     const size_t per_warp = (size_t)(ld * ld + 2 * ld) * sizeof(double);
@@ -369,7 +603,23 @@ int completion_run(const HostProblem& hp, const double* d_X, void* d_scratch, si
                                                         dwoff, T, d_W);
             return cudaGetLastError();
         };
-        if (!cache || maxnc < 2) {
+        if (L.profile) {  // rows are independent: one launch
+            RowArgs ra;
+            ra.lt_ptr = lt_ptr;
+            ra.lt_pos = (const int*)(g + L.lt_pos);
+            ra.lt_loc = (const int*)(g + L.lt_loc);
+            ra.loc = loc;
+            ra.peo_cat = peo_cat;
+            ra.peo_off = peo_off;
+            ra.first = (const int*)(g + L.first);
+            ra.rowblk = (const int*)(g + L.rowblk);
+            ra.woff = dwoff;
+            ra.T = T;
+            ra.W = d_W;
+            ra.smax = std::max(1, L.smax);
+            ra.nstep = std::max(1, std::min(32, kRowTerms / ((ra.smax + 3) / 4 * 4)));
+            CMP_CK(launch_rows(ra, L.nrowblk, st));
+        } else if (!cache || maxnc < 2) {
             CMP_CK(steps(st));
         } else {
             if (!cache->exec || cache->scratch != d_scratch || cache->W != d_W) {
