@@ -23,7 +23,7 @@ namespace {
 //   lamprev <- lambar - Wbar / rho
 template <typename T, int S>
 __global__ void __launch_bounds__(128) k_bwd_proj(Dev d, const int* __restrict__ list, int nlist, GradArgs ga) {
-    using J = BLJacobi<T, S>;
+    using J = BLJacobi<T, S, 32, true>;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     J jac;
@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(128) k_bwd_proj(Dev d, const int* __restrict__
     for (int li = blockIdx.x * wpb + warp; li < nlist; li += gridDim.x * wpb) {
         const int k = list[li];
         const int s = d.csize[k], off = d.pk_off[k], npk = s * (s + 1) / 2;
-        jac.clear(lane);
+        jac.clear(lane, s);
         T nrm = T(0);
         for (int f = lane; f < npk; f += 32) {
             const int ab = packed_ab(f, s), a = ab >> 8, b = ab & 255;
@@ -43,9 +43,9 @@ __global__ void __launch_bounds__(128) k_bwd_proj(Dev d, const int* __restrict__
         }
         nrm = warp_sum(nrm);
         __syncwarp();
-        jac.run(T(ga.tolrel) * sqrt(nrm), ga.max_sweeps, lane, false);
+        jac.run(T(ga.tolrel) * sqrt(nrm), ga.max_sweeps, lane, inv_norm(nrm));
         const T lam_lane = lane < S ? jac.X[lane * J::LDA + lane] : T(0);
-        jac.clear(lane);
+        jac.clear(lane, 0);
         if (lane < S) jac.Y[lane * J::LDA + S] = lam_lane;  // padding column: survives the congruences
         for (int f = lane; f < npk; f += 32) {
             const int ab = packed_ab(f, s), a = ab >> 8, b = ab & 255;

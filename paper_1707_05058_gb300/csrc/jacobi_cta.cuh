@@ -604,7 +604,7 @@ __device__ __forceinline__ void cta_sum(double (&v)[NV], double* sh) {
 // kernels of jacobi.cuh), FORM 3 = standalone projection; VARIANT selects the
 // solver (CTAPick).
 template <typename T, int S, int FORM, int VARIANT>
-__global__ void __launch_bounds__(CTAPick<T, S, VARIANT>::threads, CTAPick<T, S, VARIANT>::min_blocks) k_project_cta(Dev d, const int* __restrict__ list, int nlist, ProjArgs pa,
+__global__ void __launch_bounds__(CTAPick<T, S, VARIANT>::threads, CTAPick<T, S, VARIANT>::min_blocks) k_project_cta(Dev d, const int4* __restrict__ list, int nlist, ProjArgs pa,
                                                               FinishArgs fa, const int* __restrict__ off_arr,
                                                               const int* __restrict__ size_arr,
                                                               const T* __restrict__ Win, T* Xout) {
@@ -628,9 +628,8 @@ __global__ void __launch_bounds__(CTAPick<T, S, VARIANT>::threads, CTAPick<T, S,
     __shared__ double ck_d[3];
     if (tid < 6) acc[tid] = 0.0;
     for (int li = blockIdx.x; li < nlist; li += gridDim.x) {
-        const int k = FORM == 3 ? li : list[li];
-        const int s = FORM == 3 ? size_arr[k] : d.csize[k];
-        const int off = FORM == 3 ? off_arr[k] : d.pk_off[k];
+        const int4 rec = FORM == 3 ? make_int4(li, size_arr[li], off_arr[li], 0) : list[li];
+        const int k = rec.x, s = rec.y, off = rec.z;
         if (s > S || s < 1) continue;  // block-uniform
         if (FORM != 3 && frozen_clique(d, k)) continue;
         const double rho = (FORM == 0 || FORM == 1) ? rho_clique(d, k) : 1.0, irho = 1.0 / rho;

@@ -11,7 +11,7 @@ namespace cdsdp_dev {
 namespace {
 
 template <typename T, int S, int FORM, int VARIANT>
-cudaError_t launch_cta_v(const Dev& d, const int* list, int nlist, const ProjArgs& pa_in, const FinishArgs& fa,
+cudaError_t launch_cta_v(const Dev& d, const int4* list, int nlist, const ProjArgs& pa_in, const FinishArgs& fa,
                          const int* off, const int* size, const void* W, void* X, int max_sweeps, cudaStream_t st) {
     using Pick = CTAPick<T, S, VARIANT>;
     const size_t smem = Pick::type::bytes;
@@ -37,7 +37,7 @@ cudaError_t launch_cta_v(const Dev& d, const int* list, int nlist, const ProjArg
 
 // pa.cta_variant = 1 selects variant 1 (V in registers) for float32 orders 36..64.
 template <typename T, int S, int FORM>
-cudaError_t launch_cta(const Dev& d, const int* list, int nlist, const ProjArgs& pa, const FinishArgs& fa,
+cudaError_t launch_cta(const Dev& d, const int4* list, int nlist, const ProjArgs& pa, const FinishArgs& fa,
                        const int* off, const int* size, const void* W, void* X, int max_sweeps, cudaStream_t st) {
     if (nlist <= 0) return cudaSuccess;
     if constexpr (sizeof(T) == 4 && S >= 36 && S <= 64) {
@@ -48,7 +48,7 @@ cudaError_t launch_cta(const Dev& d, const int* list, int nlist, const ProjArgs&
 }
 
 template <typename T, int S>
-cudaError_t launch_cta_form(int form, const Dev& d, const int* list, int nlist, const ProjArgs& pa,
+cudaError_t launch_cta_form(int form, const Dev& d, const int4* list, int nlist, const ProjArgs& pa,
                             const FinishArgs& fa, cudaStream_t st) {
     switch (form) {
         case 0: return launch_cta<T, S, 0>(d, list, nlist, pa, fa, nullptr, nullptr, nullptr, nullptr, 0, st);
@@ -59,7 +59,7 @@ cudaError_t launch_cta_form(int form, const Dev& d, const int* list, int nlist, 
 
 }  // namespace
 
-cudaError_t CTA_SUFFIX(launch_proj_cta)(int S, int form, const Dev& d, const int* list, int nlist,
+cudaError_t CTA_SUFFIX(launch_proj_cta)(int S, int form, const Dev& d, const int4* list, int nlist,
                                         const ProjArgs& pa, const FinishArgs& fa, cudaStream_t st) {
     switch (S) {
 #define CTA_CASE(N) \

@@ -9,7 +9,7 @@ namespace cdsdp_dev {
 namespace {
 
 template <typename T, int S>
-cudaError_t launch_form(int form, const Dev& d, const int* list, int nlist, const ProjArgs& pa_in,
+cudaError_t launch_form(int form, const Dev& d, const int4* list, int nlist, const ProjArgs& pa_in,
                         const FinishArgs& fa, cudaStream_t st) {
     if (nlist <= 0) return cudaSuccess;
     constexpr int MW = proj_max_warps(S, sizeof(T) == 4);
@@ -20,13 +20,15 @@ cudaError_t launch_form(int form, const Dev& d, const int* list, int nlist, cons
     const size_t smem_max = (size_t)MW * G * J::bytes;
     ProjArgs pa = pa_in;
     pa.tolrel = jacobi_tolrel(S, sizeof(T) == 4);
-    static bool attr_done[3] = {false, false, false};  // per instantiation; setting twice is harmless
+    static bool attr_done[4] = {false, false, false, false};  // per instantiation; setting twice is harmless
     cudaError_t e = cudaSuccess;
     if (form == 0) {
-        if (!attr_done[0]) e = cudaFuncSetAttribute(k_project_primal<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
+        const auto kernel = pa.unrolled ? k_project_primal<T, S, true> : k_project_primal<T, S, false>;
+        bool& done = attr_done[pa.unrolled ? 3 : 0];
+        if (!done) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
         if (e != cudaSuccess) return e;
-        attr_done[0] = true;
-        k_project_primal<T, S><<<sh.grid, 32 * sh.wpb, smem, st>>>(d, list, nlist, pa, fa);
+        done = true;
+        kernel<<<sh.grid, 32 * sh.wpb, smem, st>>>(d, list, nlist, pa, fa);
     } else if (form == 1) {
         if (!attr_done[1]) e = cudaFuncSetAttribute(k_project_dual<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
         if (e != cudaSuccess) return e;
@@ -82,7 +84,7 @@ cudaError_t launch_standalone(int p, const int* off, const int* size, const void
 
 }  // namespace
 
-cudaError_t PROJ_SUFFIX(launch_proj)(int form, int cls, const Dev& d, const int* list, int nlist, const ProjArgs& pa,
+cudaError_t PROJ_SUFFIX(launch_proj)(int form, int cls, const Dev& d, const int4* list, int nlist, const ProjArgs& pa,
                                      const FinishArgs& fa, cudaStream_t st) {
 #define CALL(S) launch_form<PROJ_T, S>(form, d, list, nlist, pa, fa, st)
     CDSDP_CLASS_SWITCH(CALL)

@@ -25,6 +25,10 @@ __host__ __device__ constexpr int proj_lanes(int S) { return S <= 8 ? 8 : (S <= 
 // (registers: 16 warps only while a thread needs <= 128 registers).
 __host__ __device__ constexpr int proj_max_warps(int S, bool fp32) { return S <= 16 ? 16 : (fp32 ? 8 : 4); }
 
+// Where the Jacobi sweeps of a solve end: theta of BLJacobi::run over the
+// threshold on single entries.
+constexpr double kThetaSolve = 0.25;
+
 // Launch shape of a projection over `nlist` cliques, one clique per warp:
 // the grid is a multiple of the 152 SMs when it can be, and blocks are made as
 // wide as allowed so that every SM receives the same number of warps.
@@ -47,12 +51,13 @@ inline int proj_class_of(int s) {
     return -1;
 }
 
-// form 0/1/2: Algorithm 1/2/3 projection kernels over `list` (cliques of
-// order <= kProjClasses[cls]).
+// form 0/1/2: Algorithm 1/2/3 projection kernels over `list`: per clique of
+// order <= kProjClasses[cls] its (index, order, packed offset, component), one
+// 16-byte load instead of a chain of three.
 // `fa` is used by the primal form only (its last block finishes the iteration).
 // Instantiations live in proj_{f32,f64}_{small,large}.cu (orders 2..16 / 20..32).
 #define CDSDP_DECLARE_PROJ(SUF)                                                                                 \
-    cudaError_t launch_proj_##SUF(int form, int cls, const Dev& d, const int* list, int nlist,                 \
+    cudaError_t launch_proj_##SUF(int form, int cls, const Dev& d, const int4* list, int nlist,                 \
                                   const ProjArgs& pa, const FinishArgs& fa, cudaStream_t st);                    \
     cudaError_t launch_proj_standalone_##SUF(int cls, int p, const int* off, const int* size, const void* W,   \
                                              void* X, void* eig, const int* voff, void* V, const int* vvoff,  \
@@ -66,7 +71,7 @@ CDSDP_DECLARE_PROJ(f64_large)
 // Thread-block-per-clique kernels, instantiated in proj_cta_{f32a,f32b,f32c,f64a,f64b}.cu
 // (padded orders 36..48, 52..64, 96..128 in float; 36..48, 52..64 in double).
 #define CDSDP_DECLARE_CTA(SUF)                                                                                  \
-    cudaError_t launch_proj_cta_##SUF(int S, int form, const Dev& d, const int* list, int nlist,               \
+    cudaError_t launch_proj_cta_##SUF(int S, int form, const Dev& d, const int4* list, int nlist,               \
                                       const ProjArgs& pa, const FinishArgs& fa, cudaStream_t st);                \
     cudaError_t launch_proj_cta_standalone_##SUF(int S, int p, const int* off, const int* size, const void* W, \
                                                  void* X, int max_sweeps, int variant, cudaStream_t st);
@@ -77,7 +82,7 @@ CDSDP_DECLARE_CTA(f64a)
 CDSDP_DECLARE_CTA(f64b)
 #undef CDSDP_DECLARE_CTA
 
-inline cudaError_t launch_proj_cta(bool fp32, int form, int cls, const Dev& d, const int* list, int nlist,
+inline cudaError_t launch_proj_cta(bool fp32, int form, int cls, const Dev& d, const int4* list, int nlist,
                                    const ProjArgs& pa, const FinishArgs& fa, cudaStream_t st) {
     const int S = kProjClasses[cls];
     if (fp32)
@@ -98,13 +103,13 @@ inline cudaError_t launch_proj_cta_standalone(bool fp32, int cls, int p, const i
                    : launch_proj_cta_standalone_f64b(S, p, off, size, W, X, max_sweeps, 0, st);
 }
 
-inline cudaError_t launch_proj_f32(int form, int cls, const Dev& d, const int* list, int nlist, const ProjArgs& pa,
+inline cudaError_t launch_proj_f32(int form, int cls, const Dev& d, const int4* list, int nlist, const ProjArgs& pa,
                                    const FinishArgs& fa, cudaStream_t st) {
     if (kProjClasses[cls] > kMaxWarpOrder) return launch_proj_cta(true, form, cls, d, list, nlist, pa, fa, st);
     return kProjClasses[cls] <= 16 ? launch_proj_f32_small(form, cls, d, list, nlist, pa, fa, st)
                                    : launch_proj_f32_large(form, cls, d, list, nlist, pa, fa, st);
 }
-inline cudaError_t launch_proj_f64(int form, int cls, const Dev& d, const int* list, int nlist, const ProjArgs& pa,
+inline cudaError_t launch_proj_f64(int form, int cls, const Dev& d, const int4* list, int nlist, const ProjArgs& pa,
                                    const FinishArgs& fa, cudaStream_t st) {
     if (kProjClasses[cls] > kMaxWarpOrder) return launch_proj_cta(false, form, cls, d, list, nlist, pa, fa, st);
     return kProjClasses[cls] <= 16 ? launch_proj_f64_small(form, cls, d, list, nlist, pa, fa, st)

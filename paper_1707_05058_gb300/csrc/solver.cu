@@ -35,7 +35,7 @@ inline int class_of(int s) { return proj_class_of(s); }
 struct Layout {
     // constants
     size_t c, dinv, pinv, wgt, a_ptr, a_col, a_valw, a_valu, at_ptr, at_col, at_val, b, minv, kinv, gmap, pk_off, csize,
-        sc_ptr, sc_idx, zhx, zhy, atb, azhx, blist, vv_off, owner, comp_of_entry, comp_of_clique, comp_of_row, lrow,
+        sc_ptr, sc_idx, zhx, zhy, atb, azhx, blist, brec, vv_off, owner, comp_of_entry, comp_of_clique, comp_of_row, lrow,
         crow_ptr, crow_idx, ccl_ptr, ccl_idx, minv_off, cent_ptr, cent_idx, hs_nb, hs_nc, zhx_c, zhy_c, azhx_c,
         hs_zdz;
     size_t const_end;
@@ -68,6 +68,7 @@ struct cdsdp {
     // A^T rows) rather than inside the projection's gather (the default)
     bool x_split_auto = false;
     bool x_split = false;  // choice of the current solve
+    bool unrolled = false;  // inside an unrolled pass (derivatives are taken)
     // cached graph of a whole solve
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
@@ -139,6 +140,7 @@ Layout make_layout(const HostProblem& hp, int max_iter) {
     L.sc_ptr = take((NE + 1) * 4); L.sc_idx = take(nd * 4);
     L.zhx = take(NE * 8); L.zhy = take(m * 8); L.atb = take(NE * 8); L.azhx = take(m * 8);
     L.blist = take(p * 4);
+    L.brec = take(p * 16);
     L.vv_off = take((p + 1) * 4);
     L.owner = take(nd);
     L.comp_of_entry = take(NE * 4); L.comp_of_clique = take(p * 4); L.comp_of_row = take(m * 4); L.lrow = take(m * 4);
@@ -212,6 +214,16 @@ void build_image(cdsdp* h) {
     }
     h->cls_off[kNumClasses] = (int)blist.size();
     put(img, L.blist, blist);
+    // what a projection needs of a clique, in list order: index, order, packed offset, component
+    std::vector<int> brec(4 * blist.size());
+    for (size_t i = 0; i < blist.size(); ++i) {
+        const int k = blist[i];
+        brec[4 * i] = k;
+        brec[4 * i + 1] = cs[k];
+        brec[4 * i + 2] = hp.pk_off[k];
+        brec[4 * i + 3] = hp.comp_of_clique[k];
+    }
+    put(img, L.brec, brec);
     std::vector<int> vv(p + 1, 0);
     for (int k = 0; k < p; ++k) vv[k + 1] = vv[k] + cs[k] * cs[k];
     put(img, L.vv_off, vv);
@@ -323,10 +335,11 @@ void launch_scatter(const cdsdp* h, const Dev& d, const T* P, const T* Q, double
 
 template <typename T>
 cudaError_t launch_projection(cdsdp* h, int form, const cdsdp_opts& o, const FinishArgs& fa, cudaStream_t st) {
-    const int* bl = (const int*)(h->ws + h->L.blist);
+    const int4* bl = (const int4*)(h->ws + h->L.brec);
     ProjArgs pa;
     pa.tolrel = sizeof(T) == 4 ? 1.2e-7 : 2.3e-16;
     pa.max_sweeps = o.jacobi_max_sweeps;
+    pa.unrolled = h->unrolled ? 1 : 0;
     pa.warm_start = o.warm_start > 0 ? 1 : 0;
     pa.restart = o.warm_start > 0 ? o.warm_start : 1;
     int last = -1;
@@ -363,7 +376,7 @@ cudaError_t launch_projection(cdsdp* h, int form, const cdsdp_opts& o, const Fin
     int q = 0;
     for (int i = 0; i < kNumClasses && e == cudaSuccess; ++i) {
         const int c = ns > 1 ? h->cls_order[i] : i;
-        const int* list = bl + h->cls_off[c];
+        const int4* list = bl + h->cls_off[c];
         const int nl = h->cls_off[c + 1] - h->cls_off[c];
         if (nl <= 0) continue;
         cudaStream_t sc = ns > 1 ? h->side[q++ % ns] : st;
@@ -723,11 +736,13 @@ int check_unrolled(cdsdp* h, const cdsdp_opts& o, int iters, int ckpt_every) {
 int run_segment(cdsdp* h, Dev dd, const cdsdp_opts& o, int len, cudaStream_t st) {
     const Dev saved = h->dev;
     h->dev = dd;
+    h->unrolled = true;
     k_reset_ctl<<<1, 32, 0, st>>>(dd, o.rho);
     cudaError_t e = cudaGetLastError();
     for (int it = 0; it < len && e == cudaSuccess; ++it)
         e = launch_iteration_any(h, 0, o, st, 0, cudaGraphConditionalHandle{});
     h->dev = saved;
+    h->unrolled = false;
     return e == cudaSuccess ? CDSDP_SOLVED : fail_cuda(h, e, "unrolled iteration");
 }
 

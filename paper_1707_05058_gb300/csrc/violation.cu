@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(32 * kViolWarps) k_psd_violation(int p, const 
         bad = s < 1 || s > max_size;
         if (!bad) {  // warp-uniform
             const int off = off_arr[k], npk = s * (s + 1) / 2;
-            jac.clear(lane);
+            jac.clear(lane, s);
             T nrm = T(0);
             for (int f = lane; f < npk; f += 32) {
                 const int ab = packed_ab(f, s), a = ab >> 8, b = ab & 255;
@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(32 * kViolWarps) k_psd_violation(int p, const 
             }
             nrm = warp_sum(nrm);
             __syncwarp();
-            jac.run(T(tolrel) * sqrt(nrm), max_sweeps, lane);
+            jac.run(T(tolrel) * sqrt(nrm), max_sweeps, lane, inv_norm(nrm));
             double l = (lane < s) ? double(jac.X[lane * J::LDA + lane]) : 0.0;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) l = fmin(l, __shfl_xor_sync(0xffffffffu, l, o));
