@@ -5,7 +5,7 @@
 // warm start from the clique's previous eigenvectors, stagnation stop at the
 // rounding-noise floor), laid out for a CTA.
 //
-// Orders up to 64 (CTAJacobiMid, padded orders in steps of 4):
+// CTAJacobiMid (orders up to 64, padded in steps of 4):
 //  * A (lower triangle) and V live in shared memory, each double-buffered;
 //    V is kept in the same storage order as A, so a round is one uniform pass
 //    over pair-blocks: lower blocks (I, J) of A get J_I^T B J_J, blocks of V
@@ -15,11 +15,9 @@
 //    destination offsets it computes once per launch (registers);
 //  * V^T W V (warm start) and V max(Lambda, 0) V^T are 4x4-tiled products;
 //  * two barriers per round (rotations ready; buffers swapped).
-// Orders 65..128 (CTAJacobi): A double-buffered as above, V single-buffered
-// and rotated in place at the round's logical column pair (L[2k], L[2k+1]),
-// L following sigma.
 // Float32 orders 36..64 can also run CTAJacobiReg (jacobi_reg.cuh: V in
-// registers, one barrier per round); k_project_cta's VARIANT selects it.
+// registers, one barrier per round), and orders 65..128 always do;
+// k_project_cta's VARIANT selects it.
 #pragma once
 
 #include <type_traits>
@@ -39,206 +37,6 @@ template <typename T, int S>
 __host__ __device__ constexpr int cta_min_blocks() {
     return (sizeof(T) == 4 && S <= 48) ? 6 : ((sizeof(T) == 4 && S <= 64) ? 3 : 1);
 }
-
-template <typename T, int S>
-struct CTAJacobi {
-    using RR = RoundRobin<S>;
-    static constexpr int K = S / 2;
-    static constexpr int R = S - 1;
-    static constexpr int LDA = S + 1;
-    static constexpr int BUF = S * LDA;
-    static constexpr int NB = K * (K + 1) / 2;
-    static constexpr size_t bytes =
-        ((3 * (size_t)BUF + 3 * K) * sizeof(T) + 4 * (size_t)S * sizeof(int) + 64 * sizeof(T) + 15) & ~size_t(15);
-
-    T* X;    // current A
-    T* Y;    // next A
-    T* V;    // eigenvectors, row-major, logical columns
-    T* cs;   // [K] tau = s / (1 + c), [K] sin, [K] t * a_pq
-    int* L;  // logical index at each storage position (current)
-    int* Ln; // next
-    T* red;  // [32] reduction scratch
-
-    __device__ __forceinline__ void bind(unsigned char* base) {
-        X = reinterpret_cast<T*>(base);
-        Y = X + BUF;
-        V = Y + BUF;
-        cs = V + BUF;
-        red = cs + 3 * K;
-        L = reinterpret_cast<int*>(red + 64);
-        Ln = L + 2 * S;
-    }
-
-    __device__ __forceinline__ static void block_coords(int b, int& I, int& J) {
-        if (b < K) { I = J = b; return; }
-        const int o = b - K;  // off-diagonal blocks I > J, o = I (I - 1) / 2 + J
-        int i = int((1.0f + sqrtf(1.0f + 8.0f * float(o))) * 0.5f);
-        while (i * (i - 1) / 2 > o) --i;
-        while ((i + 1) * i / 2 <= o) ++i;
-        I = i;
-        J = o - i * (i - 1) / 2;
-    }
-
-    __device__ __forceinline__ void clear() {
-        for (int i = threadIdx.x; i < BUF; i += blockDim.x) X[i] = T(0);
-        __syncthreads();
-    }
-    __device__ __forceinline__ void put(int a, int b, T w) {
-        X[a * LDA + b] = w;
-        X[b * LDA + a] = w;
-    }
-
-    // block-wide max of |off-diagonal| of the lower triangle of X
-    __device__ T off_max() {
-        T m = T(0);
-        for (int idx = threadIdx.x; idx < S * S; idx += blockDim.x) {
-            const int i = idx / S, j = idx - i * S;
-            if (i > j) m = fmax(m, fabs(X[i * LDA + j]));
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        __syncthreads();
-        if (lane == 0) red[warp] = m;
-        __syncthreads();
-        T r = T(0);
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r = fmax(r, red[w]);
-        __syncthreads();
-        return r;
-    }
-
-    __device__ void round(T tol) {
-        const int tid = threadIdx.x, nt = blockDim.x;
-        if (tid < K) {  // rotation of pair tid (Rutishauser form)
-            const T app = X[(2 * tid) * LDA + 2 * tid], aqq = X[(2 * tid + 1) * LDA + 2 * tid + 1];
-            const T apq = X[(2 * tid + 1) * LDA + 2 * tid];
-            T tau = T(0), sn = T(0), ta = T(0);
-            if (fabs(apq) > tol) {
-                const T zeta = T(0.5) * (aqq - app);
-                const T r2 = zeta * zeta + apq * apq;
-                const T r = r2 * rsqrt_t<T>(r2);
-                const T tt = copysign(T(1), zeta) * div_t<T>(apq, fabs(zeta) + r);
-                const T c = rsqrt_t<T>(T(1) + tt * tt);
-                sn = tt * c;
-                tau = div_t<T>(sn, T(1) + c);
-                ta = tt * apq;
-            }
-            cs[tid] = tau;
-            cs[K + tid] = sn;
-            cs[2 * K + tid] = ta;
-        }
-        if (tid < S) Ln[RR::sigma(tid)] = L[tid];
-        __syncthreads();
-        for (int b = tid; b < NB; b += nt) {  // pair-blocks of A, into Y at permuted positions
-            int I, J;
-            block_coords(b, I, J);
-            const int r0 = 2 * I, r1 = r0 + 1, c0 = 2 * J, c1 = c0 + 1;
-            const int sr0 = RR::sigma(r0), sr1 = RR::sigma(r1), sc0 = RR::sigma(c0), sc1 = RR::sigma(c1);
-            if (I == J) {
-                const T ta = cs[2 * K + I];
-                const bool rot = ta != T(0) || cs[K + I] != T(0);
-                Y[max(sr0, sc0) * LDA + min(sr0, sc0)] = X[r0 * LDA + c0] - ta;
-                Y[max(sr1, sc0) * LDA + min(sr1, sc0)] = rot ? T(0) : X[r1 * LDA + c0];
-                Y[max(sr1, sc1) * LDA + min(sr1, sc1)] = X[r1 * LDA + c1] + ta;
-            } else {
-                const T uI = cs[I], sI = cs[K + I], uJ = cs[J], sJ = cs[K + J];
-                const T b00 = X[r0 * LDA + c0], b10 = X[r1 * LDA + c0], b01 = X[r0 * LDA + c1], b11 = X[r1 * LDA + c1];
-                const T q00 = b00 - sI * (b10 + uI * b00), q10 = b10 + sI * (b00 - uI * b10);
-                const T q01 = b01 - sI * (b11 + uI * b01), q11 = b11 + sI * (b01 - uI * b11);
-                Y[max(sr0, sc0) * LDA + min(sr0, sc0)] = q00 - sJ * (q01 + uJ * q00);
-                Y[max(sr0, sc1) * LDA + min(sr0, sc1)] = q01 + sJ * (q00 - uJ * q01);
-                Y[max(sr1, sc0) * LDA + min(sr1, sc0)] = q10 - sJ * (q11 + uJ * q10);
-                Y[max(sr1, sc1) * LDA + min(sr1, sc1)] = q11 + sJ * (q10 - uJ * q11);
-            }
-        }
-        for (int task = tid; task < S * K; task += nt) {  // V <- V J at the logical column pairs
-            const int i = task / K, k = task - i * K;
-            const T u = cs[k], sn = cs[K + k];
-            if (sn == T(0)) continue;
-            const int p = L[2 * k], q = L[2 * k + 1];
-            T* vr = V + i * LDA;
-            const T vp = vr[p], vq = vr[q];
-            vr[p] = vp - sn * (vq + u * vp);
-            vr[q] = vq + sn * (vp - u * vq);
-        }
-        __syncthreads();
-        T* t = X; X = Y; Y = t;
-        int* u = L; L = Ln; Ln = u;
-    }
-
-    // V <- identity (cold) or keep the loaded basis (warm), then sweep.
-    __device__ int run(T tol, int max_sweeps, bool v_preset) {
-        if (!v_preset)
-            for (int i = threadIdx.x; i < BUF; i += blockDim.x) V[i] = ((i / LDA) == (i % LDA)) ? T(1) : T(0);
-        if (threadIdx.x < S) L[threadIdx.x] = threadIdx.x;
-        __syncthreads();
-        const T noise = tol * T(2 * S);
-        T prev = T(3.0e38);
-        int sw = 0;
-        while (sw < max_sweeps) {
-            const T off = off_max();
-            if (off <= tol) break;
-            if (off <= noise && off > T(0.5) * prev) break;
-            prev = off;
-            ++sw;
-            for (int r = 0; r < R; ++r) round(tol);
-        }
-        return sw;
-    }
-
-    // X <- V^T X V (X holds the symmetric W in both triangles, V the basis).
-    __device__ void rotate_into_basis() {
-        const int tid = threadIdx.x, nt = blockDim.x;
-        for (int idx = tid; idx < S * S; idx += nt) {  // Y = W V
-            const int r = idx / S, j = idx - r * S;
-            T a = T(0);
-#pragma unroll 8
-            for (int i = 0; i < S; ++i) a += X[r * LDA + i] * V[i * LDA + j];
-            Y[r * LDA + j] = a;
-        }
-        __syncthreads();
-        for (int idx = tid; idx < S * S; idx += nt) {  // X = V^T Y
-            const int i = idx / S, j = idx - i * S;
-            T a = T(0);
-#pragma unroll 8
-            for (int r = 0; r < S; ++r) a += V[r * LDA + i] * Y[r * LDA + j];
-            X[i * LDA + j] = a;
-        }
-        __syncthreads();
-    }
-
-    __device__ void load_basis(const T* __restrict__ Vc, int s) {
-        for (int i = threadIdx.x; i < BUF; i += blockDim.x) {
-            const int r = i / LDA, c = i - r * LDA;
-            V[i] = (r < s && c < s) ? Vc[r * s + c] : (r == c ? T(1) : T(0));
-        }
-        __syncthreads();
-    }
-    __device__ void store_basis(T* __restrict__ Vc, int s) const {
-        for (int i = threadIdx.x; i < s * s; i += blockDim.x) {
-            const int r = i / s, c = i - r * s;
-            Vc[i] = V[r * LDA + c];
-        }
-    }
-    // Y row a <- V row a scaled by max(lambda, 0) (lambda on X's diagonal).
-    __device__ void prepare_rebuild() {
-        for (int i = threadIdx.x; i < BUF; i += blockDim.x) {
-            const int r = i / LDA, c = i - r * LDA;
-            if (c < S) {
-                const T l = X[c * LDA + c];
-                Y[i] = V[i] * (l > T(0) ? l : T(0));
-            }
-        }
-        __syncthreads();
-    }
-    __device__ __forceinline__ T rebuild(int a, int b, int s) const {
-        const T* ya = Y + a * LDA;
-        const T* vb = V + b * LDA;
-        T acc = T(0);
-        for (int i = 0; i < s; ++i) acc += ya[i] * vb[i];
-        return acc;
-    }
-};
 
 // Vector views of shared memory (the dynamic buffer is only 16-byte aligned,
 // so a 4-vector of doubles is read as two 16-byte halves).
@@ -573,15 +371,11 @@ struct CTAJacobiMid {
     }
 };
 
-template <typename T, int S>
-using CTASolver = typename std::conditional<(S <= 64), CTAJacobiMid<T, S>, CTAJacobi<T, S>>::type;
-
 // Solver of k_project_cta: VARIANT 0 keeps V in shared memory (CTAJacobiMid,
-// CTAJacobi); VARIANT 1 (float32, padded orders 36..64) keeps V in registers
-// (CTAJacobiReg).
+// orders up to 64); VARIANT 1 (float32) keeps V in registers (CTAJacobiReg).
 template <typename T, int S, int VARIANT>
 struct CTAPick {
-    using type = CTASolver<T, S>;
+    using type = CTAJacobiMid<T, S>;
     static constexpr int threads = cta_threads<T, S>();
     static constexpr int min_blocks = cta_min_blocks<T, S>();
 };
@@ -592,7 +386,7 @@ struct CTAPick<float, S, 1> {
     // blocks per SM: as many as 64 registers a thread allow at orders 36..56
     // (6, 5 or 4 blocks); 3 at orders 60 and 64, which spill at 64 registers
     // and ran slower with 4 (measured on the 256-SDP batch)
-    static constexpr int min_blocks = S >= 60 ? 3 : 65536 / (CTAJacobiReg<S>::NT * 64);
+    static constexpr int min_blocks = S > 64 ? 1 : (S >= 60 ? 3 : 65536 / (CTAJacobiReg<S>::NT * 64));
 };
 
 template <int NV>
@@ -648,7 +442,7 @@ __global__ void __launch_bounds__(CTAPick<T, S, VARIANT>::threads, CTAPick<T, S,
                 constexpr int NTH = CTAPick<T, S, VARIANT>::threads;
                 constexpr int MAXF = (S * (S + 1) / 2 + NTH - 1) / NTH;
                 int ent[MAXF];
-                double v0[MAXF], v1[MAXF], v2[MAXF];
+                T v0[MAXF], v1[MAXF], v2[MAXF];
                 bool own[MAXF];
 #pragma unroll
                 for (int u = 0; u < MAXF; ++u) {
@@ -656,9 +450,9 @@ __global__ void __launch_bounds__(CTAPick<T, S, VARIANT>::threads, CTAPick<T, S,
                     const bool ok = f < npk;
                     ent[u] = (ok && (FORM == 0 || FORM == 2)) ? d.gmap[off + f] : 0;
                     own[u] = (ok && FORM == 0) ? d.owner[off + f] != 0 : false;
-                    v1[u] = (ok && FORM != 3) ? double(c1[off + f]) : 0.0;
-                    v2[u] = (ok && (FORM == 1 || FORM == 2)) ? double(c2[off + f]) : 0.0;
-                    v0[u] = ok ? (FORM == 3 ? double(Win[off + f]) : (FORM == 2 ? double(c0[off + f]) : 0.0)) : 0.0;
+                    v1[u] = (ok && FORM != 3) ? c1[off + f] : T(0);
+                    v2[u] = (ok && (FORM == 1 || FORM == 2)) ? c2[off + f] : T(0);
+                    v0[u] = ok ? (FORM == 3 ? Win[off + f] : (FORM == 2 ? c0[off + f] : T(0))) : T(0);
                 }
 #pragma unroll
                 for (int u = 0; u < MAXF; ++u) {
@@ -669,17 +463,17 @@ __global__ void __launch_bounds__(CTAPick<T, S, VARIANT>::threads, CTAPick<T, S,
                     if (FORM == 0) {
                         const double xe = d.x[ent[u]];
                         if (own[u]) cx += d.wgt[ent[u]] * d.c[ent[u]] * xe;
-                        w = xe - v1[u] * irho;
+                        w = xe - double(v1[u]) * irho;
                         if (d.wstore) {
                             const int slot = d.ctl[CTL_ITER];
                             if (slot < d.wstore_count) reinterpret_cast<T*>(d.wstore)[(size_t)slot * d.nd + off + f] = T(w);
                         }
                     } else if (FORM == 1) {
-                        w = v1[u] - v2[u] * irho;
+                        w = double(v1[u]) - double(v2[u]) * irho;
                     } else if (FORM == 2) {
                         const double hs = d.s11[ent[u]];
-                        const double s12 = 0.5 * (v0[u] + v1[u] - v2[u] + hs);
-                        w = s12 - gamma * 0.5 * d.zhx[ent[u]] - v1[u];
+                        const double s12 = 0.5 * (double(v0[u]) + double(v1[u]) - double(v2[u]) + hs);
+                        w = s12 - gamma * 0.5 * d.zhx[ent[u]] - double(v1[u]);
                     } else {
                         w = v0[u];
                     }
@@ -735,7 +529,12 @@ __global__ void __launch_bounds__(CTAPick<T, S, VARIANT>::threads, CTAPick<T, S,
             } else {
                 jac.identity_basis();
             }
-            jac.run(T(pa.tolrel) * T(sqrt(nrm)), pa.max_sweeps, true);
+            const T fro = T(sqrt(nrm));
+            typename J::Plan plan;
+            J::plan(plan);
+            jac.run(T(pa.tolrel) * fro, pa.max_sweeps, fro > T(0) ? T(1) / fro : T(0), T(kThetaSolve * pa.tolrel), plan);
+            if (FORM != 3 && pa.warm_start) jac.store_basis(vc + (size_t)d.vv_off[ck_i[0]], ck_i[1]);
+            jac.project(plan);
         } else {
             if (warm) {
                 jac.load_basis(vc + d.vv_off[k], s);
@@ -748,8 +547,10 @@ __global__ void __launch_bounds__(CTAPick<T, S, VARIANT>::threads, CTAPick<T, S,
         const double rho = ck_d[0], gamma = ck_d[1];
         const double cxk = tid == 0 ? ck_d[2] : 0.0;
         const int npk = s * (s + 1) / 2;
-        if (FORM != 3 && pa.warm_start) jac.store_basis(vc + d.vv_off[k], s);
-        jac.prepare_rebuild();
+        if constexpr (VARIANT != 1) {
+            if (FORM != 3 && pa.warm_start) jac.store_basis(vc + d.vv_off[k], s);
+            jac.prepare_rebuild();
+        }
         double p[6] = {0, 0, 0, 0, 0, 0};
         T pf[5] = {0, 0, 0, 0, 0};  // float32 form of Algorithm 1: per-thread sums in float
         if constexpr (VARIANT == 1) {

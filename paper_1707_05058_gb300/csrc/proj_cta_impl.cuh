@@ -35,16 +35,22 @@ cudaError_t launch_cta_v(const Dev& d, const int4* list, int nlist, const ProjAr
     return cudaGetLastError();
 }
 
-// pa.cta_variant = 1 selects variant 1 (V in registers) for float32 orders 36..64.
+// pa.cta_variant = 1 selects variant 1 (V in registers) for float32 orders
+// 36..64; float32 orders above 64 and the standalone projection have
+// no other.
 template <typename T, int S, int FORM>
 cudaError_t launch_cta(const Dev& d, const int4* list, int nlist, const ProjArgs& pa, const FinishArgs& fa,
                        const int* off, const int* size, const void* W, void* X, int max_sweeps, cudaStream_t st) {
     if (nlist <= 0) return cudaSuccess;
-    if constexpr (sizeof(T) == 4 && S >= 36 && S <= 64) {
+    if constexpr (S > 64 || (sizeof(T) == 4 && FORM == 3)) {
+        return launch_cta_v<T, S, FORM, 1>(d, list, nlist, pa, fa, off, size, W, X, max_sweeps, st);
+    } else if constexpr (sizeof(T) == 4) {
         if (pa.cta_variant == 1)
             return launch_cta_v<T, S, FORM, 1>(d, list, nlist, pa, fa, off, size, W, X, max_sweeps, st);
     }
-    return launch_cta_v<T, S, FORM, 0>(d, list, nlist, pa, fa, off, size, W, X, max_sweeps, st);
+    if constexpr (S <= 64 && !(sizeof(T) == 4 && FORM == 3))
+        return launch_cta_v<T, S, FORM, 0>(d, list, nlist, pa, fa, off, size, W, X, max_sweeps, st);
+    return cudaErrorInvalidValue;
 }
 
 template <typename T, int S>
@@ -71,12 +77,11 @@ cudaError_t CTA_SUFFIX(launch_proj_cta)(int S, int form, const Dev& d, const int
 }
 
 cudaError_t CTA_SUFFIX(launch_proj_cta_standalone)(int S, int p, const int* off, const int* size, const void* W,
-                                                   void* X, int max_sweeps, int variant, cudaStream_t st) {
+                                                   void* X, int max_sweeps, cudaStream_t st) {
     Dev d{};
     ProjArgs pa{};
     FinishArgs fa{};
     pa.restart = 1;
-    pa.cta_variant = variant;
     switch (S) {
 #define CTA_CASE(N) \
     case N: return launch_cta<CTA_T, N, 3>(d, nullptr, p, pa, fa, off, size, W, X, max_sweeps, st);
