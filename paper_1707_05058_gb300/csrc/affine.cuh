@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(ETHREADS) k_scatter(Dev d, const T* __restrict
         const bool live = e < d.NE && !(check_stop && frozen_entry(d, e));
         double a = alpha, gm = gamma;
         if (live && (alpha_rho || gamma_rho)) {
-            const double ir = 1.0 / rho_entry(d, e);
+            const double ir = irho_entry(d, e);
             if (alpha_rho) a *= ir;
             if (gamma_rho) gm *= ir;
         }
@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(ETHREADS) k_scatter_owner(Dev d, const T* __re
         if (check_stop && frozen_entry(d, e)) continue;
         double a = alpha, gm = gamma;
         if (alpha_rho || gamma_rho) {
-            const double ir = 1.0 / rho_entry(d, e);
+            const double ir = irho_entry(d, e);
             if (alpha_rho) a *= ir;
             if (gamma_rho) gm *= ir;
         }

@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(128) k_vlam_dual(Dev d, FinishArgs fa) {
     double acc[4] = {0, 0, 0, 0};
     for (int k = w0; k < d.p; k += nw) {
         if (frozen_clique(d, k)) continue;  // warp-uniform
-        const double rho = rho_clique(d, k);
+        const double rho = rho_clique(d, k), irho = irho_clique(d, k);
         const int off = d.pk_off[k], s = d.csize[k], npk = s * (s + 1) / 2;
         // v and lambda are formed in float64 (z + lambda/rho + x cancels) and
         // stored in T; the per-clique sums of the stopping test are in T
@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(128) k_vlam_dual(Dev d, FinishArgs fa) {
             if (d.comp_mode && d.owner[off + f]) cx += d.wgt[ent] * d.c[ent] * d.x[ent];
             const T zt = z[off + f];
             const double zz = zt, ll = lam[off + f];
-            const T vn = T(zz + ll / rho + d.x[ent]);
+            const T vn = T(zz + ll * irho + d.x[ent]);
             const T ln = T(ll + rho * (zz - double(vn)));
             v[off + f] = vn;
             lam[off + f] = ln;
@@ -83,8 +83,19 @@ __device__ void finish_dual_block(const Dev& d, const FinishArgs& fa) {
         d.ctl[CTL_COUNTER] = 0;
         finish_common(d, bad, it > 1 && fmax(ec, el) <= fa.eps, it, fa.use_cond, fa.hnd);
         if (!d.ctl[CTL_DONE] && fa.adapt_every > 0 && it % fa.adapt_every == 0)
-            d.rho[0] = adapt_rho(rho, ec, el, fa.mu, fa.nu);
+            set_rho(d, 0, adapt_rho(rho, ec, el, fa.mu, fa.nu));
     }
+}
+
+// Called by one block per component; true in the block that arrives last.
+__device__ __forceinline__ bool last_of_components(const Dev& d) {
+    __shared__ int s_last3;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last3 = atomicAdd(reinterpret_cast<unsigned int*>(d.ctl + CTL_COUNTER), 1u) == (unsigned)d.ncomp - 1 ? 1 : 0;
+    }
+    __syncthreads();
+    return s_last3 != 0;
 }
 
 // Global state after the per-component tests, run by the block that arrives
@@ -197,7 +208,7 @@ __global__ void __launch_bounds__(256) k_finish_components(Dev d, int form, Fini
                 d.comp_status[c] = st;
                 d.comp_done[c] = 1;
             } else if (fa.adapt_every > 0 && it % fa.adapt_every == 0) {
-                d.rho[c] = adapt_rho(rho, ec, el, fa.mu, fa.nu);
+                set_rho(d, c, adapt_rho(rho, ec, el, fa.mu, fa.nu));
             }
         }
     }
@@ -303,23 +314,47 @@ __global__ void __launch_bounds__(RTHREADS) k_hsde_sigma21(Dev d, int TPR, int n
 }
 
 // The same update per independent component, each with its own embedding
-// (component mode; one block per component): gamma_c = zeta_c^T sigma over the
-// component's entries and rows, then tau_c, kappa_c.
+// (component mode): gamma_c = zeta_c^T sigma over the component's entries and
+// rows, then tau_c, kappa_c and the new u_y of the component's rows.  Block
+// (i, c) of the grid takes the i-th part of component c's entries; the last of
+// a component's blocks to arrive adds the parts in order.  (One block per
+// component read 47,000 entries by itself, 266 us a launch on a batch of eight;
+// with this and the test below split, 48 iterations went from 41.0 to 23.8 ms.)
 __global__ void __launch_bounds__(256) k_hsde_gamma_components(Dev d) {
     __shared__ double sh[32 * 2];
     if (stopped(d)) return;
-    const int c = blockIdx.x;
+    const int c = blockIdx.y, part = blockIdx.x, np = gridDim.x;
     if (d.comp_done[c]) return;
     double v[2] = {0.0, 0.0};
-    for (int j = d.cent_ptr[c] + threadIdx.x; j < d.cent_ptr[c + 1]; j += blockDim.x) {
+    const int p0 = d.cent_ptr[c], len = d.cent_ptr[c + 1] - p0;
+    const int j1 = p0 + int((long long)len * (part + 1) / np);
+    for (int j = p0 + int((long long)len * part / np) + threadIdx.x; j < j1; j += blockDim.x) {
         const int e = d.cent_idx[j];
         v[0] += d.wgt[e] * d.c[e] * d.s11[e];
     }
-    for (int j = d.crow_ptr[c] + threadIdx.x; j < d.crow_ptr[c + 1]; j += blockDim.x) {
-        const int i = d.crow_idx[j];
-        v[1] += d.b[i] * d.s21[i];
+    if (part == 0) {
+        for (int j = d.crow_ptr[c] + threadIdx.x; j < d.crow_ptr[c + 1]; j += blockDim.x) {
+            const int i = d.crow_idx[j];
+            v[1] += d.b[i] * d.s21[i];
+        }
     }
     block_sum<2>(v, sh);
+    __shared__ double s_gamma;
+    if (np > 1) {  // parts in the per-block table (free here in component mode)
+        if (threadIdx.x == 0) {
+            double* pr = d.parte + (size_t)(c * np + part) * PART_COLS;
+            pr[0] = v[0];
+            pr[1] = v[1];
+        }
+        if (!last_block_of_component(d, c)) return;
+        v[0] = v[1] = 0.0;
+        for (int j = threadIdx.x; j < np; j += blockDim.x) {
+            const double* pr = d.parte + (size_t)(c * np + j) * PART_COLS;
+            v[0] += __ldcg(pr);
+            v[1] += __ldcg(pr + 1);
+        }
+        block_sum<2>(v, sh);
+    }
     if (threadIdx.x == 0) {
         const double tau = d.hs_tau[c], kappa = d.hs_kappa[c];
         const double gamma = v[0] - v[1];
@@ -328,12 +363,19 @@ __global__ void __launch_bounds__(256) k_hsde_gamma_components(Dev d) {
         d.hs_gamma[c] = gamma;
         d.hs_tau[c] = tn;
         d.hs_kappa[c] = kappa - tauhat + tn;
+        s_gamma = gamma;
+    }
+    __syncthreads();
+    for (int j = d.crow_ptr[c] + threadIdx.x; j < d.crow_ptr[c + 1]; j += blockDim.x) {
+        const int i = d.crow_idx[j];
+        d.y[i] = d.s21[i] - s_gamma * d.zhy[i];
     }
 }
 
 // gamma = zeta^T sigma, u_hat_2 = omega_2 + zeta^T u_hat_1 = omega_2 + gamma (1 - zeta^T zeta_hat)
 // (Eqs. MatrixInverseResult, FirstBlockElimination); tau <- max(0, u_hat_tau - kappa),
-// kappa <- kappa - u_hat_tau + tau (Eqs. HsdeStep2-3 on the R_+ component).
+// kappa <- kappa - u_hat_tau + tau (Eqs. HsdeStep2-3 on the R_+ component); then
+// u_y <- sigma_21 - gamma zeta_hat_y.
 __device__ void hsde_gamma_block(const Dev& d, int nbe, int nbr) {
     __shared__ double sh[32];
     const double cs = sum_col(d.parte, nbe, 2, sh);
@@ -349,10 +391,15 @@ __device__ void hsde_gamma_block(const Dev& d, int nbe, int nbr) {
         d.scal[SC_TAU] = tn;
         d.scal[SC_KAPPA] = kappa - tauhat + tn;
         d.ctl[CTL_COUNTER] = 0;
+        sh[0] = gamma;
     }
+    __syncthreads();
+    const double gamma = sh[0];
+    for (int i = threadIdx.x; i < d.m; i += blockDim.x) d.y[i] = __ldcg(d.s21 + i) - gamma * d.zhy[i];
 }
 
-// u_x <- sigma_11 - gamma zeta_hat_x; A^T u_y with u_y = sigma_21 - gamma zeta_hat_y;
+// u_x <- sigma_11 - gamma zeta_hat_x; A^T u_y (u_y is formed with gamma, once per
+// row rather than once per nonzero here);
 // partials: |A^T u_y + H^T v_z - tau c|^2 (parte col 0) and <c, u_x> (col 1).
 template <typename T>
 __global__ void __launch_bounds__(ETHREADS) k_hsde_entry_update(Dev d, int G) {
@@ -373,7 +420,7 @@ __global__ void __launch_bounds__(ETHREADS) k_hsde_entry_update(Dev d, int G) {
             const int q1 = d.at_ptr[e + 1];
             for (int q = d.at_ptr[e] + lig; q < q1; q += G) {
                 const int i = d.at_col[q];
-                a += d.at_val[q] * (d.s21[i] - gamma * d.zhy[i]);
+                a += d.at_val[q] * d.y[i];
             }
             const int j1 = d.sc_ptr[e + 1];
             for (int j = d.sc_ptr[e] + lig; j < j1; j += G) hv += double(vz[d.sc_idx[j]]);
@@ -400,7 +447,7 @@ __global__ void __launch_bounds__(ETHREADS) k_hsde_entry_update(Dev d, int G) {
     }
 }
 
-// u_y <- sigma_21 - gamma zeta_hat_y; A u_x = A sigma_11 - gamma A zeta_hat_x;
+// A u_x = A sigma_11 - gamma A zeta_hat_x;
 // partials |A u_x - tau b|^2 (partr col 0) and <b, u_y> (col 1).
 __device__ void finish_hsde_block(const Dev& d, const FinishArgs& fa);
 
@@ -412,8 +459,7 @@ __global__ void __launch_bounds__(RTHREADS) k_hsde_row_update(Dev d, FinishArgs 
         if (frozen_row(d, i)) continue;
         const int c = comp_r(d, i);
         const double gamma = hs_gamma_c(d, c), tau = hs_tau_c(d, c);
-        const double uy = d.s21[i] - gamma * d.zhy[i];
-        d.y[i] = uy;
+        const double uy = d.y[i];
         const double r = d.as11[i] - gamma * d.azhx[i] - tau * d.b[i];
         p[0] += r * r;
         p[1] += d.b[i] * uy;
@@ -482,39 +528,70 @@ __device__ void finish_hsde_block(const Dev& d, const FinishArgs& fa) {
 }
 
 // Algorithm 3 stopping tests per independent component, each component with
-// its own embedding (component mode; one block per component): the tests of
+// its own embedding (component mode): the tests of
 // finish_hsde_block on the component's own clique rows of the partial table,
 // its own entries (|A^T u_y + H^T v_z - tau c|^2, <c, u_x>, per entry in t and
 // q) and rows (|A u_x - tau b|^2, <b, u_y>, per row in g and hh), its own
 // tau, kappa and norms of b and c.  A component that passes, proves
 // infeasibility, reaches max_iter or meets a NaN is frozen from the next
-// iteration on; the block that arrives last sets the global state.
+// iteration on; the block that arrives last sets the global state.  Block
+// (i, c) of the grid takes the i-th part of the component's entries (and the
+// first one its cliques and rows), the last of a component's blocks adds the
+// parts in order and runs the test (181 us a launch with one block per
+// component on a batch of eight).
 __global__ void __launch_bounds__(256) k_finish_hsde_components(Dev d, FinishArgs fa) {
     __shared__ double sh[32 * 10];
     __shared__ int s_was_done;
     if (stopped(d)) return;
-    const int c = blockIdx.x;
+    const int c = blockIdx.y, part = blockIdx.x, np = gridDim.x;
     const int it = d.ctl[CTL_ITER] + 1;
     if (threadIdx.x == 0) s_was_done = d.comp_done[c];
     __syncthreads();
+    double v[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     if (!s_was_done) {
-        double v[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-        for (int j = d.ccl_ptr[c] + threadIdx.x; j < d.ccl_ptr[c + 1]; j += blockDim.x) {
+        if (part == 0) for (int j = d.ccl_ptr[c] + threadIdx.x; j < d.ccl_ptr[c + 1]; j += blockDim.x) {
             const double* pr = d.part + (size_t)d.ccl_idx[j] * PART_COLS;
 #pragma unroll
             for (int q = 0; q < 6; ++q) v[q] += __ldcg(pr + q);
         }
-        for (int j = d.cent_ptr[c] + threadIdx.x; j < d.cent_ptr[c + 1]; j += blockDim.x) {
+        const int p0 = d.cent_ptr[c], len = d.cent_ptr[c + 1] - p0;
+        const int j1 = p0 + int((long long)len * (part + 1) / np);
+        for (int j = p0 + int((long long)len * part / np) + threadIdx.x; j < j1; j += blockDim.x) {
             const int e = d.cent_idx[j];
             v[6] += __ldcg(d.t + e);
             v[7] += __ldcg(d.q + e);
         }
-        for (int j = d.crow_ptr[c] + threadIdx.x; j < d.crow_ptr[c + 1]; j += blockDim.x) {
+        if (part == 0) for (int j = d.crow_ptr[c] + threadIdx.x; j < d.crow_ptr[c + 1]; j += blockDim.x) {
             const int i = d.crow_idx[j];
             v[8] += __ldcg(d.g + i);
             v[9] += __ldcg(d.hh + i);
         }
         block_sum<10>(v, sh);
+    }
+    if (np > 1) {  // parts in the per-block tables (free here in component mode)
+        if (threadIdx.x == 0) {
+            double* pr = d.parte + (size_t)(c * np + part) * PART_COLS;
+            pr[0] = v[6];
+            pr[1] = v[7];
+            if (part == 0)
+                for (int q = 0; q < 8; ++q) d.partr[(size_t)c * PART_COLS + q] = q < 6 ? v[q] : v[q + 2];
+        }
+        if (!last_block_of_component(d, c)) return;
+        if (!s_was_done) {
+            double e[2] = {0.0, 0.0};
+            for (int j = threadIdx.x; j < np; j += blockDim.x) {
+                const double* pr = d.parte + (size_t)(c * np + j) * PART_COLS;
+                e[0] += __ldcg(pr);
+                e[1] += __ldcg(pr + 1);
+            }
+            block_sum<2>(e, sh);
+            const double* pr = d.partr + (size_t)c * PART_COLS;
+            for (int q = 0; q < 8; ++q) v[q < 6 ? q : q + 2] = __ldcg(pr + q);
+            v[6] = e[0];
+            v[7] = e[1];
+        }
+    }
+    if (!s_was_done) {
         if (threadIdx.x == 0) {
             const double eps = fa.eps, tau = d.hs_tau[c], kappa = d.hs_kappa[c];
             const double rd2 = v[6], cux = v[7], rp2 = v[8], buy = v[9];
@@ -550,7 +627,7 @@ __global__ void __launch_bounds__(256) k_finish_hsde_components(Dev d, FinishArg
             }
         }
     }
-    if (!last_block_single_writer(d)) return;
+    if (!last_of_components(d)) return;
     components_global_state(d, fa, it);
 }
 
@@ -558,7 +635,7 @@ __global__ void __launch_bounds__(256) k_finish_hsde_components(Dev d, FinishArg
 
 __global__ void k_init(Dev d, int form, double rho0) {
     for (int c = threadIdx.x; c < d.ncomp; c += blockDim.x) {
-        d.rho[c] = rho0;
+        set_rho(d, c, rho0);
         d.hs_tau[c] = (form == 2) ? 1.0 : 0.0;
         d.hs_kappa[c] = (form == 2) ? 1.0 : 0.0;
         d.hs_gamma[c] = 0.0;

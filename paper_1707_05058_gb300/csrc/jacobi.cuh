@@ -719,7 +719,7 @@ __global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4)) k_proj
         const int4 rec = __ldg(list + (li < nlist ? li : li0));
         const int k = rec.x, off = rec.z, npk0 = li < nlist ? rec.y * (rec.y + 1) / 2 : 0;
         const bool active = li < nlist && !(d.comp_mode && d.comp_done[rec.w]);
-        const double rho = d.rho[d.comp_mode ? rec.w : 0];
+        const double rho = d.rho[d.comp_mode ? rec.w : 0], ir = d.irho[d.comp_mode ? rec.w : 0];
         T nrm = T(0);
         T hx[J::MAXE];
         double cx = 0.0;
@@ -731,7 +731,7 @@ __global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4)) k_proj
             s = active ? rec.y : 0;
             npk = s * (s + 1) / 2;
             rho_t = T(rho);
-            irho = UNROLLED ? T(1.0 / rho) : T(1) / T(rho);
+            irho = T(ir);
             jac.clear(lane, s);
         };
         if (pa.x_ready) {  // every load of this lane's entries issued before its use: indices, then values
@@ -881,7 +881,7 @@ __global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4)) k_proj
         const int4 rec = __ldg(list + (li < nlist ? li : li0));
         const int k = rec.x, off = rec.z, npk0 = li < nlist ? rec.y * (rec.y + 1) / 2 : 0;
         const bool active = li < nlist && !(d.comp_mode && d.comp_done[rec.w]);
-        const double rho = d.rho[d.comp_mode ? rec.w : 0];
+        const double ir = d.irho[d.comp_mode ? rec.w : 0];
         T nrm = T(0);
         T zo[J::MAXE];
         T vv[J::MAXE], lm[J::MAXE];
@@ -893,7 +893,7 @@ __global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4)) k_proj
             zo[e] = f < npk0 ? z[off + f] : T(0);
         }
         const int s = active ? rec.y : 0, npk = s * (s + 1) / 2;
-        const T irho = T(1) / T(rho);
+        const T irho = T(ir);
         jac.clear(lane, s);
         {
 #pragma unroll

@@ -426,7 +426,8 @@ __global__ void __launch_bounds__(CTAPick<T, S, VARIANT>::threads, CTAPick<T, S,
         const int k = rec.x, s = rec.y, off = rec.z;
         if (s > S || s < 1) continue;  // block-uniform
         if (FORM != 3 && frozen_clique(d, k)) continue;
-        const double rho = (FORM == 0 || FORM == 1) ? rho_clique(d, k) : 1.0, irho = 1.0 / rho;
+        const double rho = (FORM == 0 || FORM == 1) ? rho_clique(d, k) : 1.0;
+        const double irho = (FORM == 0 || FORM == 1) ? irho_clique(d, k) : 1.0;
         const double gamma = FORM == 2 ? hs_gamma_c(d, comp_k(d, k)) : 0.0;
         const int npk = s * (s + 1) / 2;
         if (tid == 0) {

@@ -90,6 +90,8 @@ struct Dev {
     int* comp_iter;             // [ncomp] iterations run by the component
     int* comp_status;           // [ncomp] cdsdp_status of the component
     double* comp_res;           // [ncomp * HIST_COLS] last stopping-test row of the component
+    double* irho;               // [ncomp] 1 / rho: a float64 division takes some forty operations of
+                                // a pipe that does two a clock and SM, so no kernel divides per entry
     double* rho;                // [ncomp] penalty of Algorithms 1-2: one per component when
                                 // components stop on their own, else entry 0 for the whole problem
     // Algorithm 3 with one embedding per independent component (component
@@ -98,6 +100,7 @@ struct Dev {
     double* hs_tau;             // [ncomp]
     double* hs_kappa;           // [ncomp]
     double* hs_gamma;           // [ncomp]
+    int* comp_cnt;              // [ncomp] blocks of a component that have arrived (several blocks per component)
     const double* hs_zdz;       // [ncomp] zeta_c^T zeta_hat_c
     const double* hs_nb;        // [ncomp] ||b_c||
     const double* hs_nc;        // [ncomp] ||c_c|| (weighted lower storage)
@@ -157,6 +160,16 @@ __device__ __forceinline__ double rho_entry(const Dev& d, int e) {
 }
 __device__ __forceinline__ double rho_row(const Dev& d, int i) {
     return d.rho[d.comp_mode ? d.comp_of_row[i] : 0];
+}
+__device__ __forceinline__ double irho_clique(const Dev& d, int k) {
+    return d.irho[d.comp_mode ? d.comp_of_clique[k] : 0];
+}
+__device__ __forceinline__ double irho_entry(const Dev& d, int e) {
+    return d.irho[d.comp_mode ? d.comp_of_entry[e] : 0];
+}
+__device__ __forceinline__ void set_rho(const Dev& d, int c, double rho) {
+    d.rho[c] = rho;
+    d.irho[c] = 1.0 / rho;
 }
 // Adaptive penalty rule (Section 7.1.2) on the residual pair (eps_c, eps_lambda).
 __device__ __forceinline__ double adapt_rho(double rho, double ep, double ed, double mu, double nu) {
@@ -255,6 +268,23 @@ __device__ __forceinline__ bool last_block_single_writer(const Dev& d) {
     }
     __syncthreads();
     return s_last1 != 0;
+}
+
+// The same among the gridDim.x blocks of one component (block (., c) of the
+// grid); the counter returns to zero.
+__device__ __forceinline__ bool last_block_of_component(const Dev& d, int c) {
+    __shared__ int s_last2;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const int ticket = atomicAdd(d.comp_cnt + c, 1);
+        s_last2 = (ticket == (int)gridDim.x - 1) ? 1 : 0;
+        if (s_last2) {
+            d.comp_cnt[c] = 0;
+            __threadfence();
+        }
+    }
+    __syncthreads();
+    return s_last2 != 0;
 }
 
 // Per-block sum of NV per-warp values (each warp's value valid in its lane 0);

@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(256) k_large_gather(Dev d, Step t) {
     const float* c0 = reinterpret_cast<const float*>(d.ck0);
     const float* c1 = reinterpret_cast<const float*>(d.ck1);
     const float* c2 = reinterpret_cast<const float*>(d.ck2);
-    const double irho = (FORM == 2) ? 1.0 : 1.0 / cdsdp_dev::rho_clique(d, k);
+    const double irho = (FORM == 2) ? 1.0 : cdsdp_dev::irho_clique(d, k);
     const double gamma = FORM == 2 ? cdsdp_dev::hs_gamma_c(d, cdsdp_dev::comp_k(d, k)) : 0.0;
     for (long long f = f0 + threadIdx.x; f < f1; f += blockDim.x) {
         int a, b;

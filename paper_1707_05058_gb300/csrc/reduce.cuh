@@ -100,7 +100,7 @@ __device__ __forceinline__ void finish_primal_block(const Dev& d, const FinishAr
         d.ctl[CTL_COUNTER] = 0;
         finish_common(d, bad, it > 1 && fmax(ec, el) <= fa.eps, it, fa.use_cond, fa.hnd);
         if (!d.ctl[CTL_DONE] && fa.adapt_every > 0 && it % fa.adapt_every == 0)
-            d.rho[0] = adapt_rho(rho, ec, el, fa.mu, fa.nu);
+            set_rho(d, 0, adapt_rho(rho, ec, el, fa.mu, fa.nu));
     }
 }
 

@@ -41,7 +41,7 @@ struct Layout {
     size_t const_end;
     // state
     size_t x, t, q, s11, atuy, y, g, hh, s21, as11, ck0, ck1, ck2, vcache, part, parte, partr, scal, ctl, hist,
-        comp_done, comp_iter, comp_status, comp_res, rho, cg_res, cg_p, cg_q, cg_u, cg_scal, hs_tau, hs_kappa,
+        comp_done, comp_iter, comp_status, comp_res, rho, irho, comp_cnt, cg_res, cg_p, cg_q, cg_u, cg_scal, hs_tau, hs_kappa,
         hs_gamma;
     size_t total;   // end of the state section (zeroed at every solve)
     size_t ns_off;  // dense buffers and tables of the large-clique projection (not zeroed per solve)
@@ -63,6 +63,7 @@ struct cdsdp {
     // per entry for scatters (Gs) and A^T rows (Ga), threads per A row (TPR)
     // and per row of the cached inverse (TPRM)
     int GE = 1, GR = 1, Gs = 1, Ga = 1, Gx = 1, TPR = 32, TPRM = 32;
+    int hs_parts = 1;   // blocks per component of Algorithm 3's component reductions
     int TPR_auto = 32;  // TPR from the row lengths (opts.row_threads = 0)
     // Algorithm 1: compute x = t - D^-1 A^T y in its own kernel (coalesced
     // A^T rows) rather than inside the projection's gather (the default)
@@ -166,7 +167,7 @@ Layout make_layout(const HostProblem& hp, int max_iter) {
     L.hist = take((size_t)std::max(max_iter, 1) * HIST_COLS * 8);
     L.comp_done = take(nc * 4); L.comp_iter = take(nc * 4); L.comp_status = take(nc * 4);
     L.comp_res = take(nc * HIST_COLS * 8);
-    L.rho = take(nc * 8);
+    L.rho = take(nc * 8); L.irho = take(nc * 8); L.comp_cnt = take(nc * 4);
     L.cg_res = take(m * 8); L.cg_p = take(m * 8); L.cg_q = take(m * 8); L.cg_u = take(NE * 8);
     L.cg_scal = take(4 * 8);
     L.hs_tau = take(nc * 8); L.hs_kappa = take(nc * 8); L.hs_gamma = take(nc * 8);
@@ -278,7 +279,7 @@ void make_dev(cdsdp* h) {
     d.minv_off = (const long long*)(w + L.minv_off);
     d.comp_done = (int*)(w + L.comp_done); d.comp_iter = (int*)(w + L.comp_iter);
     d.comp_status = (int*)(w + L.comp_status); d.comp_res = (double*)(w + L.comp_res);
-    d.rho = (double*)(w + L.rho);
+    d.rho = (double*)(w + L.rho); d.irho = (double*)(w + L.irho); d.comp_cnt = (int*)(w + L.comp_cnt);
     d.cg_res = (double*)(w + L.cg_res); d.cg_p = (double*)(w + L.cg_p); d.cg_q = (double*)(w + L.cg_q);
     d.cg_u = (double*)(w + L.cg_u); d.cg_scal = (double*)(w + L.cg_scal);
     d.cg_tol = 0.0; d.cg_max = 0;
@@ -302,6 +303,11 @@ void make_dev(cdsdp* h) {
     // low on this GPU); inside the gather it is formed once per clique holding e.
     h->x_split_auto = true;
     h->x_split = h->x_split_auto;
+    // about 512 entries a block, and at most one block per row of the table of
+    // per-block sums over all components
+    int max_ce = 0;
+    for (int c = 0; c < hp.ncomp; ++c) max_ce = std::max(max_ce, hp.cent_ptr[c + 1] - hp.cent_ptr[c]);
+    h->hs_parts = std::max(1, std::min(std::min(NBLK_E, NBLK_R) / std::max(1, hp.ncomp), std::min(64, max_ce / 512)));
     int max_mc = 0;
     for (int c = 0; c < hp.ncomp; ++c) max_mc = std::max(max_mc, hp.crow_ptr[c + 1] - hp.crow_ptr[c]);
     // threads per row of the cached inverse: about 16 entries a thread (rows of
@@ -481,7 +487,7 @@ cudaError_t launch_iteration(cdsdp* h, int form, const cdsdp_opts& o, cudaStream
         k_gemv<<<GR, RTHREADS, 0, st>>>(d, d.kinv, d.g, d.hh, -1, h->TPRM);
         k_hsde_sigma11<<<GE, ETHREADS, 0, st>>>(d, h->Ga);
         k_hsde_sigma21<<<GR, RTHREADS, 0, st>>>(d, h->TPR, GE);
-        if (d.comp_mode) k_hsde_gamma_components<<<d.ncomp, 256, 0, st>>>(d);
+        if (d.comp_mode) k_hsde_gamma_components<<<dim3(h->hs_parts, d.ncomp), 256, 0, st>>>(d);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if (ev0) cudaEventRecord(ev0, st);
         FinishArgs none = fa;
@@ -490,7 +496,7 @@ cudaError_t launch_iteration(cdsdp* h, int form, const cdsdp_opts& o, cudaStream
         if (ev1) cudaEventRecord(ev1, st);
         k_hsde_entry_update<T><<<GE, ETHREADS, 0, st>>>(d, h->Ga);
         k_hsde_row_update<<<GR, RTHREADS, 0, st>>>(d, fa);
-        if (d.comp_mode) k_finish_hsde_components<<<d.ncomp, 256, 0, st>>>(d, fa);
+        if (d.comp_mode) k_finish_hsde_components<<<dim3(h->hs_parts, d.ncomp), 256, 0, st>>>(d, fa);
     }
     return cudaGetLastError();
 }
