@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(CTAPick<T, S, VARIANT>::threads, CTAPick<T, S,
     for (int li = blockIdx.x; li < nlist; li += gridDim.x) {
         const int4 rec = FORM == 3 ? make_int4(li, size_arr[li], off_arr[li], 0) : list[li];
         const int k = rec.x, s = rec.y, off = rec.z;
-        if (s > S || s < 1) continue;  // block-uniform
+        if (s > S || s < (FORM == 3 ? pa.min_size : 1)) continue;  // block-uniform
         if (FORM != 3 && frozen_clique(d, k)) continue;
         const double rho = (FORM == 0 || FORM == 1) ? rho_clique(d, k) : 1.0;
         const double irho = (FORM == 0 || FORM == 1) ? irho_clique(d, k) : 1.0;

@@ -103,7 +103,9 @@ struct CTAJacobiReg {
         for (int j = 0; j < NPB; ++j) {
             const int b = threadIdx.x + j * NT;
             int kind = 0, I = 0, J = 0;
-            if (b < K) {
+            if ((int)threadIdx.x >= NT) {  // a launch wider than this order needs
+                kind = 0;
+            } else if (b < K) {
                 kind = 1;
                 I = J = b;
             } else if (b < NB) {

@@ -2,4 +2,5 @@
 #define CTA_T double
 #define CTA_SUFFIX(name) name##_f64b
 #define CTA_SIZES(X) X(52) X(56) X(60) X(64)
+#define CTA_STANDALONE
 #include "proj_cta_impl.cuh"

@@ -1,7 +1,8 @@
 // CTA-per-clique projection kernels (orders 33..128 in float32, 33..64 in
 // float64): instantiations and launchers.  Included once per translation unit
 // with CTA_T (element type), CTA_SUFFIX (name suffix) and CTA_SIZES (X-macro
-// list of the padded orders instantiated there) defined.
+// list of the padded orders instantiated there) defined, and CTA_STANDALONE
+// where the standalone projection of those orders is needed.
 #include <algorithm>
 
 #include "jacobi_cta.cuh"
@@ -76,12 +77,14 @@ cudaError_t CTA_SUFFIX(launch_proj_cta)(int S, int form, const Dev& d, const int
     return cudaErrorInvalidValue;
 }
 
+#ifdef CTA_STANDALONE
 cudaError_t CTA_SUFFIX(launch_proj_cta_standalone)(int S, int p, const int* off, const int* size, const void* W,
                                                    void* X, int max_sweeps, cudaStream_t st) {
     Dev d{};
     ProjArgs pa{};
     FinishArgs fa{};
     pa.restart = 1;
+    pa.min_size = S == 128 ? 97 : (S == 96 ? 65 : kMaxWarpOrder + 1);
     switch (S) {
 #define CTA_CASE(N) \
     case N: return launch_cta<CTA_T, N, 3>(d, nullptr, p, pa, fa, off, size, W, X, max_sweeps, st);
@@ -90,5 +93,6 @@ cudaError_t CTA_SUFFIX(launch_proj_cta_standalone)(int S, int p, const int* off,
     }
     return cudaErrorInvalidValue;
 }
+#endif
 
 }  // namespace cdsdp_dev

@@ -82,6 +82,13 @@ CDSDP_DECLARE_CTA(f64a)
 CDSDP_DECLARE_CTA(f64b)
 #undef CDSDP_DECLARE_CTA
 
+// Standalone projection of a batch with device-side orders (proj_ragged.cu):
+// entries of order 1..min(limit, 32), and float entries of order 33..min(limit, 64).
+cudaError_t launch_project_ragged(bool fp32, int p, int limit, const int* off, const int* size, const void* W, void* X,
+                                  int max_sweeps, cudaStream_t st);
+cudaError_t launch_project_cta_ragged(int p, int limit, const int* off, const int* size, const void* W, void* X,
+                                      int max_sweeps, cudaStream_t st);
+
 inline cudaError_t launch_proj_cta(bool fp32, int form, int cls, const Dev& d, const int4* list, int nlist,
                                    const ProjArgs& pa, const FinishArgs& fa, cudaStream_t st) {
     const int S = kProjClasses[cls];
@@ -92,13 +99,11 @@ inline cudaError_t launch_proj_cta(bool fp32, int form, int cls, const Dev& d, c
     return S <= 48 ? launch_proj_cta_f64a(S, form, d, list, nlist, pa, fa, st)
                    : launch_proj_cta_f64b(S, form, d, list, nlist, pa, fa, st);
 }
+// Float orders above 64 (a class skips orders at or below the one before it), double orders 33..64.
 inline cudaError_t launch_proj_cta_standalone(bool fp32, int cls, int p, const int* off, const int* size,
                                               const void* W, void* X, int max_sweeps, cudaStream_t st) {
     const int S = kProjClasses[cls];
-    if (fp32)
-        return S <= 48 ? launch_proj_cta_standalone_f32a(S, p, off, size, W, X, max_sweeps, st)
-                       : (S <= 64 ? launch_proj_cta_standalone_f32b(S, p, off, size, W, X, max_sweeps, st)
-                                  : launch_proj_cta_standalone_f32c(S, p, off, size, W, X, max_sweeps, st));
+    if (fp32) return launch_proj_cta_standalone_f32c(S, p, off, size, W, X, max_sweeps, st);
     return S <= 48 ? launch_proj_cta_standalone_f64a(S, p, off, size, W, X, max_sweeps, st)
                    : launch_proj_cta_standalone_f64b(S, p, off, size, W, X, max_sweeps, st);
 }
@@ -122,21 +127,37 @@ inline int proj_launch_grid(int cls, int nlist, bool fp32, int warps_div = 1) {
     const int G = 32 / proj_lanes(S);
     return proj_shape((nlist + G - 1) / G, std::max(1, proj_max_warps(S, fp32) / std::max(1, warps_div))).grid;
 }
+// The batch of cdsdp_psd_project, orders up to kProjClasses[cls] (others are
+// left alone): the largest orders first, each family of kernels skipping the
+// entries of the others.  Eigenvalues and eigenvectors (orders <= 32) come from
+// the kernel of the class alone, one warp per entry.
 inline cudaError_t launch_proj_standalone_f32(int cls, int p, const int* off, const int* size, const void* W, void* X,
                                               void* eig, const int* voff, void* V, const int* vvoff, double tolrel,
                                               int max_sweeps, cudaStream_t st) {
-    if (kProjClasses[cls] > kMaxWarpOrder) return launch_proj_cta_standalone(true, cls, p, off, size, W, X, max_sweeps, st);
-    return kProjClasses[cls] <= 16
-               ? launch_proj_standalone_f32_small(cls, p, off, size, W, X, eig, voff, V, vvoff, tolrel, max_sweeps, st)
-               : launch_proj_standalone_f32_large(cls, p, off, size, W, X, eig, voff, V, vvoff, tolrel, max_sweeps, st);
+    const int limit = kProjClasses[cls];
+    if (eig || V)
+        return limit <= 16
+                   ? launch_proj_standalone_f32_small(cls, p, off, size, W, X, eig, voff, V, vvoff, tolrel, max_sweeps, st)
+                   : launch_proj_standalone_f32_large(cls, p, off, size, W, X, eig, voff, V, vvoff, tolrel, max_sweeps, st);
+    cudaError_t e = cudaSuccess;
+    for (int c = cls; e == cudaSuccess && kProjClasses[c] > 64; --c)
+        e = launch_proj_cta_standalone(true, c, p, off, size, W, X, max_sweeps, st);
+    if (e == cudaSuccess && limit > kMaxWarpOrder) e = launch_project_cta_ragged(p, limit, off, size, W, X, max_sweeps, st);
+    if (e == cudaSuccess) e = launch_project_ragged(true, p, limit, off, size, W, X, max_sweeps, st);
+    return e;
 }
 inline cudaError_t launch_proj_standalone_f64(int cls, int p, const int* off, const int* size, const void* W, void* X,
                                               void* eig, const int* voff, void* V, const int* vvoff, double tolrel,
                                               int max_sweeps, cudaStream_t st) {
-    if (kProjClasses[cls] > kMaxWarpOrder) return launch_proj_cta_standalone(false, cls, p, off, size, W, X, max_sweeps, st);
-    return kProjClasses[cls] <= 16
-               ? launch_proj_standalone_f64_small(cls, p, off, size, W, X, eig, voff, V, vvoff, tolrel, max_sweeps, st)
-               : launch_proj_standalone_f64_large(cls, p, off, size, W, X, eig, voff, V, vvoff, tolrel, max_sweeps, st);
+    const int limit = kProjClasses[cls];
+    if (eig || V)
+        return limit <= 16
+                   ? launch_proj_standalone_f64_small(cls, p, off, size, W, X, eig, voff, V, vvoff, tolrel, max_sweeps, st)
+                   : launch_proj_standalone_f64_large(cls, p, off, size, W, X, eig, voff, V, vvoff, tolrel, max_sweeps, st);
+    cudaError_t e = cudaSuccess;
+    if (limit > kMaxWarpOrder) e = launch_proj_cta_standalone(false, cls, p, off, size, W, X, max_sweeps, st);
+    if (e == cudaSuccess) e = launch_project_ragged(false, p, limit, off, size, W, X, max_sweeps, st);
+    return e;
 }
 
 }  // namespace cdsdp_dev
