@@ -2,16 +2,18 @@
 // iteration on the tensor cores (see large.cuh for the method), and the C ABI
 // entry point that projects a batch of packed blocks this way.
 //
-// Product kernel (one CTA per 128 x 128 output tile, 128 threads):
-//  * thread 0 of warp 0 streams 128 x 32 float tiles of A_hi, A_lo, B_hi, B_lo
+// Product kernel (one CTA of 256 threads per output tile of 128 rows and 128,
+// 64 or 32 columns):
+//  * thread 0 of warp 0 streams 32-float wide tiles of A_hi, A_lo, B_hi, B_lo
 //    into a 3-stage shared-memory ring with TMA (cp.async.bulk.tensor, 128-byte
 //    swizzle), one mbarrier per stage with the transaction byte count;
-//  * thread 0 of warp 1 issues tcgen05.mma kind::tf32 (M = N = 128, K = 8):
+//  * thread 0 of warp 1 issues tcgen05.mma kind::tf32 (M = 128, K = 8):
 //    three products per K step into one float32 accumulator in tensor memory,
 //    and frees a stage with tcgen05.commit on that stage's "empty" mbarrier;
-//  * all four warps read the accumulator back (tcgen05.ld 32x32b, one row per
-//    thread), apply D = alpha acc + beta C, split D into (tf32(D), D - tf32(D))
-//    and store the tile and its mirror (the products are symmetric).
+//  * the warps read the accumulator back (tcgen05.ld 32x32b, one row per
+//    thread, the columns split between the two groups of four warps), apply
+//    D = alpha acc + beta C, split D into (tf32(D), D - tf32(D)) and store the
+//    tile and its mirror (the products are symmetric).
 // Every wait is bounded (about a second of clock cycles): on a timeout the
 // kernel records an error code, lets its in-flight copies land (bounded
 // again), frees its tensor memory and returns; the host reports
@@ -33,6 +35,7 @@
 namespace cdsdp_large {
 namespace {
 
+constexpr int kSMs = 152;
 constexpr long long kSpinCycles = 2000000000LL;  // ~1 s at 2 GHz
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -86,16 +89,18 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
     return d;
 }
 
-// Instruction descriptor: D float32, A and B tf32, both K-major, N = M = 128.
-constexpr uint32_t kIdesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(kTile >> 3) << 17) |
-                            ((uint32_t)(kTile >> 4) << 24);
+// Instruction descriptor: D float32, A and B tf32, both K-major, M = 128, N = cols.
+__host__ __device__ constexpr uint32_t idesc(int cols) {
+    return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(cols >> 3) << 17) | ((uint32_t)(kTile >> 4) << 24);
+}
 
+template <int N>
 __device__ __forceinline__ void mma_tf32(uint32_t tmem, uint64_t a, uint64_t b, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem), "l"(a), "l"(b), "r"(kIdesc), "r"(accumulate)
+        ::"r"(tmem), "l"(a), "l"(b), "r"(idesc(N)), "r"(accumulate)
         : "memory");
 }
 
@@ -122,7 +127,9 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+template <int N>
 __global__ void __launch_bounds__(kGemmThreads, 1) k_tf32x3_sym(GemmArgs g) {
+    constexpr int kStageBytes = stage_bytes(N), kColBytes = N * kChunk * 4;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                            ~static_cast<uintptr_t>(1023));
@@ -154,7 +161,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tf32x3_sym(GemmArgs g) {
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                     "r"(kTile)
+                     "r"(N)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -178,8 +185,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tf32x3_sym(GemmArgs g) {
             const int x = kc * kChunk;
             tma_load_2d(base, mAh, x, t.ti * kTile, full0 + 8 * s);
             tma_load_2d(base + kTileBytes, mAl, x, t.ti * kTile, full0 + 8 * s);
-            tma_load_2d(base + 2 * kTileBytes, mBh, x, t.tj * kTile, full0 + 8 * s);
-            tma_load_2d(base + 3 * kTileBytes, mBl, x, t.tj * kTile, full0 + 8 * s);
+            tma_load_2d(base + 2 * kTileBytes, mBh, x, t.tj * N, full0 + 8 * s);
+            tma_load_2d(base + 2 * kTileBytes + kColBytes, mBl, x, t.tj * N, full0 + 8 * s);
             ++issued;
         }
         *issued_slot = issued;
@@ -196,10 +203,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tf32x3_sym(GemmArgs g) {
 #pragma unroll
             for (int k = 0; k < kChunk / 8; ++k) {
                 const uint64_t ah = sdesc(base + 32 * k), al = sdesc(base + kTileBytes + 32 * k);
-                const uint64_t bh = sdesc(base + 2 * kTileBytes + 32 * k), bl = sdesc(base + 3 * kTileBytes + 32 * k);
-                mma_tf32(tmem, ah, bh, (kc | k) != 0 ? 1u : 0u);
-                mma_tf32(tmem, ah, bl, 1u);
-                mma_tf32(tmem, al, bh, 1u);
+                const uint64_t bh = sdesc(base + 2 * kTileBytes + 32 * k);
+                const uint64_t bl = sdesc(base + 2 * kTileBytes + kColBytes + 32 * k);
+                mma_tf32<N>(tmem, ah, bh, (kc | k) != 0 ? 1u : 0u);
+                mma_tf32<N>(tmem, ah, bl, 1u);
+                mma_tf32<N>(tmem, al, bh, 1u);
             }
             mma_commit(empty0 + 8 * s);
         }
@@ -207,7 +215,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tf32x3_sym(GemmArgs g) {
     }
     __syncwarp();
 
-    // epilogue: thread (warp w, lane l) owns row 32 w + l of the tile
+    // epilogue: thread (warp w, lane l) owns row 32 (w mod 4) + l of the tile
     bool ok = mbar_wait(done, 0);
     if (!ok) atomicExch(g.err, 3);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -219,18 +227,19 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tf32x3_sym(GemmArgs g) {
         // B operand enters transposed, so an antisymmetric remainder left in an
         // iterate would be amplified by the sign iteration near eigenvalue 0.
         const int S = B.S;
-        const int r = 32 * warp + lane;
-        const bool diag = t.ti == t.tj;
+        const int wr = warp & 3, half = warp >> 2;
+        const int r = 32 * wr + lane;
+        const bool diag = t.tj * N >= t.ti * kTile;  // the tile reaches the diagonal
         const long long gr = (long long)t.ti * kTile + r;
         const float* Ch = g.C_hi ? g.C_hi + B.off : nullptr;
         const float* Cl = g.C_lo ? g.C_lo + B.off : nullptr;
         float* Dh = g.D_hi + B.off;
         float* Dl = g.D_lo ? g.D_lo + B.off : nullptr;
 #pragma unroll 1
-        for (int cc = 0; cc < kTile / 32; ++cc) {
+        for (int cc = half; cc < N / 32; cc += 2) {
             uint32_t v[32];
-            tmem_ld32(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(32 * cc), v);
-            const long long gc0 = (long long)t.tj * kTile + 32 * cc;
+            tmem_ld32(tmem + ((uint32_t)(32 * wr) << 16) + (uint32_t)(32 * cc), v);
+            const long long gc0 = (long long)t.tj * N + 32 * cc;
             float hi[32], lo[32];
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
@@ -260,11 +269,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tf32x3_sym(GemmArgs g) {
             } else {
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
-                    const int lc = 32 * cc + j;  // column within the tile
-                    if (lc > r) continue;        // upper triangle: written as the mirror of (lc, r)
+                    const long long gc = gc0 + j;
+                    if (gc > gr) continue;       // upper triangle: written as the mirror of (gc, gr)
                     Dh[gr * S + gc0 + j] = hi[j];
                     if (Dl) Dl[gr * S + gc0 + j] = lo[j];
-                    if (lc < r) {
+                    if (gc < gr) {
                         Dh[(gc0 + j) * S + gr] = hi[j];
                         if (Dl) Dl[(gc0 + j) * S + gr] = lo[j];
                     }
@@ -283,22 +292,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tf32x3_sym(GemmArgs g) {
     __syncthreads();
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTile) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(N) : "memory");
     }
 }
 
 // ---- element-wise kernels ---------------------------------------------------
-
-// (a, b), a >= b, of packed (lower, column-major) element f of an s x s block.
-__device__ __forceinline__ void packed_rc(long long f, int s, int& a, int& b) {
-    const double t = 2.0 * s + 1.0;
-    int bb = (int)((t - sqrt(t * t - 8.0 * (double)f)) * 0.5);
-    bb = max(0, min(bb, s - 1));
-    while (bb > 0 && (long long)bb * (2 * s - bb + 1) / 2 > f) --bb;
-    while (bb + 1 < s && (long long)(bb + 1) * (2 * s - bb) / 2 <= f) ++bb;
-    b = bb;
-    a = bb + (int)(f - (long long)bb * (2 * s - bb + 1) / 2);
-}
 
 // Dense symmetric W (hi, lo) of block k from its packed lower values (grid.y = block).
 __global__ void k_dense_from_packed(const Block* __restrict__ blocks, const long long* __restrict__ poff,
@@ -320,7 +318,7 @@ __global__ void k_dense_from_packed(const Block* __restrict__ blocks, const long
 
 // Partial sums of ||W||_F^2 over fixed chunks of each block's dense rows
 // (deterministic: one partial per (block, chunk), summed in order below).
-constexpr int kNormChunkRows = 32;
+constexpr int kNormChunkRows = 8;  // 190 thread blocks at order 1500
 __global__ void k_norm_partials(const Block* __restrict__ blocks, const int* __restrict__ chunk_off,
                                 const float* __restrict__ Wh, const float* __restrict__ Wl, double* partial) {
     const int k = blockIdx.y;
@@ -353,11 +351,22 @@ __global__ void k_scale_start(const Block* __restrict__ blocks, const int* __res
                               const float* __restrict__ Wl, float* Xh, float* Xl, double* scale) {
     const int k = blockIdx.y;
     const Block B = blocks[k];
-    double s2 = 0.0;
-    for (int c = chunk_off[k]; c < chunk_off[k + 1]; ++c) s2 += partial[c];
-    const double nrm = sqrt(s2);
-    if (blockIdx.x == 0 && threadIdx.x == 0) scale[k] = nrm;
-    const float inv = nrm > 0.0 ? (float)(1.0 / nrm) : 0.f;
+    // one warp adds the partial sums for its block (every thread did: 93 us of
+    // float64 additions at order 1500)
+    __shared__ float s_inv;
+    if (threadIdx.x < 32) {
+        double s2 = 0.0;
+        for (int c = chunk_off[k] + threadIdx.x; c < chunk_off[k + 1]; c += 32) s2 += partial[c];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        if (threadIdx.x == 0) {
+            const double nrm = sqrt(s2);
+            if (blockIdx.x == 0) scale[k] = nrm;
+            s_inv = nrm > 0.0 ? (float)(1.0 / nrm) : 0.f;
+        }
+    }
+    __syncthreads();
+    const float inv = s_inv;
     const long long ne = (long long)B.S * B.S;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < ne; e += (long long)gridDim.x * blockDim.x) {
         const float x = (Wh[B.off + e] + Wl[B.off + e]) * inv;
@@ -399,10 +408,10 @@ bool get_encode() {
     return true;
 }
 
-bool encode_map(CUtensorMap* m, const float* base, int S) {
+bool encode_map(CUtensorMap* m, const float* base, int S, int rows) {
     const cuuint64_t dims[2] = {(cuuint64_t)S, (cuuint64_t)S};
     const cuuint64_t strides[1] = {(cuuint64_t)S * 4};
-    const cuuint32_t box[2] = {(cuuint32_t)kChunk, (cuuint32_t)kTile};
+    const cuuint32_t box[2] = {(cuuint32_t)kChunk, (cuuint32_t)rows};
     const cuuint32_t estr[2] = {1, 1};
     return g_encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -428,9 +437,6 @@ NsLayout ns_layout(const std::vector<int>& sizes) {
         b.off = off;
         off += (long long)b.S * b.S;
         L.blocks.push_back(b);
-        const int nt = b.S / kTile;
-        for (int i = 0; i < nt; ++i)
-            for (int j = 0; j <= i; ++j) L.tiles.push_back(Tile{(int)L.blocks.size() - 1, i, j, 0});
         chunks += (b.S + kNormChunkRows - 1) / kNormChunkRows;
         L.chunk_off.push_back(chunks);
         L.max_S = std::max(L.max_S, b.S);
@@ -440,10 +446,19 @@ NsLayout ns_layout(const std::vector<int>& sizes) {
         L.max_upd = std::max(L.max_upd, nu);
     }
     if (L.upd_off.empty()) L.upd_off.push_back(0);
+    long long wide = 0;  // 128 x 128 tiles
+    for (const Block& b : L.blocks) wide += (long long)(b.S / kTile) * (b.S / kTile + 1) / 2;
+    L.cols = wide * 4 <= kSMs ? 32 : (wide * 2 <= kSMs ? 64 : kMaxCols);
+    for (size_t k = 0; k < L.blocks.size(); ++k)
+        for (int i = 0; i < L.blocks[k].S / kTile; ++i)
+            for (int j = 0; j * L.cols < (i + 1) * kTile; ++j) L.tiles.push_back(Tile{(int)k, i, j, 0});
     L.elems = off;
     size_t o = 0;
     L.o_err = o; o = up256(o + 16);
     L.o_maps = o; o = up256(o + sizeof(CUtensorMap) * 2 * NBUF * (size_t)std::max(1, L.nb));
+    L.o_maps_b = o;  // operand B's boxes are as high as a tile is wide
+    if (L.cols != kTile) o = up256(o + sizeof(CUtensorMap) * 2 * NBUF * (size_t)std::max(1, L.nb));
+    else L.o_maps_b = L.o_maps;
     L.o_tiles = o; o = up256(o + sizeof(Tile) * std::max<size_t>(1, L.tiles.size()));
     L.o_blocks = o; o = up256(o + sizeof(Block) * std::max(1, L.nb));
     L.o_chunk = o; o = up256(o + sizeof(int) * (L.nb + 1));
@@ -469,10 +484,12 @@ bool ns_tables(const NsLayout& L, unsigned char* base, const std::vector<long lo
     if (!get_encode()) return false;
     img.assign(L.o_buf[0], 0);
     CUtensorMap* maps = reinterpret_cast<CUtensorMap*>(img.data() + L.o_maps);
+    CUtensorMap* maps_b = reinterpret_cast<CUtensorMap*>(img.data() + L.o_maps_b);
     for (int buf = 0; buf < 2 * NBUF; ++buf)
         for (int k = 0; k < L.nb; ++k) {
             const float* p = reinterpret_cast<const float*>(base + L.o_buf[buf]) + L.blocks[k].off;
-            if (!encode_map(&maps[buf * L.nb + k], p, L.blocks[k].S)) return false;
+            if (!encode_map(&maps[buf * L.nb + k], p, L.blocks[k].S, kTile)) return false;
+            if (L.cols != kTile && !encode_map(&maps_b[buf * L.nb + k], p, L.blocks[k].S, L.cols)) return false;
         }
     std::memcpy(img.data() + L.o_tiles, L.tiles.data(), sizeof(Tile) * L.tiles.size());
     std::memcpy(img.data() + L.o_blocks, L.blocks.data(), sizeof(Block) * L.blocks.size());
@@ -485,20 +502,27 @@ bool ns_tables(const NsLayout& L, unsigned char* base, const std::vector<long lo
 
 namespace {
 
-cudaError_t gemm(const NsLayout& L, unsigned char* base, int a, int bsrc, int c, int d, float alpha, float beta,
-                 bool split, cudaStream_t st) {
+template <int N>
+cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t st) {
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_tf32x3_sym, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
+        cudaError_t e = cudaFuncSetAttribute(k_tf32x3_sym<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(N));
         if (e != cudaSuccess) return e;
         attr = true;
     }
+    k_tf32x3_sym<N><<<g.ntiles, kGemmThreads, gemm_smem(N), st>>>(g);
+    return cudaGetLastError();
+}
+
+cudaError_t gemm(const NsLayout& L, unsigned char* base, int a, int bsrc, int c, int d, float alpha, float beta,
+                 bool split, cudaStream_t st) {
     const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(base + L.o_maps);
+    const CUtensorMap* maps_b = reinterpret_cast<const CUtensorMap*>(base + L.o_maps_b);
     GemmArgs g;
     g.mapA_hi = maps + (2 * a) * L.nb;
     g.mapA_lo = maps + (2 * a + 1) * L.nb;
-    g.mapB_hi = maps + (2 * bsrc) * L.nb;
-    g.mapB_lo = maps + (2 * bsrc + 1) * L.nb;
+    g.mapB_hi = maps_b + (2 * bsrc) * L.nb;
+    g.mapB_lo = maps_b + (2 * bsrc + 1) * L.nb;
     g.C_hi = c >= 0 ? reinterpret_cast<const float*>(base + L.o_buf[2 * c]) : nullptr;
     g.C_lo = c >= 0 ? reinterpret_cast<const float*>(base + L.o_buf[2 * c + 1]) : nullptr;
     g.D_hi = reinterpret_cast<float*>(base + L.o_buf[2 * d]);
@@ -509,8 +533,7 @@ cudaError_t gemm(const NsLayout& L, unsigned char* base, int a, int bsrc, int c,
     g.alpha = alpha;
     g.beta = beta;
     g.err = reinterpret_cast<int*>(base + L.o_err);
-    k_tf32x3_sym<<<g.ntiles, kGemmThreads, kGemmSmem, st>>>(g);
-    return cudaGetLastError();
+    return L.cols == 32 ? launch_gemm<32>(g, st) : (L.cols == 64 ? launch_gemm<64>(g, st) : launch_gemm<128>(g, st));
 }
 
 }  // namespace

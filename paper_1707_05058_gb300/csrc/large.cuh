@@ -33,19 +33,28 @@
 
 namespace cdsdp_large {
 
-constexpr int kTile = 128;         // output tile (M = N = 128), one CTA each
+constexpr int kTile = 128;         // rows of an output tile, one CTA each
+// Columns of an output tile: 128, or 64 or 32 when the batch has so few
+// 128 x 128 tiles that the narrower ones still fit one wave of the 152 SMs.  An
+// SM takes in about 45 B a clock from L2, which is what a K step costs (64 KB
+// of operands at 128 columns, 48 KB at 64, 40 KB at 32, where its MMAs take
+// 840, 420 and 210 clocks), so the narrow tiles are less efficient but finish
+// sooner while SMs would stand idle otherwise.  Every entry is the same sum in
+// the same order at each width.
+constexpr int kMaxCols = 128;
 constexpr int kChunk = 32;         // K floats per stage: one 128-byte swizzle row
 constexpr int kStages = 3;
-constexpr int kTileBytes = kTile * kChunk * 4;       // 16 KB per operand tile
-constexpr int kStageBytes = 4 * kTileBytes;          // A_hi, A_lo, B_hi, B_lo
-constexpr int kGemmSmem = kStages * kStageBytes + 1024 + 256;
-constexpr int kGemmThreads = 128;
+constexpr int kTileBytes = kTile * kChunk * 4;       // 16 KB per operand tile of 128 rows
+__host__ __device__ constexpr int stage_bytes(int cols) { return 2 * kTileBytes + 2 * cols * kChunk * 4; }  // A_hi, A_lo, B_hi, B_lo
+constexpr int gemm_smem(int cols) { return kStages * stage_bytes(cols) + 1024 + 256; }
+constexpr int kGemmThreads = 256;  // producer, MMA issuer; all warps read the accumulator
 
 // Phase-1 polynomial and the iteration counts.
 constexpr float kPa = 3.30f, kPb = -3.66f, kPc = 1.36f;
 constexpr int kPhase1 = 16, kPhase2 = 5;
 
-// One output tile (ti, tj), ti >= tj, of block `blk`.
+// One output tile of block `blk`: rows 128 ti .., columns (tile width) tj ..; it
+// reaches into the lower triangle.
 struct Tile { int blk, ti, tj, pad; };
 
 // Dense layout of one block in every buffer: float offset and padded order.
@@ -67,5 +76,18 @@ struct GemmArgs {
     float alpha, beta;
     int* err;                                   // set on a timed-out wait (kernel returns early)
 };
+
+// (a, b), a >= b, of packed (lower, column-major) element f of an s x s block:
+// the column from an exact integer radicand and a float32 root (a float64 root
+// costs some forty operations of the slow float64 pipe), then exact.
+__device__ __forceinline__ void packed_rc(long long f, int s, int& a, int& b) {
+    const long long t = 2LL * s + 1;
+    int bb = (int)(((float)t - sqrtf((float)(t * t - 8 * f))) * 0.5f);
+    bb = max(0, min(bb, s - 1));
+    while (bb > 0 && (long long)bb * (2 * s - bb + 1) / 2 > f) --bb;
+    while (bb + 1 < s && (long long)(bb + 1) * (2 * s - bb) / 2 <= f) ++bb;
+    b = bb;
+    a = bb + (int)(f - (long long)bb * (2 * s - bb + 1) / 2);
+}
 
 }  // namespace cdsdp_large

@@ -16,21 +16,22 @@ constexpr int kMaxLargeOrder = 8192;
 constexpr int kLargeFrom = 129;
 
 // Packed entries per thread block of the gather and update kernels.
-constexpr int kUpdChunk = 8192;
+constexpr int kUpdChunk = 2048;
 
 // Device memory of one batch of large blocks: tables, then 2 * NBUF dense
 // float buffers (the (hi, lo) pairs of W, X_a, X_b, X^2, B), each holding
 // every block at Block::off with row pitch Block::S.
 struct NsLayout {
     int nb = 0;
+    int cols = kMaxCols;            // columns of an output tile
     int max_S = 0;
     long long elems = 0;            // floats per buffer
     std::vector<Block> blocks;
-    std::vector<Tile> tiles;        // lower output tiles of every block
+    std::vector<Tile> tiles;        // output tiles of every block that reach its lower triangle
     std::vector<int> chunk_off;     // row chunks of the norm reduction, per block
     std::vector<int> upd_off;       // packed-entry chunks of the gather / update, per block
     int max_upd = 0;                // most packed-entry chunks of one block
-    size_t o_err = 0, o_maps = 0, o_tiles = 0, o_blocks = 0, o_chunk = 0, o_partial = 0, o_scale = 0, o_poff = 0;
+    size_t o_err = 0, o_maps = 0, o_maps_b = 0, o_tiles = 0, o_blocks = 0, o_chunk = 0, o_partial = 0, o_scale = 0, o_poff = 0;
     size_t o_list = 0, o_upd = 0, o_updpart = 0;
     size_t o_buf[2 * NBUF] = {0};
     size_t bytes = 0;

@@ -26,17 +26,6 @@ __device__ __forceinline__ float tf32_rn(float x) {
     return __uint_as_float(r);
 }
 
-// (a, b), a >= b, of packed (lower, column-major) element f of an s x s block.
-__device__ __forceinline__ void packed_ab64(long long f, int s, int& a, int& b) {
-    const double t = 2.0 * s + 1.0;
-    int bb = (int)((t - sqrt(t * t - 8.0 * (double)f)) * 0.5);
-    bb = max(0, min(bb, s - 1));
-    while (bb > 0 && (long long)bb * (2 * s - bb + 1) / 2 > f) --bb;
-    while (bb + 1 < s && (long long)(bb + 1) * (2 * s - bb) / 2 <= f) ++bb;
-    b = bb;
-    a = bb + (int)(f - (long long)bb * (2 * s - bb + 1) / 2);
-}
-
 struct Step {
     const Block* blocks;
     const int* list;     // clique of each block
@@ -64,7 +53,7 @@ __global__ void __launch_bounds__(256) k_large_gather(Dev d, Step t) {
     const double gamma = FORM == 2 ? cdsdp_dev::hs_gamma_c(d, cdsdp_dev::comp_k(d, k)) : 0.0;
     for (long long f = f0 + threadIdx.x; f < f1; f += blockDim.x) {
         int a, b;
-        packed_ab64(f, B.s, a, b);
+        packed_rc(f, B.s, a, b);
         double w;
         if (FORM == 0) {         // H_k x - lambda_k / rho (x from its own kernel)
             w = d.x[d.gmap[off + f]] - double(c1[off + f]) * irho;
@@ -102,7 +91,7 @@ __global__ void __launch_bounds__(256) k_large_update(Dev d, Step t) {
     double p[6] = {0, 0, 0, 0, 0, 0};
     for (long long f = f0 + threadIdx.x; f < f1; f += blockDim.x) {
         int a, b;
-        packed_ab64(f, B.s, a, b);
+        packed_rc(f, B.s, a, b);
         const float xn = t.P[B.off + (long long)a * B.S + b];
         const double w = (a == b) ? 1.0 : 2.0;
         if (FORM == 0) {  // x_k <- P(W), lambda_k <- lambda_k + rho (x_k - H_k x)
@@ -151,10 +140,13 @@ __global__ void __launch_bounds__(128) k_large_reduce(Dev d, Step t, int row_off
     const int i = blockIdx.x;
     const int k = t.list[i];
     const bool frozen = cdsdp_dev::frozen_clique(d, k);
-    if (threadIdx.x == 0 && !frozen) {
-        double s[6] = {0, 0, 0, 0, 0, 0};
-        for (int c = t.upd[i]; c < t.upd[i + 1]; ++c)
+    double s[6] = {0, 0, 0, 0, 0, 0};
+    if (threadIdx.x < 32 && !frozen) {
+        for (int c = t.upd[i] + threadIdx.x; c < t.upd[i + 1]; c += 32)
             for (int j = 0; j < 6; ++j) s[j] += t.part[(size_t)c * 8 + j];
+        for (int j = 0; j < 6; ++j) s[j] = cdsdp_dev::warp_sum(s[j]);
+    }
+    if (threadIdx.x == 0 && !frozen) {
         double* pr = d.part + (size_t)(d.comp_mode ? k : row_off + i) * cdsdp_dev::PART_COLS;
         if (FORM == 1) {
             pr[5] = s[0];
