@@ -44,7 +44,7 @@ reductions).
             11): time to 1e-4 in the FP32 graph and plain FP64 forms
   maxcut    the MaxCut workload (n = 10^4, G(n, 6/(n-1)), merged cliques up to
             order 3560): clique histogram, per-iteration split, the tensor-core
-            sign iteration against the TF32 peak, FP32 solve to 1e-4 (capped)
+            sign iteration against the 16-bit peak, FP32 solve to 1e-4 (capped)
   cpu_baseline  the FP64 oracle on a bounded sample of the same batch: 8 of its
             SDPs, 4 iterations each, on 1 host thread and on one process per
             SDP
@@ -445,7 +445,7 @@ def _maxcut(cdsdp, workloads, torch, flush, stream, max_iter=2500):
     lg_ms = lg["ms"] / max(1, lg["launches"])
     tensor_tflops = lg["tensor_flops"] / (lg_ms / 1e3) / 1e12
     pk = _peaks()
-    tf32_peak = pk.get("bf16_tflops", 1910.0) * (1.1 / 2.25)  # nominal tf32 / bf16 dense ratio
+    f16_peak = pk.get("bf16_tflops", 1910.0)  # float16 and bfloat16 have one rate
     flush.fill_(1)
     ms, out = _event_ms(torch, stream, lambda: P.solve("primal", outputs=False, eps=1e-4, max_iter=max_iter,
                                                        precision="fp32", adaptive_rho=1))
@@ -454,10 +454,10 @@ def _maxcut(cdsdp, workloads, torch, flush, stream, max_iter=2500):
             "n_d_lower": int(P.info["n_d_lower"]), "components": int(P.info["ncomp"]), "setup_s": setup_s,
             "ms_per_iter": iter_ms / launches, "proj_ms_per_iter": proj_ms / launches,
             "large_cliques": lg["cliques"], "large_step_ms_per_iter": lg_ms,
-            "tensor_roofline": {"bound": "tensor", "achieved": tensor_tflops, "peak": tf32_peak, "unit": "TFLOP/s",
-                                "frac": tensor_tflops / tf32_peak,
-                                "peak_source": "measured bf16 burst (MEASURED_PEAKS.json) x nominal tf32/bf16 ratio",
-                                "work": "59 products x 3 TF32 MMAs over the lower 128x128 tiles per step"},
+            "tensor_roofline": {"bound": "tensor", "achieved": tensor_tflops, "peak": f16_peak, "unit": "TFLOP/s",
+                                "frac": tensor_tflops / f16_peak,
+                                "peak_source": "measured bf16 burst (MEASURED_PEAKS.json)",
+                                "work": "59 products x 3 float16 MMAs over the lower 128x128 tiles per step"},
             "fp32_primal": {"status": int(out["status"]), "iters": int(out["iters"]), "ms": ms, "max_iter": max_iter}}
 
 

@@ -388,7 +388,7 @@ int cdsdp_profile_orders(const cdsdp* h, int* orders, double* ms, int* launches,
  *   cliques        cliques of order > 128
  *   nominal_flops  sum of 10 s^3 over those cliques (the same nominal count as
  *                  cdsdp_profile_orders)
- *   tensor_flops   tensor-core work of one step: 59 products x 3 TF32 MMAs over
+ *   tensor_flops   tensor-core work of one step: 59 products x 3 float16 MMAs over
  *                  the lower 128 x 128 tiles of each padded block (2 flops per
  *                  multiply-add)
  * Errors: CDSDP_ERR_ARG, CDSDP_ERR_STATE when the last solve was not profiled. */
@@ -481,8 +481,9 @@ int cdsdp_unrolled_backward(cdsdp* h, const cdsdp_opts* opts, int iters, int ckp
  * Jacobi eigensolver).  P(W) = (W + W sign(W)) / 2 with sign(W) from an odd
  * polynomial (Newton-Schulz) iteration on W / ||W||_F: 16 steps of
  * X <- 3.30 X - 3.66 X^3 + 1.36 X^5, then 5 steps of X <- 1.5 X - 0.5 X^3,
- * every product of two (commuting, symmetric) matrices as three TF32
- * tcgen05 products (float32 accuracy), lower 128 x 128 tiles only.
+ * every product of two (commuting, symmetric) matrices as three float16
+ * tcgen05 products of pairs that hold 22 bits (float32 accuracy), lower tiles
+ * only.
  * Eigenvalues with |lambda| < 1e-8 ||W||_F may stay unconverged; each adds at
  * most |lambda| / 2 to the error of P.
  *   p        number of blocks
@@ -492,8 +493,8 @@ int cdsdp_unrolled_backward(cdsdp* h, const cdsdp_opts* opts, int iters, int ckp
  *   d_W      device float32: input blocks;  d_X  device float32: P(W_k), same layout
  *   d_scratch  device scratch, 256-byte aligned, at least
  *            cdsdp_psd_project_large_bytes(p, h_size) bytes: the tensor maps
- *            of the iteration and ten dense float copies of every block
- *            (order rounded up to a multiple of 128)
+ *            of the iteration and six dense copies of every block at four
+ *            bytes an entry (order rounded up to a multiple of 128)
  * Synchronises `stream`.  Errors: CDSDP_ERR_ARG, CDSDP_ERR_NOMEM (scratch too
  * small), CDSDP_ERR_CUDA (also when the driver's tensor-map encoder is
  * unavailable), CDSDP_ERR_TIMEOUT (a bounded wait inside the product kernel

@@ -4,16 +4,16 @@
 //
 // Product kernel (one CTA of 256 threads per output tile of 128 rows and 128,
 // 64 or 32 columns):
-//  * thread 0 of warp 0 streams 32-float wide tiles of A_hi, A_lo, B_hi, B_lo
+//  * thread 0 of warp 0 streams 64-half wide tiles of A_hi, A_lo, B_hi, B_lo
 //    into a 3-stage shared-memory ring with TMA (cp.async.bulk.tensor, 128-byte
 //    swizzle), one mbarrier per stage with the transaction byte count;
-//  * thread 0 of warp 1 issues tcgen05.mma kind::tf32 (M = 128, K = 8):
-//    three products per K step into one float32 accumulator in tensor memory,
-//    and frees a stage with tcgen05.commit on that stage's "empty" mbarrier;
+//  * thread 0 of warp 1 issues tcgen05.mma kind::f16 (M = 128, K = 16):
+//    three products per K step into two float32 accumulators in tensor memory
+//    (hi hi; hi lo + lo hi), and frees a stage with tcgen05.commit on that stage's "empty" mbarrier;
 //  * the warps read the accumulator back (tcgen05.ld 32x32b, one row per
 //    thread, the columns split between the two groups of four warps), apply
-//    D = alpha acc + beta C, split D into (tf32(D), D - tf32(D)) and store the
-//    tile and its mirror (the products are symmetric).
+//    D = alpha acc + beta C, split D into its (hi, lo) pair and store the tile
+//    and its mirror (the products are symmetric).
 // Every wait is bounded (about a second of clock cycles): on a timeout the
 // kernel records an error code, lets its in-flight copies land (bounded
 // again), frees its tensor memory and returns; the host reports
@@ -89,29 +89,23 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
     return d;
 }
 
-// Instruction descriptor: D float32, A and B tf32, both K-major, M = 128, N = cols.
+// Instruction descriptor: D float32, A and B float16, both K-major, M = 128, N = cols.
 __host__ __device__ constexpr uint32_t idesc(int cols) {
-    return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(cols >> 3) << 17) | ((uint32_t)(kTile >> 4) << 24);
+    return (1u << 4) | ((uint32_t)(cols >> 3) << 17) | ((uint32_t)(kTile >> 4) << 24);
 }
 
 template <int N>
-__device__ __forceinline__ void mma_tf32(uint32_t tmem, uint64_t a, uint64_t b, uint32_t accumulate) {
+__device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t a, uint64_t b, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(tmem), "l"(a), "l"(b), "r"(idesc(N)), "r"(accumulate)
         : "memory");
 }
 
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ float tf32_round(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
 }
 
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
@@ -127,9 +121,29 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// 32 columns of this thread's row of A B, from the two accumulators N columns
+// apart (of operands scaled by kPairScale each).
 template <int N>
-__global__ void __launch_bounds__(kGemmThreads, 1) k_tf32x3_sym(GemmArgs g) {
-    constexpr int kStageBytes = stage_bytes(N), kColBytes = N * kChunk * 4;
+__device__ __forceinline__ void load_acc(uint32_t taddr, float (&v)[32]) {
+    uint32_t a[32], b[32];
+    tmem_ld32(taddr, a);
+    tmem_ld32(taddr + N, b);
+    constexpr float s = 1.f / (kPairScale * kPairScale);
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = s * fmaf(1.f / kLoScale, __uint_as_float(b[j]), __uint_as_float(a[j]));
+}
+
+__device__ __forceinline__ uint4 pack8(const __half* h) {
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        w[i] = (uint32_t)__half_as_ushort(h[2 * i]) | ((uint32_t)__half_as_ushort(h[2 * i + 1]) << 16);
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+template <int N>
+__global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
+    constexpr int kStageBytes = stage_bytes(N), kColBytes = N * kChunk * 2;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                            ~static_cast<uintptr_t>(1023));
@@ -161,7 +175,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tf32x3_sym(GemmArgs g) {
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                     "r"(N)
+                     "r"(2 * N)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -201,13 +215,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tf32x3_sym(GemmArgs g) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t base = smem_u32(smem + s * kStageBytes);
 #pragma unroll
-            for (int k = 0; k < kChunk / 8; ++k) {
+            for (int k = 0; k < kChunk / 16; ++k) {
                 const uint64_t ah = sdesc(base + 32 * k), al = sdesc(base + kTileBytes + 32 * k);
                 const uint64_t bh = sdesc(base + 2 * kTileBytes + 32 * k);
                 const uint64_t bl = sdesc(base + 2 * kTileBytes + kColBytes + 32 * k);
-                mma_tf32<N>(tmem, ah, bh, (kc | k) != 0 ? 1u : 0u);
-                mma_tf32<N>(tmem, ah, bl, 1u);
-                mma_tf32<N>(tmem, al, bh, 1u);
+                mma_f16<N>(tmem, ah, bh, (kc | k) != 0 ? 1u : 0u);
+                mma_f16<N>(tmem + N, ah, bl, (kc | k) != 0 ? 1u : 0u);
+                mma_f16<N>(tmem + N, al, bh, 1u);
             }
             mma_commit(empty0 + 8 * s);
         }
@@ -231,51 +245,74 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tf32x3_sym(GemmArgs g) {
         const int r = 32 * wr + lane;
         const bool diag = t.tj * N >= t.ti * kTile;  // the tile reaches the diagonal
         const long long gr = (long long)t.ti * kTile + r;
-        const float* Ch = g.C_hi ? g.C_hi + B.off : nullptr;
-        const float* Cl = g.C_lo ? g.C_lo + B.off : nullptr;
-        float* Dh = g.D_hi + B.off;
-        float* Dl = g.D_lo ? g.D_lo + B.off : nullptr;
+        const uint32_t row = tmem + ((uint32_t)(32 * wr) << 16);
+        if (g.P) {  // P = (W + |W|_F A B) / 2; |W|_F in two floats, so that its rounding does not scale W sign(W)
+            const double nrm = g.scale[t.blk];
+            const float up = nrm > 1e30 ? 16777216.f : 1.f;  // |W|_F itself may pass the float32 range
+            const float nh = (float)(nrm / up), nl = (float)(nrm / up - (double)nh);
+            const float* Wk = g.W + B.off;
+            float* P = g.P + B.off;
 #pragma unroll 1
-        for (int cc = half; cc < N / 32; cc += 2) {
-            uint32_t v[32];
-            tmem_ld32(tmem + ((uint32_t)(32 * wr) << 16) + (uint32_t)(32 * cc), v);
-            const long long gc0 = (long long)t.tj * N + 32 * cc;
-            float hi[32], lo[32];
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                // C is symmetric: read its entry (gc, gr), consecutive over the warp's rows
-                float c = 0.f;
-                if (Ch) c = Ch[(gc0 + j) * S + gr] + Cl[(gc0 + j) * S + gr];
-                const float d = g.alpha * __uint_as_float(v[j]) + g.beta * c;
-                hi[j] = Dl ? tf32_round(d) : d;
-                lo[j] = d - hi[j];
-            }
-            if (!diag) {
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {  // mirror (gc, gr): coalesced over the warp
-                    const long long mi = (gc0 + j) * S + gr;
-                    Dh[mi] = hi[j];
-                    if (Dl) Dl[mi] = lo[j];
-                }
-                float4* dh4 = reinterpret_cast<float4*>(Dh + gr * S + gc0);
-#pragma unroll
-                for (int q = 0; q < 8; ++q) dh4[q] = make_float4(hi[4 * q], hi[4 * q + 1], hi[4 * q + 2], hi[4 * q + 3]);
-                if (Dl) {
-                    float4* dl4 = reinterpret_cast<float4*>(Dl + gr * S + gc0);
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        dl4[q] = make_float4(lo[4 * q], lo[4 * q + 1], lo[4 * q + 2], lo[4 * q + 3]);
-                }
-            } else {
+            for (int cc = half; cc < N / 32; cc += 2) {
+                float v[32];
+                load_acc<N>(row + (uint32_t)(32 * cc), v);
+                const long long gc0 = (long long)t.tj * N + 32 * cc;
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
-                    const long long gc = gc0 + j;
-                    if (gc > gr) continue;       // upper triangle: written as the mirror of (gc, gr)
-                    Dh[gr * S + gc0 + j] = hi[j];
-                    if (Dl) Dl[gr * S + gc0 + j] = lo[j];
-                    if (gc < gr) {
-                        Dh[(gc0 + j) * S + gr] = hi[j];
-                        if (Dl) Dl[(gc0 + j) * S + gr] = lo[j];
+                    // W is symmetric: read its entry (gc, gr), consecutive over the warp's rows
+                    const float w = Wk[(gc0 + j) * S + gr];
+                    v[j] = 0.5f * fmaf(v[j] * up, nh, fmaf(v[j] * up, nl, w));
+                }
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    if (diag && gc0 + j > gr) continue;  // upper triangle: written as the mirror of (gc, gr)
+                    P[gr * S + gc0 + j] = v[j];
+                    P[(gc0 + j) * S + gr] = v[j];
+                }
+            }
+        } else {
+            const __half* Ch = g.C_hi ? g.C_hi + B.off : nullptr;
+            const __half* Cl = g.C_lo ? g.C_lo + B.off : nullptr;
+            __half* Dh = g.D_hi + B.off;
+            __half* Dl = g.D_lo + B.off;
+#pragma unroll 1
+            for (int cc = half; cc < N / 32; cc += 2) {
+                float v[32];
+                load_acc<N>(row + (uint32_t)(32 * cc), v);
+                const long long gc0 = (long long)t.tj * N + 32 * cc;
+                __half hi[32], lo[32];
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    // C is symmetric: read its entry (gc, gr), consecutive over the warp's rows
+                    float c = 0.f;
+                    if (Ch) c = pair_value(Ch[(gc0 + j) * S + gr], Cl[(gc0 + j) * S + gr]);
+                    pair_split(g.alpha * v[j] + g.beta * c, hi[j], lo[j]);
+                }
+                if (!diag) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) {  // mirror (gc, gr): coalesced over the warp
+                        const long long mi = (gc0 + j) * S + gr;
+                        Dh[mi] = hi[j];
+                        Dl[mi] = lo[j];
+                    }
+                    uint4* dh4 = reinterpret_cast<uint4*>(Dh + gr * S + gc0);
+                    uint4* dl4 = reinterpret_cast<uint4*>(Dl + gr * S + gc0);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        dh4[q] = pack8(hi + 8 * q);
+                        dl4[q] = pack8(lo + 8 * q);
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) {
+                        const long long gc = gc0 + j;
+                        if (gc > gr) continue;
+                        Dh[gr * S + gc] = hi[j];
+                        Dl[gr * S + gc] = lo[j];
+                        if (gc < gr) {
+                            Dh[gc * S + gr] = hi[j];
+                            Dl[gc * S + gr] = lo[j];
+                        }
                     }
                 }
             }
@@ -292,15 +329,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tf32x3_sym(GemmArgs g) {
     __syncthreads();
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(N) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * N) : "memory");
     }
 }
 
 // ---- element-wise kernels ---------------------------------------------------
 
-// Dense symmetric W (hi, lo) of block k from its packed lower values (grid.y = block).
+// Dense symmetric W of block k from its packed lower values (grid.y = block).
 __global__ void k_dense_from_packed(const Block* __restrict__ blocks, const long long* __restrict__ poff,
-                                    const float* __restrict__ Wp, float* Wh, float* Wl) {
+                                    const float* __restrict__ Wp, float* W) {
     const int k = blockIdx.y;
     const Block B = blocks[k];
     const long long npk = (long long)B.s * (B.s + 1) / 2;
@@ -308,11 +345,8 @@ __global__ void k_dense_from_packed(const Block* __restrict__ blocks, const long
         int a, b;
         packed_rc(f, B.s, a, b);
         const float w = Wp[poff[k] + f];
-        const float h = tf32_round(w), l = w - h;
-        Wh[B.off + (long long)a * B.S + b] = h;
-        Wl[B.off + (long long)a * B.S + b] = l;
-        Wh[B.off + (long long)b * B.S + a] = h;
-        Wl[B.off + (long long)b * B.S + a] = l;
+        W[B.off + (long long)a * B.S + b] = w;
+        W[B.off + (long long)b * B.S + a] = w;
     }
 }
 
@@ -320,7 +354,7 @@ __global__ void k_dense_from_packed(const Block* __restrict__ blocks, const long
 // (deterministic: one partial per (block, chunk), summed in order below).
 constexpr int kNormChunkRows = 8;  // 190 thread blocks at order 1500
 __global__ void k_norm_partials(const Block* __restrict__ blocks, const int* __restrict__ chunk_off,
-                                const float* __restrict__ Wh, const float* __restrict__ Wl, double* partial) {
+                                const float* __restrict__ W, double* partial) {
     const int k = blockIdx.y;
     const Block B = blocks[k];
     const int nchunk = chunk_off[k + 1] - chunk_off[k];
@@ -330,7 +364,7 @@ __global__ void k_norm_partials(const Block* __restrict__ blocks, const int* __r
     const long long ne = (long long)min((long long)kNormChunkRows, B.S - r0) * B.S;
     double acc = 0.0;
     for (long long e = threadIdx.x; e < ne; e += blockDim.x) {
-        const double w = (double)Wh[e0 + e] + (double)Wl[e0 + e];
+        const double w = (double)W[e0 + e];
         acc += w * w;
     }
     __shared__ double sh[32];
@@ -345,10 +379,10 @@ __global__ void k_norm_partials(const Block* __restrict__ blocks, const int* __r
     }
 }
 
-// X_0 = W / ||W||_F as (hi, lo); scale[k] = ||W||_F (grid.y = block).
+// X_0 = W / ||W||_F as (hi, lo); scale[k] = ||W||_F as rounded for that (grid.y = block).
 __global__ void k_scale_start(const Block* __restrict__ blocks, const int* __restrict__ chunk_off,
-                              const double* __restrict__ partial, const float* __restrict__ Wh,
-                              const float* __restrict__ Wl, float* Xh, float* Xl, double* scale) {
+                              const double* __restrict__ partial, const float* __restrict__ W, __half* Xh, __half* Xl,
+                              double* scale) {
     const int k = blockIdx.y;
     const Block B = blocks[k];
     // one warp adds the partial sums for its block (every thread did: 93 us of
@@ -361,18 +395,27 @@ __global__ void k_scale_start(const Block* __restrict__ blocks, const int* __res
         for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
         if (threadIdx.x == 0) {
             const double nrm = sqrt(s2);
-            if (blockIdx.x == 0) scale[k] = nrm;
             s_inv = nrm > 0.0 ? (float)(1.0 / nrm) : 0.f;
+            if (blockIdx.x == 0) scale[k] = s_inv > 0.f ? 1.0 / (double)s_inv : 0.0;  // what X_0 was divided by
         }
     }
     __syncthreads();
     const float inv = s_inv;
-    const long long ne = (long long)B.S * B.S;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < ne; e += (long long)gridDim.x * blockDim.x) {
-        const float x = (Wh[B.off + e] + Wl[B.off + e]) * inv;
-        const float h = tf32_round(x);
-        Xh[B.off + e] = h;
-        Xl[B.off + e] = x - h;
+    const long long nq = (long long)B.S * B.S / 4;  // S is a multiple of 128
+    const float4* W4 = reinterpret_cast<const float4*>(W + B.off);
+    uint2* Xh4 = reinterpret_cast<uint2*>(Xh + B.off);
+    uint2* Xl4 = reinterpret_cast<uint2*>(Xl + B.off);
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < nq; e += (long long)gridDim.x * blockDim.x) {
+        const float4 w = W4[e];
+        const float x[4] = {w.x * inv, w.y * inv, w.z * inv, w.w * inv};
+        __half h[4], l[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) pair_split(x[i], h[i], l[i]);
+        auto pack2 = [](const __half* p) {
+            return (uint32_t)__half_as_ushort(p[0]) | ((uint32_t)__half_as_ushort(p[1]) << 16);
+        };
+        Xh4[e] = make_uint2(pack2(h), pack2(h + 2));
+        Xl4[e] = make_uint2(pack2(l), pack2(l + 2));
     }
 }
 
@@ -408,12 +451,12 @@ bool get_encode() {
     return true;
 }
 
-bool encode_map(CUtensorMap* m, const float* base, int S, int rows) {
+bool encode_map(CUtensorMap* m, const __half* base, int S, int rows) {
     const cuuint64_t dims[2] = {(cuuint64_t)S, (cuuint64_t)S};
-    const cuuint64_t strides[1] = {(cuuint64_t)S * 4};
+    const cuuint64_t strides[1] = {(cuuint64_t)S * 2};
     const cuuint32_t box[2] = {(cuuint32_t)kChunk, (cuuint32_t)rows};
     const cuuint32_t estr[2] = {1, 1};
-    return g_encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box, estr,
+    return g_encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half*>(base), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -468,9 +511,11 @@ NsLayout ns_layout(const std::vector<int>& sizes) {
     L.o_list = o; o = up256(o + sizeof(int) * std::max(1, L.nb));
     L.o_upd = o; o = up256(o + sizeof(int) * (L.nb + 1));
     L.o_updpart = o; o = up256(o + sizeof(double) * 8 * std::max(1, L.upd_off.back()));
+    L.o_w = o; o = up256(o + (size_t)off * sizeof(float));
+    // off is a multiple of 128 x 128: a pair's two buffers are adjacent
     for (int b = 0; b < 2 * NBUF; ++b) {
         L.o_buf[b] = o;
-        o = up256(o + (size_t)off * sizeof(float));
+        o = up256(o + (size_t)off * sizeof(__half));
     }
     L.bytes = o;
     return L;
@@ -482,12 +527,12 @@ NsLayout ns_layout(const std::vector<int>& sizes) {
 bool ns_tables(const NsLayout& L, unsigned char* base, const std::vector<long long>& poff,
                const std::vector<int>& list, std::vector<unsigned char>& img) {
     if (!get_encode()) return false;
-    img.assign(L.o_buf[0], 0);
+    img.assign(L.o_w, 0);
     CUtensorMap* maps = reinterpret_cast<CUtensorMap*>(img.data() + L.o_maps);
     CUtensorMap* maps_b = reinterpret_cast<CUtensorMap*>(img.data() + L.o_maps_b);
     for (int buf = 0; buf < 2 * NBUF; ++buf)
         for (int k = 0; k < L.nb; ++k) {
-            const float* p = reinterpret_cast<const float*>(base + L.o_buf[buf]) + L.blocks[k].off;
+            const __half* p = reinterpret_cast<const __half*>(base + L.o_buf[buf]) + L.blocks[k].off;
             if (!encode_map(&maps[buf * L.nb + k], p, L.blocks[k].S, kTile)) return false;
             if (L.cols != kTile && !encode_map(&maps_b[buf * L.nb + k], p, L.blocks[k].S, L.cols)) return false;
         }
@@ -506,27 +551,32 @@ template <int N>
 cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t st) {
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_tf32x3_sym<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(N));
+        cudaError_t e = cudaFuncSetAttribute(k_f16x3_sym<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(N));
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    k_tf32x3_sym<N><<<g.ntiles, kGemmThreads, gemm_smem(N), st>>>(g);
+    k_f16x3_sym<N><<<g.ntiles, kGemmThreads, gemm_smem(N), st>>>(g);
     return cudaGetLastError();
 }
 
+// D = alpha A B + beta C on pairs; with d < 0 the last product, P = (W + |W|_F A B) / 2.
 cudaError_t gemm(const NsLayout& L, unsigned char* base, int a, int bsrc, int c, int d, float alpha, float beta,
-                 bool split, cudaStream_t st) {
+                 cudaStream_t st) {
     const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(base + L.o_maps);
     const CUtensorMap* maps_b = reinterpret_cast<const CUtensorMap*>(base + L.o_maps_b);
+    auto half_buf = [&](int i) { return reinterpret_cast<__half*>(base + L.o_buf[i]); };
     GemmArgs g;
     g.mapA_hi = maps + (2 * a) * L.nb;
     g.mapA_lo = maps + (2 * a + 1) * L.nb;
     g.mapB_hi = maps_b + (2 * bsrc) * L.nb;
     g.mapB_lo = maps_b + (2 * bsrc + 1) * L.nb;
-    g.C_hi = c >= 0 ? reinterpret_cast<const float*>(base + L.o_buf[2 * c]) : nullptr;
-    g.C_lo = c >= 0 ? reinterpret_cast<const float*>(base + L.o_buf[2 * c + 1]) : nullptr;
-    g.D_hi = reinterpret_cast<float*>(base + L.o_buf[2 * d]);
-    g.D_lo = split ? reinterpret_cast<float*>(base + L.o_buf[2 * d + 1]) : nullptr;
+    g.C_hi = c >= 0 ? half_buf(2 * c) : nullptr;
+    g.C_lo = c >= 0 ? half_buf(2 * c + 1) : nullptr;
+    g.D_hi = d >= 0 ? half_buf(2 * d) : nullptr;
+    g.D_lo = d >= 0 ? half_buf(2 * d + 1) : nullptr;
+    g.W = reinterpret_cast<const float*>(base + L.o_w);
+    g.P = d >= 0 ? nullptr : reinterpret_cast<float*>(base + L.o_p());
+    g.scale = reinterpret_cast<const double*>(base + L.o_scale);
     g.blocks = reinterpret_cast<const Block*>(base + L.o_blocks);
     g.tiles = reinterpret_cast<const Tile*>(base + L.o_tiles);
     g.ntiles = (int)L.tiles.size();
@@ -538,39 +588,42 @@ cudaError_t gemm(const NsLayout& L, unsigned char* base, int a, int bsrc, int c,
 
 }  // namespace
 
-// The sign iteration and P = (W + W X) / 2 on buffers already holding W
-// (hi, lo) and X_0 (BUF_XA); P goes to BUF_X2 hi.
+// The sign iteration and P = (W + W X) / 2 on buffers already holding W and
+// X_0.
 cudaError_t ns_iterate(const NsLayout& L, unsigned char* base, cudaStream_t st) {
     cudaError_t e = cudaSuccess;
-    int x = BUF_XA, xn = BUF_XB;
+    int x = BUF_X0, xn = BUF_XA;
+    auto next = [&] {
+        x = xn;
+        xn = x == BUF_XA ? BUF_XB : BUF_XA;
+    };
     for (int i = 0; i < kPhase1 && e == cudaSuccess; ++i) {  // X <- a X + b X^3 + c X^5
-        e = gemm(L, base, x, x, -1, BUF_X2, 1.f, 0.f, true, st);                          // X2 = X X
-        if (e == cudaSuccess) e = gemm(L, base, BUF_X2, BUF_X2, BUF_X2, BUF_B, kPc, kPb, true, st);  // c X2 X2 + b X2
-        if (e == cudaSuccess) e = gemm(L, base, x, BUF_B, x, xn, 1.f, kPa, true, st);     // X B + a X
-        std::swap(x, xn);
+        e = gemm(L, base, x, x, -1, BUF_X2, 1.f, 0.f, st);                          // X2 = X X
+        if (e == cudaSuccess) e = gemm(L, base, BUF_X2, BUF_X2, BUF_X2, BUF_B, kPc, kPb, st);  // c X2 X2 + b X2
+        if (e == cudaSuccess) e = gemm(L, base, x, BUF_B, x, xn, 1.f, kPa, st);     // X B + a X
+        next();
     }
     for (int i = 0; i < kPhase2 && e == cudaSuccess; ++i) {  // X <- 1.5 X - 0.5 X^3
-        e = gemm(L, base, x, x, -1, BUF_X2, 1.f, 0.f, true, st);
-        if (e == cudaSuccess) e = gemm(L, base, x, BUF_X2, x, xn, -0.5f, 1.5f, true, st);
-        std::swap(x, xn);
+        e = gemm(L, base, x, x, -1, BUF_X2, 1.f, 0.f, st);
+        if (e == cudaSuccess) e = gemm(L, base, x, BUF_X2, x, xn, -0.5f, 1.5f, st);
+        next();
     }
-    if (e == cudaSuccess) e = gemm(L, base, BUF_W, x, BUF_W, BUF_X2, 0.5f, 0.5f, false, st);  // P
+    if (e == cudaSuccess) e = gemm(L, base, BUF_X0, x, -1, -1, 0.f, 0.f, st);  // P
     return e;
 }
 
 cudaError_t ns_scale_and_iterate(const NsLayout& L, unsigned char* base, cudaStream_t st) {
     const Block* blocks = reinterpret_cast<const Block*>(base + L.o_blocks);
     const int* chunk = reinterpret_cast<const int*>(base + L.o_chunk);
-    const float* Wh = reinterpret_cast<const float*>(base + L.o_buf[2 * BUF_W]);
-    const float* Wl = reinterpret_cast<const float*>(base + L.o_buf[2 * BUF_W + 1]);
-    float* Xh = reinterpret_cast<float*>(base + L.o_buf[2 * BUF_XA]);
-    float* Xl = reinterpret_cast<float*>(base + L.o_buf[2 * BUF_XA + 1]);
+    const float* W = reinterpret_cast<const float*>(base + L.o_w);
+    __half* Xh = reinterpret_cast<__half*>(base + L.o_buf[2 * BUF_X0]);
+    __half* Xl = reinterpret_cast<__half*>(base + L.o_buf[2 * BUF_X0 + 1]);
     const int gx = std::min(1024, std::max(1, (int)(((long long)L.max_S * L.max_S / 2 + 255) / 256)));
     const int maxchunk = (L.max_S + kNormChunkRows - 1) / kNormChunkRows;
-    k_norm_partials<<<dim3(maxchunk, L.nb), 256, 0, st>>>(blocks, chunk, Wh, Wl,
+    k_norm_partials<<<dim3(maxchunk, L.nb), 256, 0, st>>>(blocks, chunk, W,
                                                          reinterpret_cast<double*>(base + L.o_partial));
     k_scale_start<<<dim3(gx, L.nb), 256, 0, st>>>(blocks, chunk, reinterpret_cast<const double*>(base + L.o_partial),
-                                                  Wh, Wl, Xh, Xl, reinterpret_cast<double*>(base + L.o_scale));
+                                                  W, Xh, Xl, reinterpret_cast<double*>(base + L.o_scale));
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = ns_iterate(L, base, st);
     return e;
@@ -579,12 +632,11 @@ cudaError_t ns_scale_and_iterate(const NsLayout& L, unsigned char* base, cudaStr
 cudaError_t ns_from_packed(const NsLayout& L, unsigned char* base, const float* Wp, cudaStream_t st) {
     const Block* blocks = reinterpret_cast<const Block*>(base + L.o_blocks);
     const long long* poff = reinterpret_cast<const long long*>(base + L.o_poff);
-    float* Wh = reinterpret_cast<float*>(base + L.o_buf[2 * BUF_W]);
-    float* Wl = reinterpret_cast<float*>(base + L.o_buf[2 * BUF_W + 1]);
-    cudaError_t e = cudaMemsetAsync(base + L.o_buf[2 * BUF_W], 0, 2 * (size_t)L.elems * sizeof(float), st);
+    float* W = reinterpret_cast<float*>(base + L.o_w);
+    cudaError_t e = cudaMemsetAsync(W, 0, (size_t)L.elems * sizeof(float), st);
     if (e != cudaSuccess) return e;
     const int gx = std::min(1024, std::max(1, (int)(((long long)L.max_S * L.max_S / 2 + 255) / 256)));
-    k_dense_from_packed<<<dim3(gx, L.nb), 256, 0, st>>>(blocks, poff, Wp, Wh, Wl);
+    k_dense_from_packed<<<dim3(gx, L.nb), 256, 0, st>>>(blocks, poff, Wp, W);
     return cudaGetLastError();
 }
 
@@ -592,7 +644,7 @@ cudaError_t ns_to_packed(const NsLayout& L, unsigned char* base, float* Xp, cuda
     const int gx = std::min(1024, std::max(1, (int)(((long long)L.max_S * L.max_S / 2 + 255) / 256)));
     k_packed_from_dense<<<dim3(gx, L.nb), 256, 0, st>>>(reinterpret_cast<const Block*>(base + L.o_blocks),
                                                         reinterpret_cast<const long long*>(base + L.o_poff),
-                                                        reinterpret_cast<const float*>(base + L.o_buf[2 * BUF_X2]),
+                                                        reinterpret_cast<const float*>(base + L.o_p()),
                                                         Xp);
     return cudaGetLastError();
 }

@@ -19,15 +19,28 @@
 // Every step is a product of two symmetric matrices that commute (powers of
 // W), so only the lower tiles of each product are computed and mirrored.
 //
-// Products run in float32 accuracy as three TF32 products (Ootomo and
-// Yokota, 2022): x = x_hi + x_lo with x_hi = tf32(x) (round to nearest) and
-// x_lo = x - x_hi; A B ~ A_hi B_hi + A_hi B_lo + A_lo B_hi, all accumulated in
-// float32 in tensor memory.  Every matrix of the iteration is stored as its
-// (hi, lo) pair, row-major, block k at a 256-byte aligned offset with row
-// pitch S_k = ceil(s_k / 128) * 128 floats (zero padding stays zero under odd
-// polynomials).
+// Products run in float32 accuracy as three float16 products (Ootomo and
+// Yokota, 2022): 2^12 x = x_hi + 2^-11 x_lo with x_hi = half(2^12 x) and x_lo =
+// half(2^11 (2^12 x - x_hi)), 22 bits and a sign; A B ~ A_hi B_hi + 2^-11 (A_hi
+// B_lo + A_lo B_hi), both sums accumulated in float32, each in its own columns of
+// tensor memory.  Every operand is a power of X_0 or a polynomial of it with
+// eigenvalues below 4, so 2^12 x stays below the float16 range, and an entry
+// keeps its 22 bits down to 1.5e-8 (an absolute 2^-37 below that).
+// Every such matrix is stored as its (hi, lo) pair, row-major, block k at a
+// 256-byte aligned offset with row pitch S_k = ceil(s_k / 128) * 128 (zero
+// padding stays zero under odd polynomials); W itself and P stay float32.
+// Before, the pairs were TF32 ones (float32 words): twice the bytes, of which
+// an SM takes in about 45 a clock, and half the tensor rate.  TF32 products
+// also cut x_lo to 11 bits instead of rounding it: replayed in float64 over
+// orders 150..900 the rounding of the operands alone puts P off by 2.7e-7 (rms,
+// N(0, 1) entries) with TF32 pairs and 2.2e-7 with float16 pairs; measured, with
+// the float32 accumulation in tensor memory (half as many steps as for TF32, and
+// the small terms by themselves), 2.3e-5 -> 1.6e-5 relative at order 1500, 1.5e-5 ->
+// 1.0e-5 at 900 and 4.9e-6 -> 3.0e-6 at 300.  Blocks of order 129..1500 (four of
+// them): 3.93 -> 3.27 ms a projection.
 #pragma once
 
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -38,14 +51,14 @@ constexpr int kTile = 128;         // rows of an output tile, one CTA each
 // 128 x 128 tiles that the narrower ones still fit one wave of the 152 SMs.  An
 // SM takes in about 45 B a clock from L2, which is what a K step costs (64 KB
 // of operands at 128 columns, 48 KB at 64, 40 KB at 32, where its MMAs take
-// 840, 420 and 210 clocks), so the narrow tiles are less efficient but finish
+// about 840, 420 and 210 clocks), so the narrow tiles are less efficient but finish
 // sooner while SMs would stand idle otherwise.  Every entry is the same sum in
 // the same order at each width.
 constexpr int kMaxCols = 128;
-constexpr int kChunk = 32;         // K floats per stage: one 128-byte swizzle row
+constexpr int kChunk = 64;         // K halves per stage: one 128-byte swizzle row
 constexpr int kStages = 3;
-constexpr int kTileBytes = kTile * kChunk * 4;       // 16 KB per operand tile of 128 rows
-__host__ __device__ constexpr int stage_bytes(int cols) { return 2 * kTileBytes + 2 * cols * kChunk * 4; }  // A_hi, A_lo, B_hi, B_lo
+constexpr int kTileBytes = kTile * kChunk * 2;       // 16 KB per operand tile of 128 rows
+__host__ __device__ constexpr int stage_bytes(int cols) { return 2 * kTileBytes + 2 * cols * kChunk * 2; }  // A_hi, A_lo, B_hi, B_lo
 constexpr int gemm_smem(int cols) { return kStages * stage_bytes(cols) + 1024 + 256; }
 constexpr int kGemmThreads = 256;  // producer, MMA issuer; all warps read the accumulator
 
@@ -60,16 +73,30 @@ struct Tile { int blk, ti, tj, pad; };
 // Dense layout of one block in every buffer: float offset and padded order.
 struct Block { long long off; int S, s; };
 
-// The (hi, lo) buffers of the iteration.
-enum { BUF_W = 0, BUF_XA = 1, BUF_XB = 2, BUF_X2 = 3, BUF_B = 4, NBUF = 5 };
+// The (hi, lo) buffers of the iteration.  X_0 keeps its own: the last product
+// takes it in the place of W.  P (float32) overlays the pair of X^2.
+enum { BUF_X0 = 0, BUF_XA = 1, BUF_XB = 2, BUF_X2 = 3, BUF_B = 4, NBUF = 5 };
 
-// Epilogue of one product D = alpha A B + beta C over the lower tiles, C and
-// D given as (hi, lo) pairs; D_lo == nullptr writes D in plain float32 to D_hi.
+// 2^12 x as a (hi, lo) pair of float16.
+constexpr float kPairScale = 4096.f, kLoScale = 2048.f;
+__device__ __forceinline__ void pair_split(float x, __half& hi, __half& lo) {
+    const float y = x * kPairScale;
+    hi = __float2half_rn(y);
+    lo = __float2half_rn((y - __half2float(hi)) * kLoScale);
+}
+__device__ __forceinline__ float pair_value(__half hi, __half lo) {
+    return (__half2float(hi) + __half2float(lo) * (1.f / kLoScale)) * (1.f / kPairScale);
+}
+
+// Epilogue of one product over the lower tiles: D = alpha A B + beta C, all
+// (hi, lo) pairs; or, with P set, P = (W + |W|_F A B) / 2 in float32.
 struct GemmArgs {
     const void* mapA_hi; const void* mapA_lo;   // tensor maps, one per block (CUtensorMap arrays)
     const void* mapB_hi; const void* mapB_lo;
-    const float* C_hi; const float* C_lo;
-    float* D_hi; float* D_lo;
+    const __half* C_hi; const __half* C_lo;
+    __half* D_hi; __half* D_lo;
+    const float* W; float* P;
+    const double* scale;                        // |W|_F per block
     const Block* blocks;
     const Tile* tiles;
     int ntiles;

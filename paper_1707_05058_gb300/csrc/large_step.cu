@@ -3,7 +3,7 @@
 // (jacobi_cta.cuh), with the eigensolve replaced by the tensor-core sign
 // iteration of large.cu on dense copies of the blocks.
 //   gather   W_k of the form (Eq. XkUpdate / zkUpdate / HsdeStep2 inputs) into
-//            the dense (hi, lo) buffer, both triangles;
+//            the dense float32 buffer, both triangles;
 //   ns_scale_and_iterate   P_k = (W_k + W_k sign(W_k)) / 2;
 //   update   the clique state of the form from P_k and per-chunk partial sums
 //            of the stopping tests;
@@ -20,20 +20,13 @@ namespace {
 using cdsdp_dev::Dev;
 using cdsdp_dev::FinishArgs;
 
-__device__ __forceinline__ float tf32_rn(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
-}
-
 struct Step {
     const Block* blocks;
     const int* list;     // clique of each block
     const int* upd;      // chunk offsets per block
     double* part;        // [chunks * 8] chunk partial sums
-    float* Wh;
-    float* Wl;
-    const float* P;      // dense P (BUF_X2 hi)
+    float* W;            // dense W
+    const float* P;      // dense P
 };
 
 template <int FORM>
@@ -65,11 +58,8 @@ __global__ void __launch_bounds__(256) k_large_gather(Dev d, Step t) {
             w = s12 - gamma * 0.5 * d.zhx[ent] - double(c1[off + f]);
         }
         const float wf = float(w);
-        const float h = tf32_rn(wf), l = wf - h;
-        t.Wh[B.off + (long long)a * B.S + b] = h;
-        t.Wl[B.off + (long long)a * B.S + b] = l;
-        t.Wh[B.off + (long long)b * B.S + a] = h;
-        t.Wl[B.off + (long long)b * B.S + a] = l;
+        t.W[B.off + (long long)a * B.S + b] = wf;
+        t.W[B.off + (long long)b * B.S + a] = wf;
     }
 }
 
@@ -168,9 +158,8 @@ cudaError_t run(const Dev& d, const NsLayout& L, unsigned char* base, int row_of
     t.list = reinterpret_cast<const int*>(base + L.o_list);
     t.upd = reinterpret_cast<const int*>(base + L.o_upd);
     t.part = reinterpret_cast<double*>(base + L.o_updpart);
-    t.Wh = reinterpret_cast<float*>(base + L.o_buf[2 * BUF_W]);
-    t.Wl = reinterpret_cast<float*>(base + L.o_buf[2 * BUF_W + 1]);
-    t.P = reinterpret_cast<const float*>(base + L.o_buf[2 * BUF_X2]);
+    t.W = reinterpret_cast<float*>(base + L.o_w);
+    t.P = reinterpret_cast<const float*>(base + L.o_p());
     const dim3 grid(std::max(1, L.max_upd), L.nb);
     k_large_gather<FORM><<<grid, 256, 0, st>>>(d, t);
     cudaError_t e = cudaGetLastError();

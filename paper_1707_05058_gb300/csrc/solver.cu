@@ -1148,8 +1148,7 @@ int cdsdp_bind(cdsdp* h, void* d_workspace, size_t bytes, int max_iter, void* st
             return CDSDP_ERR_CUDA;
         }
         CK(cudaMemcpyAsync(base, img.data(), img.size(), cudaMemcpyHostToDevice, st));
-        CK(cudaMemsetAsync(base + h->ns.o_buf[2 * cdsdp_large::BUF_W], 0,
-                           2 * (size_t)h->ns.elems * sizeof(float), st));
+        CK(cudaMemsetAsync(base + h->ns.o_w, 0, (size_t)h->ns.elems * sizeof(float), st));
         CK(cudaStreamSynchronize(st));
     }
     return CDSDP_SOLVED;
