@@ -5,15 +5,20 @@
 // Product kernel (one CTA of 256 threads per output tile of 128 rows and 128,
 // 64 or 32 columns):
 //  * thread 0 of warp 0 streams 64-half wide tiles of A_hi, A_lo, B_hi, B_lo
-//    into a 3-stage shared-memory ring with TMA (cp.async.bulk.tensor, 128-byte
-//    swizzle), one mbarrier per stage with the transaction byte count;
+//    into a shared-memory ring of 3 to 5 stages with TMA (cp.async.bulk.tensor, 128-byte
+//    swizzle), one mbarrier per stage with the transaction byte count, and after
+//    them the tile of C as one more stage;
 //  * thread 0 of warp 1 issues tcgen05.mma kind::f16 (M = 128, K = 16):
 //    three products per K step into two float32 accumulators in tensor memory
 //    (hi hi; hi lo + lo hi), and frees a stage with tcgen05.commit on that stage's "empty" mbarrier;
 //  * the warps read the accumulator back (tcgen05.ld 32x32b, one row per
 //    thread, the columns split between the two groups of four warps), apply
-//    D = alpha acc + beta C, split D into its (hi, lo) pair and store the tile
-//    and its mirror (the products are symmetric).
+//    D = alpha acc + beta C, split D into its (hi, lo) pair and lay the tile and
+//    its mirror (the products are symmetric) out in the free stages, from which
+//    they go to global memory in whole lines.  Stored from the accumulator's
+//    layout instead (16 bytes a lane and row, 2 bytes a lane and column, and C
+//    read likewise) the epilogue took 26 of 48 us a product at order 1500, 15 of
+//    32 us at order 903 and 11 of 22 us at order 300.
 // Every wait is bounded (about a second of clock cycles): on a timeout the
 // kernel records an error code, lets its in-flight copies land (bounded
 // again), frees its tensor memory and returns; the host reports
@@ -121,6 +126,10 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* m) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
+}
+
 // 32 columns of this thread's row of A B, from the two accumulators N columns
 // apart (of operands scaled by kPairScale each).
 template <int N>
@@ -143,11 +152,11 @@ __device__ __forceinline__ uint4 pack8(const __half* h) {
 
 template <int N>
 __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
-    constexpr int kStageBytes = stage_bytes(N), kColBytes = N * kChunk * 2;
+    constexpr int kStages = stages(N), kStageBytes = stage_bytes(N), kColBytes = N * kChunk * 2;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                            ~static_cast<uintptr_t>(1023));
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);  // full[3], empty[3], done
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);  // full[kStages], empty[kStages], done
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     int* issued_slot = reinterpret_cast<int*>(tmem_slot + 2);
@@ -160,6 +169,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
     const CUtensorMap* mAl = reinterpret_cast<const CUtensorMap*>(g.mapA_lo) + t.blk;
     const CUtensorMap* mBh = reinterpret_cast<const CUtensorMap*>(g.mapB_hi) + t.blk;
     const CUtensorMap* mBl = reinterpret_cast<const CUtensorMap*>(g.mapB_lo) + t.blk;
+    const bool has_c = g.mapC_hi != nullptr;
+    const CUtensorMap* mCh = reinterpret_cast<const CUtensorMap*>(g.mapC_hi) + (has_c ? t.blk : 0);
+    const CUtensorMap* mCl = reinterpret_cast<const CUtensorMap*>(g.mapC_lo) + (has_c ? t.blk : 0);
     const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + kStages), done = smem_u32(bars + 2 * kStages);
 
     if (tid == 0) {
@@ -172,6 +184,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
         *issued_slot = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (tid == 32) {  // the descriptors come from global memory, once per SM and launch
+        prefetch_map(mAh);
+        prefetch_map(mAl);
+        prefetch_map(mBh);
+        prefetch_map(mBl);
+        if (has_c) {
+            prefetch_map(mCh);
+            prefetch_map(mCl);
+        }
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -186,7 +208,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
 
     if (warp == 0 && lane == 0) {  // TMA producer
         int issued = 0;
-        for (int kc = 0; kc < nk; ++kc) {
+        for (int kc = 0; kc < nk + (has_c ? 1 : 0); ++kc) {
             const int s = kc % kStages;
             if (kc >= kStages && !mbar_wait(empty0 + 8 * s, ((kc / kStages) - 1) & 1)) {
                 *abort_flag = 1;
@@ -195,6 +217,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
             }
             if (*abort_flag) break;
             const uint32_t base = smem_u32(smem + s * kStageBytes);
+            if (kc == nk) {  // C by its symmetric entries (tj, ti): two boxes of 64 columns each, hi then lo
+                mbar_expect_tx(full0 + 8 * s, 4 * kColBytes);
+                for (int q = 0; q < 2; ++q) {
+                    tma_load_2d(base + q * kColBytes, mCh, t.ti * kTile + q * kChunk, t.tj * N, full0 + 8 * s);
+                    tma_load_2d(base + (2 + q) * kColBytes, mCl, t.ti * kTile + q * kChunk, t.tj * N, full0 + 8 * s);
+                }
+                ++issued;
+                break;
+            }
             mbar_expect_tx(full0 + 8 * s, kStageBytes);
             const int x = kc * kChunk;
             tma_load_2d(base, mAh, x, t.ti * kTile, full0 + 8 * s);
@@ -230,11 +261,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
     __syncwarp();
 
     // epilogue: thread (warp w, lane l) owns row 32 (w mod 4) + l of the tile
+    const int c_slot = nk % kStages;
     bool ok = mbar_wait(done, 0);
+    if (ok && has_c && !*abort_flag) ok = mbar_wait(full0 + 8 * c_slot, (nk / kStages) & 1);
     if (!ok) atomicExch(g.err, 3);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    __syncwarp();
-    if (ok && !*abort_flag) {
+    if (__syncthreads_and(ok && !*abort_flag)) {
         // Every stored matrix is kept exactly symmetric: an off-diagonal tile is
         // stored with its mirror, a diagonal tile only from its lower triangle
         // (mirrored).  The products are symmetric only up to rounding, and the
@@ -243,10 +275,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
         const int S = B.S;
         const int wr = warp & 3, half = warp >> 2;
         const int r = 32 * wr + lane;
-        const bool diag = t.tj * N >= t.ti * kTile;  // the tile reaches the diagonal
-        const long long gr = (long long)t.ti * kTile + r;
+        // A tile that reaches the diagonal holds columns c0 .. c0 + N - 1 of its
+        // 128 x 128 diagonal block: rows above c0 belong to the mirrors of other
+        // tiles, rows c0 .. c0 + N - 1 are a symmetric square, the rest lies below.
+        const int c0 = t.tj * N - t.ti * kTile;
+        const bool diag = c0 >= 0;
         const uint32_t row = tmem + ((uint32_t)(32 * wr) << 16);
         if (g.P) {  // P = (W + |W|_F A B) / 2; |W|_F in two floats, so that its rounding does not scale W sign(W)
+            const long long gr = (long long)t.ti * kTile + r;
             const double nrm = g.scale[t.blk];
             const float up = nrm > 1e30 ? 16777216.f : 1.f;  // |W|_F itself may pass the float32 range
             const float nh = (float)(nrm / up), nl = (float)(nrm / up - (double)nh);
@@ -271,50 +307,77 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
                 }
             }
         } else {
-            const __half* Ch = g.C_hi ? g.C_hi + B.off : nullptr;
-            const __half* Cl = g.C_lo ? g.C_lo + B.off : nullptr;
-            __half* Dh = g.D_hi + B.off;
-            __half* Dl = g.D_lo + B.off;
+            // tile (rows of N halves, 16-byte units permuted within a row so that
+            // eight rows' units fall into different banks) and mirror (N rows of 128)
+            unsigned char* tile = smem + ((c_slot + 1) % kStages) * kStageBytes;
+            unsigned char* mirr = smem + ((c_slot + 2) % kStages) * kStageBytes;
+            constexpr int kOut = kTile * N * 2;  // bytes of one of hi, lo
+            auto perm = [](int rr) { return N >= 64 ? (rr & 7) : ((rr >> 1) & 3); };
+            auto tile_at = [&](int rr, int col) { return rr * (2 * N) + ((((col >> 3) ^ perm(rr)) << 4) | ((col & 7) << 1)); };
+            // C (gc, gr): row gc of box r / 64, its 16-byte units permuted by the TMA swizzle
+            const unsigned char* cbase = smem + c_slot * kStageBytes + (r >> 6) * kColBytes + ((r & 7) << 1);
+            const int cq = (r & 63) >> 3;
+            const int lc = r - c0;  // own column within the diagonal square
+            const bool square = diag && lc >= 0 && lc < N;
 #pragma unroll 1
             for (int cc = half; cc < N / 32; cc += 2) {
                 float v[32];
                 load_acc<N>(row + (uint32_t)(32 * cc), v);
-                const long long gc0 = (long long)t.tj * N + 32 * cc;
                 __half hi[32], lo[32];
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
-                    // C is symmetric: read its entry (gc, gr), consecutive over the warp's rows
                     float c = 0.f;
-                    if (Ch) c = pair_value(Ch[(gc0 + j) * S + gr], Cl[(gc0 + j) * S + gr]);
+                    if (has_c) {
+                        const unsigned char* pc = cbase + (32 * cc + j) * 128 + ((cq ^ (j & 7)) << 4);
+                        c = pair_value(*reinterpret_cast<const __half*>(pc),
+                                       *reinterpret_cast<const __half*>(pc + 2 * kColBytes));
+                    }
                     pair_split(g.alpha * v[j] + g.beta * c, hi[j], lo[j]);
                 }
-                if (!diag) {
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) {  // mirror (gc, gr): coalesced over the warp
-                        const long long mi = (gc0 + j) * S + gr;
-                        Dh[mi] = hi[j];
-                        Dl[mi] = lo[j];
-                    }
-                    uint4* dh4 = reinterpret_cast<uint4*>(Dh + gr * S + gc0);
-                    uint4* dl4 = reinterpret_cast<uint4*>(Dl + gr * S + gc0);
+                if (!square) {
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
-                        dh4[q] = pack8(hi + 8 * q);
-                        dl4[q] = pack8(lo + 8 * q);
+                        const int at = tile_at(r, 32 * cc + 8 * q);
+                        *reinterpret_cast<uint4*>(tile + at) = pack8(hi + 8 * q);
+                        *reinterpret_cast<uint4*>(tile + kOut + at) = pack8(lo + 8 * q);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) {
+                        const int at = (32 * cc + j) * (2 * kTile) + 2 * r;
+                        *reinterpret_cast<__half*>(mirr + at) = hi[j];
+                        *reinterpret_cast<__half*>(mirr + kOut + at) = lo[j];
                     }
                 } else {
 #pragma unroll
                     for (int j = 0; j < 32; ++j) {
-                        const long long gc = gc0 + j;
-                        if (gc > gr) continue;
-                        Dh[gr * S + gc] = hi[j];
-                        Dl[gr * S + gc] = lo[j];
-                        if (gc < gr) {
-                            Dh[gc * S + gr] = hi[j];
-                            Dl[gc * S + gr] = lo[j];
-                        }
+                        const int col = 32 * cc + j;
+                        if (col > lc) continue;
+                        const int at = tile_at(r, col), am = tile_at(c0 + col, lc);
+                        *reinterpret_cast<__half*>(tile + at) = hi[j];
+                        *reinterpret_cast<__half*>(tile + kOut + at) = lo[j];
+                        *reinterpret_cast<__half*>(tile + am) = hi[j];
+                        *reinterpret_cast<__half*>(tile + kOut + am) = lo[j];
                     }
                 }
+            }
+            __syncthreads();
+            __half* Dh = g.D_hi + B.off;
+            __half* Dl = g.D_lo + B.off;
+            const int r0 = diag ? c0 : 0;
+            for (int i = tid; i < (kTile - r0) * (N / 8); i += kGemmThreads) {
+                const int rr = r0 + i / (N / 8), q = i % (N / 8);
+                const int at = tile_at(rr, 8 * q);
+                const long long to = ((long long)t.ti * kTile + rr) * S + (long long)t.tj * N + 8 * q;
+                *reinterpret_cast<uint4*>(Dh + to) = *reinterpret_cast<const uint4*>(tile + at);
+                *reinterpret_cast<uint4*>(Dl + to) = *reinterpret_cast<const uint4*>(tile + kOut + at);
+            }
+            const int m0 = diag ? c0 + N : 0, nv = (kTile - m0) / 8;
+            for (int i = tid; i < N * nv; i += kGemmThreads) {
+                const int gc = i / nv, q = m0 / 8 + i - gc * nv;
+                const int at = gc * (2 * kTile) + 16 * q;
+                const long long to = ((long long)t.tj * N + gc) * S + (long long)t.ti * kTile + 8 * q;
+                *reinterpret_cast<uint4*>(Dh + to) = *reinterpret_cast<const uint4*>(mirr + at);
+                *reinterpret_cast<uint4*>(Dl + to) = *reinterpret_cast<const uint4*>(mirr + kOut + at);
             }
         }
     }
@@ -322,7 +385,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
     __syncthreads();
     // after an abort, let the copies already issued land before the CTA exits
     if (*abort_flag && warp == 0 && lane == 0) {
-        const int issued = *issued_slot;
+        const int issued = *issued_slot;  // the chunks, then C
         for (int kc = max(0, issued - kStages); kc < issued; ++kc)
             (void)mbar_wait(full0 + 8 * (kc % kStages), (kc / kStages) & 1);
     }
@@ -570,8 +633,8 @@ cudaError_t gemm(const NsLayout& L, unsigned char* base, int a, int bsrc, int c,
     g.mapA_lo = maps + (2 * a + 1) * L.nb;
     g.mapB_hi = maps_b + (2 * bsrc) * L.nb;
     g.mapB_lo = maps_b + (2 * bsrc + 1) * L.nb;
-    g.C_hi = c >= 0 ? half_buf(2 * c) : nullptr;
-    g.C_lo = c >= 0 ? half_buf(2 * c + 1) : nullptr;
+    g.mapC_hi = c >= 0 ? maps_b + (2 * c) * L.nb : nullptr;
+    g.mapC_lo = c >= 0 ? maps_b + (2 * c + 1) * L.nb : nullptr;
     g.D_hi = d >= 0 ? half_buf(2 * d) : nullptr;
     g.D_lo = d >= 0 ? half_buf(2 * d + 1) : nullptr;
     g.W = reinterpret_cast<const float*>(base + L.o_w);

@@ -56,10 +56,11 @@ constexpr int kTile = 128;         // rows of an output tile, one CTA each
 // the same order at each width.
 constexpr int kMaxCols = 128;
 constexpr int kChunk = 64;         // K halves per stage: one 128-byte swizzle row
-constexpr int kStages = 3;
+// Stages of the operand ring: about 192 KB in flight at every width.
+__host__ __device__ constexpr int stages(int cols) { return cols == 128 ? 3 : (cols == 64 ? 4 : 5); }
 constexpr int kTileBytes = kTile * kChunk * 2;       // 16 KB per operand tile of 128 rows
 __host__ __device__ constexpr int stage_bytes(int cols) { return 2 * kTileBytes + 2 * cols * kChunk * 2; }  // A_hi, A_lo, B_hi, B_lo
-constexpr int gemm_smem(int cols) { return kStages * stage_bytes(cols) + 1024 + 256; }
+constexpr int gemm_smem(int cols) { return stages(cols) * stage_bytes(cols) + 1024 + 256; }
 constexpr int kGemmThreads = 256;  // producer, MMA issuer; all warps read the accumulator
 
 // Phase-1 polynomial and the iteration counts.
@@ -93,7 +94,7 @@ __device__ __forceinline__ float pair_value(__half hi, __half lo) {
 struct GemmArgs {
     const void* mapA_hi; const void* mapA_lo;   // tensor maps, one per block (CUtensorMap arrays)
     const void* mapB_hi; const void* mapB_lo;
-    const __half* C_hi; const __half* C_lo;
+    const void* mapC_hi; const void* mapC_lo;   // C's (boxes as B's); nullptr without C
     __half* D_hi; __half* D_lo;
     const float* W; float* P;
     const double* scale;                        // |W|_F per block
