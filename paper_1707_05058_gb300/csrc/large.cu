@@ -205,6 +205,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
+    // Launched while the previous product still ran (launch_gemm): let the next
+    // one be launched, and wait for the previous one's results.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 
     if (warp == 0 && lane == 0) {  // TMA producer
         int issued = 0;
@@ -618,8 +622,17 @@ cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t st) {
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    k_f16x3_sym<N><<<g.ntiles, kGemmThreads, gemm_smem(N), st>>>(g);
-    return cudaGetLastError();
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(g.ntiles);
+    cfg.blockDim = dim3(kGemmThreads);
+    cfg.dynamicSmemBytes = gemm_smem(N);
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_f16x3_sym<N>, g);
 }
 
 // D = alpha A B + beta C on pairs; with d < 0 the last product, P = (W + |W|_F A B) / 2.
