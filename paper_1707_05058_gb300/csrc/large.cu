@@ -30,6 +30,8 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <functional>
+#include <map>
 #include <mutex>
 #include <vector>
 
@@ -99,13 +101,12 @@ __host__ __device__ constexpr uint32_t idesc(int cols) {
     return (1u << 4) | ((uint32_t)(cols >> 3) << 17) | ((uint32_t)(kTile >> 4) << 24);
 }
 
-template <int N>
-__device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t a, uint64_t b, uint32_t accumulate) {
+__device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t a, uint64_t b, uint32_t desc, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem), "l"(a), "l"(b), "r"(idesc(N)), "r"(accumulate)
+        ::"r"(tmem), "l"(a), "l"(b), "r"(desc), "r"(accumulate)
         : "memory");
 }
 
@@ -130,13 +131,12 @@ __device__ __forceinline__ void prefetch_map(const CUtensorMap* m) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
 }
 
-// 32 columns of this thread's row of A B, from the two accumulators N columns
-// apart (of operands scaled by kPairScale each).
-template <int N>
-__device__ __forceinline__ void load_acc(uint32_t taddr, float (&v)[32]) {
+// 32 columns of this thread's row of A B, from the two accumulators (of operands
+// scaled by kPairScale each).
+__device__ __forceinline__ void load_acc(uint32_t taddr, int N, float (&v)[32]) {
     uint32_t a[32], b[32];
     tmem_ld32(taddr, a);
-    tmem_ld32(taddr + N, b);
+    tmem_ld32(taddr + (uint32_t)N, b);
     constexpr float s = 1.f / (kPairScale * kPairScale);
 #pragma unroll
     for (int j = 0; j < 32; ++j) v[j] = s * fmaf(1.f / kLoScale, __uint_as_float(b[j]), __uint_as_float(a[j]));
@@ -150,28 +150,28 @@ __device__ __forceinline__ uint4 pack8(const __half* h) {
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-template <int N>
-__global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
-    constexpr int kStages = stages(N), kStageBytes = stage_bytes(N), kColBytes = N * kChunk * 2;
+__global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(const __grid_constant__ GemmArgs g) {
+    const Tile t = g.tiles[blockIdx.x];
+    const int N = width_of(t.w);
+    const int kStages = stages(N), kStageBytes = stage_bytes(N), kColBytes = N * kChunk * 2;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                            ~static_cast<uintptr_t>(1023));
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);  // full[kStages], empty[kStages], done
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kRingBytes);  // full[kStages], empty[kStages], done
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     int* issued_slot = reinterpret_cast<int*>(tmem_slot + 2);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const Tile t = g.tiles[blockIdx.x];
     const Block B = g.blocks[t.blk];
     const int nk = B.S / kChunk;
-    const CUtensorMap* mAh = reinterpret_cast<const CUtensorMap*>(g.mapA_hi) + t.blk;
-    const CUtensorMap* mAl = reinterpret_cast<const CUtensorMap*>(g.mapA_lo) + t.blk;
-    const CUtensorMap* mBh = reinterpret_cast<const CUtensorMap*>(g.mapB_hi) + t.blk;
-    const CUtensorMap* mBl = reinterpret_cast<const CUtensorMap*>(g.mapB_lo) + t.blk;
-    const bool has_c = g.mapC_hi != nullptr;
-    const CUtensorMap* mCh = reinterpret_cast<const CUtensorMap*>(g.mapC_hi) + (has_c ? t.blk : 0);
-    const CUtensorMap* mCl = reinterpret_cast<const CUtensorMap*>(g.mapC_lo) + (has_c ? t.blk : 0);
+    const CUtensorMap* mAh = g.maps[0] + 2 * g.a * g.nb + t.blk;
+    const CUtensorMap* mAl = mAh + g.nb;
+    const CUtensorMap* mBh = g.maps[t.w] + 2 * g.b * g.nb + t.blk;
+    const CUtensorMap* mBl = mBh + g.nb;
+    const bool has_c = g.c >= 0;
+    const CUtensorMap* mCh = g.maps[t.w] + 2 * max(g.c, 0) * g.nb + t.blk;
+    const CUtensorMap* mCl = mCh + g.nb;
     const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + kStages), done = smem_u32(bars + 2 * kStages);
 
     if (tid == 0) {
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                     "r"(2 * N)
+                     "r"(2 * kTile)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -212,9 +212,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
 
     if (warp == 0 && lane == 0) {  // TMA producer
         int issued = 0;
-        for (int kc = 0; kc < nk + (has_c ? 1 : 0); ++kc) {
-            const int s = kc % kStages;
-            if (kc >= kStages && !mbar_wait(empty0 + 8 * s, ((kc / kStages) - 1) & 1)) {
+        uint32_t lap = 0;  // kc / kStages
+        for (int kc = 0, s = 0; kc < nk + (has_c ? 1 : 0); ++kc, s = s + 1 == kStages ? (++lap, 0) : s + 1) {
+            if (kc >= kStages && !mbar_wait(empty0 + 8 * s, (lap - 1) & 1)) {
                 *abort_flag = 1;
                 atomicExch(g.err, 1);
                 break;
@@ -240,9 +240,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
         }
         *issued_slot = issued;
     } else if (warp == 1 && lane == 0) {  // MMA issuer
-        for (int kc = 0; kc < nk; ++kc) {
-            const int s = kc % kStages;
-            if (!mbar_wait(full0 + 8 * s, (kc / kStages) & 1)) {
+        const uint32_t desc = idesc(N), desc2 = idesc(2 * N);
+        uint32_t lap = 0;
+        for (int kc = 0, s = 0; kc < nk; ++kc, s = s + 1 == kStages ? (++lap, 0) : s + 1) {
+            if (!mbar_wait(full0 + 8 * s, lap & 1)) {
                 *abort_flag = 1;
                 atomicExch(g.err, 2);
                 break;
@@ -253,10 +254,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
             for (int k = 0; k < kChunk / 16; ++k) {
                 const uint64_t ah = sdesc(base + 32 * k), al = sdesc(base + kTileBytes + 32 * k);
                 const uint64_t bh = sdesc(base + 2 * kTileBytes + 32 * k);
-                const uint64_t bl = sdesc(base + 2 * kTileBytes + kColBytes + 32 * k);
-                mma_f16<N>(tmem, ah, bh, (kc | k) != 0 ? 1u : 0u);
-                mma_f16<N>(tmem + N, ah, bl, (kc | k) != 0 ? 1u : 0u);
-                mma_f16<N>(tmem + N, al, bh, 1u);
+                // B_lo lies behind B_hi, and so do the accumulators: A_hi [B_hi; B_lo]
+                // is one product of 2 N columns, which reads A_hi once
+                mma_f16(tmem, ah, bh, desc2, (kc | k) != 0 ? 1u : 0u);
+                mma_f16(tmem + N, al, bh, desc, 1u);
             }
             mma_commit(empty0 + 8 * s);
         }
@@ -295,7 +296,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
 #pragma unroll 1
             for (int cc = half; cc < N / 32; cc += 2) {
                 float v[32];
-                load_acc<N>(row + (uint32_t)(32 * cc), v);
+                load_acc(row + (uint32_t)(32 * cc), N, v);
                 const long long gc0 = (long long)t.tj * N + 32 * cc;
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
@@ -315,8 +316,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
             // eight rows' units fall into different banks) and mirror (N rows of 128)
             unsigned char* tile = smem + ((c_slot + 1) % kStages) * kStageBytes;
             unsigned char* mirr = smem + ((c_slot + 2) % kStages) * kStageBytes;
-            constexpr int kOut = kTile * N * 2;  // bytes of one of hi, lo
-            auto perm = [](int rr) { return N >= 64 ? (rr & 7) : ((rr >> 1) & 3); };
+            const int kOut = kTile * N * 2;  // bytes of one of hi, lo
+            auto perm = [&](int rr) { return N >= 64 ? (rr & 7) : ((rr >> 1) & 3); };
             auto tile_at = [&](int rr, int col) { return rr * (2 * N) + ((((col >> 3) ^ perm(rr)) << 4) | ((col & 7) << 1)); };
             // C (gc, gr): row gc of box r / 64, its 16-byte units permuted by the TMA swizzle
             const unsigned char* cbase = smem + c_slot * kStageBytes + (r >> 6) * kColBytes + ((r & 7) << 1);
@@ -326,7 +327,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
 #pragma unroll 1
             for (int cc = half; cc < N / 32; cc += 2) {
                 float v[32];
-                load_acc<N>(row + (uint32_t)(32 * cc), v);
+                load_acc(row + (uint32_t)(32 * cc), N, v);
                 __half hi[32], lo[32];
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
@@ -368,8 +369,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
             __half* Dh = g.D_hi + B.off;
             __half* Dl = g.D_lo + B.off;
             const int r0 = diag ? c0 : 0;
-            for (int i = tid; i < (kTile - r0) * (N / 8); i += kGemmThreads) {
-                const int rr = r0 + i / (N / 8), q = i % (N / 8);
+            const int lg = 4 - t.w;  // units of a row: N / 8 = 2^lg
+            for (int i = tid; i < ((kTile - r0) << lg); i += kGemmThreads) {
+                const int rr = r0 + (i >> lg), q = i & ((1 << lg) - 1);
                 const int at = tile_at(rr, 8 * q);
                 const long long to = ((long long)t.ti * kTile + rr) * S + (long long)t.tj * N + 8 * q;
                 *reinterpret_cast<uint4*>(Dh + to) = *reinterpret_cast<const uint4*>(tile + at);
@@ -396,7 +398,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_f16x3_sym(GemmArgs g) {
     __syncthreads();
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * N) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * kTile) : "memory");
     }
 }
 
@@ -528,6 +530,85 @@ bool encode_map(CUtensorMap* m, const __half* base, int S, int rows) {
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Time an SM spends on a tile of width w and nk K steps, in us (fitted to single
+// blocks of order 300..1500 at each width).
+double tile_cost(int w, int nk) {
+    constexpr double step[kWidths] = {0.50, 0.42, 0.42}, rest[kWidths] = {6.0, 3.7, 3.0};
+    return rest[w] + step[w] * nk;
+}
+
+// Blocks of one padded order: their count and, with a width, their tiles.
+struct Group { int S, count; };
+long long tiles_of(const Group& g, int w) {
+    const long long T = g.S / kTile;
+    return (g.count * T * (T + 1) / 2) << w;
+}
+
+// Time until 152 SMs, each taking the longest tile left, are through; the groups
+// before `cut` have tiles of width a, the others of width b.
+double makespan(const std::vector<Group>& gs, int cut, int a, int b) {
+    std::vector<std::pair<double, long long>> jobs;  // cost, count
+    for (int i = 0; i < (int)gs.size(); ++i) {
+        const int w = i < cut ? a : b;
+        jobs.push_back({tile_cost(w, gs[i].S / kChunk), tiles_of(gs[i], w)});
+    }
+    std::stable_sort(jobs.begin(), jobs.end(), [](const auto& x, const auto& y) { return x.first > y.first; });
+    std::map<double, long long> load;  // busy until -> SMs
+    load[0.0] = kSMs;
+    for (auto [cost, n] : jobs)
+        while (n > 0) {
+            const auto it = load.begin();
+            const double at = it->first;
+            const long long k = std::min(n, it->second);
+            if (k == it->second) load.erase(it);
+            else it->second -= k;
+            load[at + cost] += k;
+            n -= k;
+        }
+    return load.rbegin()->first;
+}
+
+// The output tiles of every block.  Batches whose 32-column (64-column) tiles
+// fit the SMs at once take those; up to four waves of 128-column tiles, the
+// widths are one for the larger blocks and one for the smaller ones, whichever
+// pair and cut end first (four blocks of order 1500, 1052, 943 and 245: 162
+// tiles of 128 columns took 34.3 us a product, with these 32.4); beyond that 128.
+// The longest tiles come first, so that the last ones taken are short.
+void choose_tiles(NsLayout& L) {
+    std::vector<Group> gs;
+    std::map<int, int, std::greater<int>> by_order;
+    for (const Block& b : L.blocks) ++by_order[b.S];
+    long long wide = 0;
+    for (auto [S, n] : by_order) {
+        gs.push_back({S, n});
+        wide += tiles_of(gs.back(), 0);
+    }
+    int a = 0, b = 0, cut = 0;
+    if (wide * 4 <= kSMs) {
+        a = b = 2;
+    } else if (wide * 2 <= kSMs) {
+        a = b = 1;
+    } else if (wide <= 4 * kSMs && gs.size() <= 16) {
+        double best = 1e300;
+        for (int w0 = 0; w0 < kWidths; ++w0)
+            for (int w1 = w0; w1 < kWidths; ++w1)
+                for (int c = w0 == w1 ? (int)gs.size() : 1; c <= (int)gs.size(); ++c) {
+                    const double t = makespan(gs, c, w0, w1);
+                    if (t < best - 1e-9) { best = t; a = w0; b = w1; cut = c; }
+                }
+    }
+    const int small = cut < (int)gs.size() && !gs.empty() ? gs[cut].S : 0;  // orders up to it: width b
+    for (int k = 0; k < L.nb; ++k) {
+        const int w = L.blocks[k].S > small ? a : b;
+        L.widths[w] = true;
+        for (int i = 0; i < L.blocks[k].S / kTile; ++i)
+            for (int j = 0; j * width_of(w) < (i + 1) * kTile; ++j) L.tiles.push_back(Tile{k, i, j, w});
+    }
+    std::stable_sort(L.tiles.begin(), L.tiles.end(), [&](const Tile& x, const Tile& y) {
+        return tile_cost(x.w, L.blocks[x.blk].S / kChunk) > tile_cost(y.w, L.blocks[y.blk].S / kChunk);
+    });
+}
+
 inline size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
 
 }  // namespace
@@ -556,19 +637,15 @@ NsLayout ns_layout(const std::vector<int>& sizes) {
         L.max_upd = std::max(L.max_upd, nu);
     }
     if (L.upd_off.empty()) L.upd_off.push_back(0);
-    long long wide = 0;  // 128 x 128 tiles
-    for (const Block& b : L.blocks) wide += (long long)(b.S / kTile) * (b.S / kTile + 1) / 2;
-    L.cols = wide * 4 <= kSMs ? 32 : (wide * 2 <= kSMs ? 64 : kMaxCols);
-    for (size_t k = 0; k < L.blocks.size(); ++k)
-        for (int i = 0; i < L.blocks[k].S / kTile; ++i)
-            for (int j = 0; j * L.cols < (i + 1) * kTile; ++j) L.tiles.push_back(Tile{(int)k, i, j, 0});
+    choose_tiles(L);
     L.elems = off;
     size_t o = 0;
     L.o_err = o; o = up256(o + 16);
-    L.o_maps = o; o = up256(o + sizeof(CUtensorMap) * 2 * NBUF * (size_t)std::max(1, L.nb));
-    L.o_maps_b = o;  // operand B's boxes are as high as a tile is wide
-    if (L.cols != kTile) o = up256(o + sizeof(CUtensorMap) * 2 * NBUF * (size_t)std::max(1, L.nb));
-    else L.o_maps_b = L.o_maps;
+    // operand A's boxes are 128 rows high, B's and C's as high as a tile is wide
+    for (int w = 0; w < kWidths; ++w) {
+        L.o_maps[w] = o;
+        if (w == 0 || L.widths[w]) o = up256(o + sizeof(CUtensorMap) * 2 * NBUF * (size_t)std::max(1, L.nb));
+    }
     L.o_tiles = o; o = up256(o + sizeof(Tile) * std::max<size_t>(1, L.tiles.size()));
     L.o_blocks = o; o = up256(o + sizeof(Block) * std::max(1, L.nb));
     L.o_chunk = o; o = up256(o + sizeof(int) * (L.nb + 1));
@@ -595,14 +672,15 @@ bool ns_tables(const NsLayout& L, unsigned char* base, const std::vector<long lo
                const std::vector<int>& list, std::vector<unsigned char>& img) {
     if (!get_encode()) return false;
     img.assign(L.o_w, 0);
-    CUtensorMap* maps = reinterpret_cast<CUtensorMap*>(img.data() + L.o_maps);
-    CUtensorMap* maps_b = reinterpret_cast<CUtensorMap*>(img.data() + L.o_maps_b);
-    for (int buf = 0; buf < 2 * NBUF; ++buf)
-        for (int k = 0; k < L.nb; ++k) {
-            const __half* p = reinterpret_cast<const __half*>(base + L.o_buf[buf]) + L.blocks[k].off;
-            if (!encode_map(&maps[buf * L.nb + k], p, L.blocks[k].S, kTile)) return false;
-            if (L.cols != kTile && !encode_map(&maps_b[buf * L.nb + k], p, L.blocks[k].S, L.cols)) return false;
-        }
+    for (int w = 0; w < kWidths; ++w) {
+        if (w > 0 && !L.widths[w]) continue;
+        CUtensorMap* maps = reinterpret_cast<CUtensorMap*>(img.data() + L.o_maps[w]);
+        for (int buf = 0; buf < 2 * NBUF; ++buf)
+            for (int k = 0; k < L.nb; ++k) {
+                const __half* p = reinterpret_cast<const __half*>(base + L.o_buf[buf]) + L.blocks[k].off;
+                if (!encode_map(&maps[buf * L.nb + k], p, L.blocks[k].S, width_of(w))) return false;
+            }
+    }
     std::memcpy(img.data() + L.o_tiles, L.tiles.data(), sizeof(Tile) * L.tiles.size());
     std::memcpy(img.data() + L.o_blocks, L.blocks.data(), sizeof(Block) * L.blocks.size());
     std::memcpy(img.data() + L.o_chunk, L.chunk_off.data(), sizeof(int) * L.chunk_off.size());
@@ -614,11 +692,10 @@ bool ns_tables(const NsLayout& L, unsigned char* base, const std::vector<long lo
 
 namespace {
 
-template <int N>
 cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t st) {
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_f16x3_sym<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(N));
+        cudaError_t e = cudaFuncSetAttribute(k_f16x3_sym, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
         if (e != cudaSuccess) return e;
         attr = true;
     }
@@ -628,26 +705,23 @@ cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(g.ntiles);
     cfg.blockDim = dim3(kGemmThreads);
-    cfg.dynamicSmemBytes = gemm_smem(N);
+    cfg.dynamicSmemBytes = kGemmSmem;
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_f16x3_sym<N>, g);
+    return cudaLaunchKernelEx(&cfg, k_f16x3_sym, g);
 }
 
 // D = alpha A B + beta C on pairs; with d < 0 the last product, P = (W + |W|_F A B) / 2.
 cudaError_t gemm(const NsLayout& L, unsigned char* base, int a, int bsrc, int c, int d, float alpha, float beta,
                  cudaStream_t st) {
-    const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(base + L.o_maps);
-    const CUtensorMap* maps_b = reinterpret_cast<const CUtensorMap*>(base + L.o_maps_b);
     auto half_buf = [&](int i) { return reinterpret_cast<__half*>(base + L.o_buf[i]); };
     GemmArgs g;
-    g.mapA_hi = maps + (2 * a) * L.nb;
-    g.mapA_lo = maps + (2 * a + 1) * L.nb;
-    g.mapB_hi = maps_b + (2 * bsrc) * L.nb;
-    g.mapB_lo = maps_b + (2 * bsrc + 1) * L.nb;
-    g.mapC_hi = c >= 0 ? maps_b + (2 * c) * L.nb : nullptr;
-    g.mapC_lo = c >= 0 ? maps_b + (2 * c + 1) * L.nb : nullptr;
+    for (int w = 0; w < kWidths; ++w) g.maps[w] = reinterpret_cast<const CUtensorMap*>(base + L.o_maps[w]);
+    g.a = a;
+    g.b = bsrc;
+    g.c = c;
+    g.nb = L.nb;
     g.D_hi = d >= 0 ? half_buf(2 * d) : nullptr;
     g.D_lo = d >= 0 ? half_buf(2 * d + 1) : nullptr;
     g.W = reinterpret_cast<const float*>(base + L.o_w);
@@ -659,7 +733,7 @@ cudaError_t gemm(const NsLayout& L, unsigned char* base, int a, int bsrc, int c,
     g.alpha = alpha;
     g.beta = beta;
     g.err = reinterpret_cast<int*>(base + L.o_err);
-    return L.cols == 32 ? launch_gemm<32>(g, st) : (L.cols == 64 ? launch_gemm<64>(g, st) : launch_gemm<128>(g, st));
+    return launch_gemm(g, st);
 }
 
 }  // namespace

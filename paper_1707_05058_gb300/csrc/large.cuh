@@ -40,6 +40,7 @@
 // them): 3.93 -> 3.27 ms a projection.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -47,29 +48,33 @@
 namespace cdsdp_large {
 
 constexpr int kTile = 128;         // rows of an output tile, one CTA each
-// Columns of an output tile: 128, or 64 or 32 when the batch has so few
-// 128 x 128 tiles that the narrower ones still fit one wave of the 152 SMs.  An
-// SM takes in about 45 B a clock from L2, which is what a K step costs (64 KB
-// of operands at 128 columns, 48 KB at 64, 40 KB at 32, where its MMAs take
-// about 840, 420 and 210 clocks), so the narrow tiles are less efficient but finish
-// sooner while SMs would stand idle otherwise.  Every entry is the same sum in
-// the same order at each width.
-constexpr int kMaxCols = 128;
+// Columns of an output tile: 128, 64 or 32, chosen block by block (choose_tiles).
+// A K step of 64 costs 0.50 us at 128 columns and 0.42 us at 64 and 32 (shared
+// memory: the operands are written once and read by two MMAs a 16-wide step), a
+// launch with its first loads and its epilogue 11, 8.7 and 8.0 us: narrow tiles
+// are less efficient but finish sooner while SMs would stand idle otherwise.
+// (A_hi B_hi, A_hi B_lo and A_lo B_hi as three MMAs read A_hi twice: 0.65, 0.64
+// and 0.61 us a K step.)  Every entry is the same sum in the same order at each
+// width.
+constexpr int kWidths = 3;
+__host__ __device__ constexpr int width_of(int w) { return kTile >> w; }
 constexpr int kChunk = 64;         // K halves per stage: one 128-byte swizzle row
-// Stages of the operand ring: about 192 KB in flight at every width.
-__host__ __device__ constexpr int stages(int cols) { return cols == 128 ? 3 : (cols == 64 ? 4 : 5); }
 constexpr int kTileBytes = kTile * kChunk * 2;       // 16 KB per operand tile of 128 rows
 __host__ __device__ constexpr int stage_bytes(int cols) { return 2 * kTileBytes + 2 * cols * kChunk * 2; }  // A_hi, A_lo, B_hi, B_lo
-constexpr int gemm_smem(int cols) { return stages(cols) * stage_bytes(cols) + 1024 + 256; }
+// Stages of the operand ring: about 192 KB in flight at every width.
+__host__ __device__ constexpr int stages(int cols) { return cols == 128 ? 3 : (cols == 64 ? 4 : 5); }
+constexpr int kRingBytes = 5 * stage_bytes(32);      // the largest of the three rings
+constexpr int kGemmSmem = kRingBytes + 1024 + 256;
+static_assert(kRingBytes >= 3 * stage_bytes(128) && kRingBytes >= 4 * stage_bytes(64), "ring");
 constexpr int kGemmThreads = 256;  // producer, MMA issuer; all warps read the accumulator
 
 // Phase-1 polynomial and the iteration counts.
 constexpr float kPa = 3.30f, kPb = -3.66f, kPc = 1.36f;
 constexpr int kPhase1 = 16, kPhase2 = 5;
 
-// One output tile of block `blk`: rows 128 ti .., columns (tile width) tj ..; it
+// One output tile of block `blk`: rows 128 ti .., columns width_of(w) tj ..; it
 // reaches into the lower triangle.
-struct Tile { int blk, ti, tj, pad; };
+struct Tile { int blk, ti, tj, w; };
 
 // Dense layout of one block in every buffer: float offset and padded order.
 struct Block { long long off; int S, s; };
@@ -92,9 +97,8 @@ __device__ __forceinline__ float pair_value(__half hi, __half lo) {
 // Epilogue of one product over the lower tiles: D = alpha A B + beta C, all
 // (hi, lo) pairs; or, with P set, P = (W + |W|_F A B) / 2 in float32.
 struct GemmArgs {
-    const void* mapA_hi; const void* mapA_lo;   // tensor maps, one per block (CUtensorMap arrays)
-    const void* mapB_hi; const void* mapB_lo;
-    const void* mapC_hi; const void* mapC_lo;   // C's (boxes as B's); nullptr without C
+    const CUtensorMap* maps[kWidths];  // per box height width_of(w): [buffer][hi, lo][block]
+    int a, b, c, nb;                   // operands' buffers (c < 0: no C), number of blocks
     __half* D_hi; __half* D_lo;
     const float* W; float* P;
     const double* scale;                        // |W|_F per block

@@ -23,7 +23,7 @@ constexpr int kUpdChunk = 2048;
 // each holding every block at Block::off with row pitch Block::S.
 struct NsLayout {
     int nb = 0;
-    int cols = kMaxCols;            // columns of an output tile
+    bool widths[kWidths] = {false}; // tile widths in use
     int max_S = 0;
     long long elems = 0;            // elements per buffer
     std::vector<Block> blocks;
@@ -31,7 +31,7 @@ struct NsLayout {
     std::vector<int> chunk_off;     // row chunks of the norm reduction, per block
     std::vector<int> upd_off;       // packed-entry chunks of the gather / update, per block
     int max_upd = 0;                // most packed-entry chunks of one block
-    size_t o_err = 0, o_maps = 0, o_maps_b = 0, o_tiles = 0, o_blocks = 0, o_chunk = 0, o_partial = 0, o_scale = 0, o_poff = 0;
+    size_t o_err = 0, o_maps[kWidths] = {0}, o_tiles = 0, o_blocks = 0, o_chunk = 0, o_partial = 0, o_scale = 0, o_poff = 0;
     size_t o_list = 0, o_upd = 0, o_updpart = 0;
     size_t o_w = 0;                 // dense W
     size_t o_buf[2 * NBUF] = {0};
