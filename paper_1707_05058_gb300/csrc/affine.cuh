@@ -59,8 +59,9 @@ __global__ void __launch_bounds__(ETHREADS) k_scatter(Dev d, const T* __restrict
 // The same scatter walked in packed-position order, for problems whose
 // entries mostly lie in one clique (Gs = 1): the thread of position q reads
 // the clique values at q, and only the entry's first position (owner[q])
-// writes out[e]; an entry in several cliques sums its positions in the order
-// of the CSR row, as k_scatter with one lane per entry does (bit-identical).
+// writes out[e]; an entry in several cliques, but not more than kLongList, sums
+// its positions in the order of the CSR row, as k_scatter with one lane per entry
+// does (bit-identical).
 // Clique values and the index map are read in order (coalesced); the entry
 // data are read in the order the cliques list their entries.
 template <typename T>
@@ -70,6 +71,27 @@ __global__ void __launch_bounds__(ETHREADS) k_scatter_owner(Dev d, const T* __re
                                                             double* __restrict__ out, int check_stop) {
     if (check_stop && stopped(d)) return;
     const int stride = gridDim.x * blockDim.x;
+    // entries in many cliques: a warp each, before its share of the others
+    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < d.nlong; i += stride >> 5) {
+        const int e = d.lent[i];
+        if (check_stop && frozen_entry(d, e)) continue;  // warp-uniform
+        double a = alpha, gm = gamma;
+        if (alpha_rho || gamma_rho) {
+            const double ir = irho_entry(d, e);
+            if (alpha_rho) a *= ir;
+            if (gamma_rho) gm *= ir;
+        }
+        double acc = 0.0;
+        for (int j = d.sc_ptr[e] + (threadIdx.x & 31); j < d.sc_ptr[e + 1]; j += 32) {
+            const int qq = d.sc_idx[j];
+            acc += Q ? double(P[qq]) + gm * double(Q[qq]) : double(P[qq]);
+        }
+        acc = warp_sum(acc);
+        if ((threadIdx.x & 31) == 0) {
+            const double r = a * d.c[e] + beta * acc;
+            out[e] = scale ? r * scale[e] : r;
+        }
+    }
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < d.nd; q += stride) {
         if (!d.owner[q]) continue;
         const int e = d.gmap[q];
@@ -81,6 +103,7 @@ __global__ void __launch_bounds__(ETHREADS) k_scatter_owner(Dev d, const T* __re
             if (gamma_rho) gm *= ir;
         }
         const int j0 = d.sc_ptr[e], j1 = d.sc_ptr[e + 1];
+        if (j1 - j0 > kLongList) continue;
         double acc = 0.0;
         if (j1 - j0 == 1) {
             acc += Q ? double(P[q]) + gm * double(Q[q]) : double(P[q]);
@@ -140,8 +163,11 @@ __global__ void __launch_bounds__(RTHREADS) k_rows_aw(Dev d, const double* __res
         double s = 0.0;
         const bool live = i < d.m && !frozen_row(d, i);
         if (live) {
-            const int q1 = d.a_ptr[i + 1];
-            for (int q = d.a_ptr[i] + tig; q < q1; q += TPR) s += d.a_valw[q] * v[d.a_col[q]];
+            const int q0 = d.a_ptr[i], q1 = d.a_ptr[i + 1];
+            // long rows: more in flight (409 rows of 25,710: 67 us one term at a time,
+            // 48 four, 39 eight; 3,600 rows of 900: 45, 40 and 46 us)
+            s = q1 - q0 > 8 * TPR ? sparse_dot<8, true>(d.a_valw, d.a_col, v, q0 + tig, q1, TPR)
+                                  : sparse_dot<4, true>(d.a_valw, d.a_col, v, q0 + tig, q1, TPR);
         }
         s = row_group_sum(s, TPR, sh);
         if (live && tig == 0) out[i] = s + (delta_rho ? delta / rho_row(d, i) : delta) * d.b[i];

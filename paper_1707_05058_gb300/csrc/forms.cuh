@@ -13,13 +13,18 @@ namespace cdsdp_dev {
 __device__ void finish_dual_block(const Dev& d, const FinishArgs& fa);
 
 template <typename T>
-__global__ void __launch_bounds__(128) k_vlam_dual(Dev d, FinishArgs fa) {
+__global__ void __launch_bounds__(128) k_vlam_dual(Dev d, FinishArgs fa, int whole) {
     if (stopped(d)) return;
-    const int lane = threadIdx.x & 31;
-    const int w0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    __shared__ double sh[4][5];
+    const int warp = threadIdx.x >> 5, step = whole ? 128 : 32;
+    const int lane = whole ? threadIdx.x : threadIdx.x & 31;
+    const int w0 = whole ? blockIdx.x : blockIdx.x * 4 + warp, nw = whole ? gridDim.x : gridDim.x * 4;
     const T* z = reinterpret_cast<const T*>(d.ck0);
     T* v = reinterpret_cast<T*>(d.ck1);
     T* lam = reinterpret_cast<T*>(d.ck2);
+    // Eight of a lane's entries at a time: their loads cannot pass the stores, and
+    // one after the other an order-30 clique's 15 a lane took 37 us, so 25.
+    constexpr int B = 8;
     double acc[4] = {0, 0, 0, 0};
     for (int k = w0; k < d.p; k += nw) {
         if (frozen_clique(d, k)) continue;  // warp-uniform
@@ -29,25 +34,53 @@ __global__ void __launch_bounds__(128) k_vlam_dual(Dev d, FinishArgs fa) {
         // stored in T; the per-clique sums of the stopping test are in T
         T p0 = 0, p1 = 0, p2 = 0, p3 = 0;
         double cx = 0;
-        for (int f = lane; f < npk; f += 32) {
-            const int ent = d.gmap[off + f];
-            if (d.comp_mode && d.owner[off + f]) cx += d.wgt[ent] * d.c[ent] * d.x[ent];
-            const T zt = z[off + f];
-            const double zz = zt, ll = lam[off + f];
-            const T vn = T(zz + ll * irho + d.x[ent]);
-            const T ln = T(ll + rho * (zz - double(vn)));
-            v[off + f] = vn;
-            lam[off + f] = ln;
-            const T wt = T(d.wgt[ent]);
-            const T dv = zt - vn;
-            p0 += wt * dv * dv;
-            p1 += wt * zt * zt;
-            p2 += wt * vn * vn;
-            p3 += wt * ln * ln;
+        for (int f0 = lane; f0 < npk; f0 += step * B) {
+            int ent[B];
+            T zt[B], lm[B], wt[B];
+            double xe[B];
+#pragma unroll
+            for (int u = 0; u < B; ++u) {
+                const int f = f0 + step * u;
+                const bool ok = f < npk;
+                ent[u] = ok ? d.gmap[off + f] : -1;
+                zt[u] = ok ? z[off + f] : T(0);
+                lm[u] = ok ? lam[off + f] : T(0);
+            }
+#pragma unroll
+            for (int u = 0; u < B; ++u) {
+                xe[u] = ent[u] >= 0 ? d.x[ent[u]] : 0.0;
+                wt[u] = ent[u] >= 0 ? T(d.wgt[ent[u]]) : T(0);
+            }
+#pragma unroll
+            for (int u = 0; u < B; ++u) {
+                const int f = f0 + step * u;
+                if (f >= npk) break;
+                if (d.comp_mode && d.owner[off + f]) cx += d.wgt[ent[u]] * d.c[ent[u]] * xe[u];
+                const double zz = zt[u], ll = lm[u];
+                const T vn = T(zz + ll * irho + xe[u]);
+                const T ln = T(ll + rho * (zz - double(vn)));
+                v[off + f] = vn;
+                lam[off + f] = ln;
+                const T dv = zt[u] - vn;
+                p0 += wt[u] * dv * dv;
+                p1 += wt[u] * zt[u] * zt[u];
+                p2 += wt[u] * vn * vn;
+                p3 += wt[u] * ln * ln;
+            }
         }
-        const double q[4] = {double(warp_sum(p0)), double(warp_sum(p1)), double(warp_sum(p2)), double(warp_sum(p3))};
+        double q[4] = {double(warp_sum(p0)), double(warp_sum(p1)), double(warp_sum(p2)), double(warp_sum(p3))};
+        double cxk = d.comp_mode ? warp_sum(cx) : 0.0;
+        if (whole) {  // over the warps, in order; warp 0 goes on with the sums
+            __syncthreads();  // the previous clique's are read
+            if ((threadIdx.x & 31) == 0) {
+                for (int c = 0; c < 4; ++c) sh[warp][c] = q[c];
+                sh[warp][4] = cxk;
+            }
+            __syncthreads();
+            for (int c = 0; c < 4; ++c) q[c] = warp == 0 ? ((sh[0][c] + sh[1][c]) + sh[2][c]) + sh[3][c] : 0.0;
+            cxk = ((sh[0][4] + sh[1][4]) + sh[2][4]) + sh[3][4];
+        }
         if (d.comp_mode) {  // per-clique row (column 6: <c, x> over the entries the clique owns)
-            const double cxk = warp_sum(cx);
             if (lane == 0) {
                 double* pr = d.part + (size_t)k * PART_COLS;
                 for (int c = 0; c < 4; ++c) pr[c] = q[c];
@@ -232,23 +265,31 @@ __global__ void __launch_bounds__(ETHREADS) k_hsde_eta(Dev d, int G) {
     const int gid = (blockIdx.x * blockDim.x + threadIdx.x) / G, lig = threadIdx.x & (G - 1);
     const int ng = (gridDim.x * blockDim.x) / G;
     const int nloop = (d.NE + ng - 1) / ng;
+    auto gather = [&](int e, int l, int step) {
+        double acc = 0.0;
+        const int j1 = d.sc_ptr[e + 1];
+        for (int j = d.sc_ptr[e] + l; j < j1; j += step) {
+            const int q = d.sc_idx[j];
+            acc += double(us[q]) + double(vz[q]) + double(ut[q]);
+        }
+        return acc;
+    };
+    auto store = [&](int e, double acc) {
+        const int c = comp_e(d, e);
+        const double w2 = hs_tau_c(d, c) + hs_kappa_c(d, c);
+        const double eta = d.x[e] - w2 * d.c[e] + d.atuy[e] + w2 * d.atb[e] + 0.5 * acc;
+        d.q[e] = eta * d.pinv[e];
+    };
+    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < d.nlong; i += (gridDim.x * blockDim.x) >> 5) {
+        const int e = d.lent[i];
+        const double acc = warp_sum(gather(e, threadIdx.x & 31, 32));
+        if ((threadIdx.x & 31) == 0 && !frozen_entry(d, e)) store(e, acc);
+    }
     for (int it = 0; it < nloop; ++it) {
         const int e = gid + it * ng;
-        double acc = 0.0;
-        if (e < d.NE) {
-            const int j1 = d.sc_ptr[e + 1];
-            for (int j = d.sc_ptr[e] + lig; j < j1; j += G) {
-                const int q = d.sc_idx[j];
-                acc += double(us[q]) + double(vz[q]) + double(ut[q]);
-            }
-        }
-        acc = group_sum(acc, G);
-        if (e < d.NE && lig == 0 && !frozen_entry(d, e)) {
-            const int c = comp_e(d, e);
-            const double w2 = hs_tau_c(d, c) + hs_kappa_c(d, c);
-            const double eta = d.x[e] - w2 * d.c[e] + d.atuy[e] + w2 * d.atb[e] + 0.5 * acc;
-            d.q[e] = eta * d.pinv[e];
-        }
+        const bool mine = e < d.NE && d.sc_ptr[e + 1] - d.sc_ptr[e] <= kLongList;
+        const double acc = group_sum(mine ? gather(e, lig, G) : 0.0, G);
+        if (mine && lig == 0 && !frozen_entry(d, e)) store(e, acc);
     }
 }
 
@@ -265,8 +306,7 @@ __global__ void __launch_bounds__(ETHREADS) k_hsde_sigma11(Dev d, int G) {
         const int e = gid + it * ng;
         double s = 0.0;
         if (e < d.NE) {
-            const int q1 = d.at_ptr[e + 1];
-            for (int q = d.at_ptr[e] + lig; q < q1; q += G) s += d.at_val[q] * d.hh[d.at_col[q]];
+            s = sparse_dot<4, false>(d.at_val, d.at_col, d.hh, d.at_ptr[e] + lig, d.at_ptr[e + 1], G);
         }
         s = group_sum(s, G);
         if (e < d.NE && lig == 0 && !frozen_entry(d, e)) {
@@ -295,7 +335,7 @@ __global__ void __launch_bounds__(RTHREADS) k_hsde_sigma21(Dev d, int TPR, int n
         double s = 0.0;
         if (i < d.m) {
             const int q1 = d.a_ptr[i + 1];
-            for (int q = d.a_ptr[i] + tig; q < q1; q += TPR) s += d.a_valw[q] * d.s11[d.a_col[q]];
+            s = sparse_dot<4, true>(d.a_valw, d.a_col, d.s11, d.a_ptr[i] + tig, q1, TPR);
         }
         s = row_group_sum(s, TPR, sh);
         if (i < d.m && tig == 0 && !frozen_row(d, i)) {
@@ -410,35 +450,43 @@ __global__ void __launch_bounds__(ETHREADS) k_hsde_entry_update(Dev d, int G) {
     const int ng = (gridDim.x * blockDim.x) / G;
     const int nloop = (d.NE + ng - 1) / ng;
     double p[2] = {0.0, 0.0};
+    auto gather = [&](int e, int l, int step, double& a, double& hv) {
+        a = sparse_dot<4, false>(d.at_val, d.at_col, d.y, d.at_ptr[e] + l, d.at_ptr[e + 1], step);
+        const int j1 = d.sc_ptr[e + 1];
+        for (int j = d.sc_ptr[e] + l; j < j1; j += step) hv += double(vz[d.sc_idx[j]]);
+    };
+    auto store = [&](int e, double a, double hv) {
+        const int ce = comp_e(d, e);
+        const double gamma = hs_gamma_c(d, ce), tau = hs_tau_c(d, ce);
+        const double ux = d.s11[e] - gamma * d.zhx[e];
+        const double r = a + hv - tau * d.c[e];
+        const double we = d.wgt[e], cw = we * d.c[e] * ux;
+        d.x[e] = ux;
+        d.atuy[e] = a;
+        p[0] += we * r * r;
+        p[1] += cw;
+        if (d.comp_mode) {  // per-entry terms, summed per component by k_finish_hsde_components
+            d.t[e] = we * r * r;
+            d.q[e] = cw;
+        }
+    };
+    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < d.nlong; i += (gridDim.x * blockDim.x) >> 5) {
+        const int e = d.lent[i];
+        if (frozen_entry(d, e)) continue;  // warp-uniform
+        double a = 0.0, hv = 0.0;
+        gather(e, threadIdx.x & 31, 32, a, hv);
+        a = warp_sum(a);
+        hv = warp_sum(hv);
+        if ((threadIdx.x & 31) == 0) store(e, a, hv);
+    }
     for (int it = 0; it < nloop; ++it) {
         const int e = gid + it * ng;
         double a = 0.0, hv = 0.0;
-        const bool live = e < d.NE && !frozen_entry(d, e);
-        const int ce = live ? comp_e(d, e) : 0;
-        const double gamma = live ? hs_gamma_c(d, ce) : 0.0, tau = live ? hs_tau_c(d, ce) : 0.0;
-        if (live) {
-            const int q1 = d.at_ptr[e + 1];
-            for (int q = d.at_ptr[e] + lig; q < q1; q += G) {
-                const int i = d.at_col[q];
-                a += d.at_val[q] * d.y[i];
-            }
-            const int j1 = d.sc_ptr[e + 1];
-            for (int j = d.sc_ptr[e] + lig; j < j1; j += G) hv += double(vz[d.sc_idx[j]]);
-        }
+        const bool live = e < d.NE && !frozen_entry(d, e) && d.sc_ptr[e + 1] - d.sc_ptr[e] <= kLongList;
+        if (live) gather(e, lig, G, a, hv);
         a = group_sum(a, G);
         hv = group_sum(hv, G);
-        if (live && lig == 0) {
-            const double ux = d.s11[e] - gamma * d.zhx[e];
-            d.x[e] = ux;
-            d.atuy[e] = a;
-            const double r = a + hv - tau * d.c[e];
-            p[0] += d.wgt[e] * r * r;
-            p[1] += d.wgt[e] * d.c[e] * ux;
-            if (d.comp_mode) {  // per-entry terms, summed per component by k_finish_hsde_components
-                d.t[e] = d.wgt[e] * r * r;
-                d.q[e] = d.wgt[e] * d.c[e] * ux;
-            }
-        }
+        if (live && lig == 0) store(e, a, hv);
     }
     block_sum<2>(p, sh);
     if (threadIdx.x == 0) {

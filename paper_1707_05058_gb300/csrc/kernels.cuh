@@ -63,6 +63,8 @@ struct Dev {
     const unsigned char* owner;  // [nd] 1 at the first packed position of each pattern entry
     const double* a_valu; // [nnzA] A_ie unweighted, CSR by rows (reverse pass)
     void* wstore;         // when set, primal projections record W of iteration n at wstore + n * nd
+    const int* lent;      // [nlong] entries in more than kLongList cliques
+    int nlong;
     int wstore_count;     // iterations that fit in wstore
     double* part;         // [p * PART_COLS] per-clique partial sums
     double* parte;        // [NBLK_E * PART_COLS] per-block partials, pattern-entry kernels
@@ -114,6 +116,10 @@ struct Dev {
     int cg_max;
 };
 
+// Entries in more cliques than this have a warp to themselves in the kernels that
+// give an entry few lanes (d.lent): a lane's chain of 100 gathers, one per clique
+// of a block-arrow SDP's head entry, took 30 us a scatter.
+constexpr int kLongList = 16;
 constexpr int NBLK_E = 1216;  // 152 SMs x 8
 constexpr int NBLK_R = 1216;
 constexpr int ETHREADS = 256;
@@ -221,6 +227,32 @@ __device__ __forceinline__ double factor_row_dot(const Dev& d, const double* __r
     } else {
         const int* idx = d.crow_idx + r0;
         for (int j = t0; j < mc; j += step) s += row[j] * g[idx[j]];
+    }
+    return s;
+}
+
+// sum over q = q0, q0 + step, .. < q1 of val[q] v[col[q]], in that order, U
+// terms' loads at a time.  STREAM: the matrix is read past L1, which keeps v (for
+// warps that read it in whole lines; a lane that walks a short row of its own
+// finds its next elements in L1).
+template <int U, bool STREAM>
+__device__ __forceinline__ double sparse_dot(const double* __restrict__ val, const int* __restrict__ col,
+                                             const double* __restrict__ v, int q0, int q1, int step) {
+    double s = 0.0;
+    for (int q = q0; q < q1; q += U * step) {
+        int c[U];
+        double a[U], x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const bool ok = q + u * step < q1;
+            c[u] = ok ? (STREAM ? __ldcs(col + q + u * step) : __ldg(col + q + u * step)) : -1;
+            a[u] = ok ? (STREAM ? __ldcs(val + q + u * step) : __ldg(val + q + u * step)) : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) x[u] = c[u] >= 0 ? v[c[u]] : 0.0;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (c[u] >= 0) s += a[u] * x[u];
     }
     return s;
 }

@@ -37,7 +37,7 @@ struct Layout {
     size_t c, dinv, pinv, wgt, a_ptr, a_col, a_valw, a_valu, at_ptr, at_col, at_val, b, minv, kinv, gmap, pk_off, csize,
         sc_ptr, sc_idx, zhx, zhy, atb, azhx, blist, brec, vv_off, owner, comp_of_entry, comp_of_clique, comp_of_row, lrow,
         crow_ptr, crow_idx, ccl_ptr, ccl_idx, minv_off, cent_ptr, cent_idx, hs_nb, hs_nc, zhx_c, zhy_c, azhx_c,
-        hs_zdz;
+        hs_zdz, lent;
     size_t const_end;
     // state
     size_t x, t, q, s11, atuy, y, g, hh, s21, as11, ck0, ck1, ck2, vcache, part, parte, partr, scal, ctl, hist,
@@ -125,6 +125,14 @@ std::vector<int> large_sizes(const HostProblem& hp) {
     return s;
 }
 
+// Entries in more than kLongList cliques (the head of a block-arrow SDP).
+std::vector<int> long_entries(const HostProblem& hp) {
+    std::vector<int> l;
+    for (size_t e = 0; e < hp.prow.size(); ++e)
+        if (hp.sc_ptr[e + 1] - hp.sc_ptr[e] > kLongList) l.push_back((int)e);
+    return l;
+}
+
 Layout make_layout(const HostProblem& hp, int max_iter) {
     Layout L{};
     size_t o = 0;
@@ -149,6 +157,7 @@ Layout make_layout(const HostProblem& hp, int max_iter) {
     L.minv_off = take(nc * 8);
     L.cent_ptr = take((nc + 1) * 4); L.cent_idx = take(NE * 4); L.hs_nb = take(nc * 8); L.hs_nc = take(nc * 8);
     L.zhx_c = take(NE * 8); L.zhy_c = take(m * 8); L.azhx_c = take(m * 8); L.hs_zdz = take(nc * 8);
+    L.lent = take(long_entries(hp).size() * 4);
     L.const_end = o;
     L.x = take(NE * 8); L.t = take(NE * 8); L.q = take(NE * 8); L.s11 = take(NE * 8); L.atuy = take(NE * 8);
     L.y = take(m * 8); L.g = take(m * 8); L.hh = take(m * 8); L.s21 = take(m * 8); L.as11 = take(m * 8);
@@ -238,6 +247,7 @@ void build_image(cdsdp* h) {
     put(img, L.ccl_ptr, hp.ccl_ptr); put(img, L.ccl_idx, hp.ccl_idx); put(img, L.minv_off, hp.minv_off);
     put(img, L.cent_ptr, hp.cent_ptr); put(img, L.cent_idx, hp.cent_idx);
     put(img, L.hs_nb, hp.comp_nb); put(img, L.hs_nc, hp.comp_nc);
+    put(img, L.lent, long_entries(hp));
 }
 
 void make_dev(cdsdp* h) {
@@ -286,6 +296,8 @@ void make_dev(cdsdp* h) {
     d.hs_tau = (double*)(w + L.hs_tau); d.hs_kappa = (double*)(w + L.hs_kappa); d.hs_gamma = (double*)(w + L.hs_gamma);
     d.hs_zdz = (const double*)(w + L.hs_zdz); d.hs_nb = (const double*)(w + L.hs_nb);
     d.hs_nc = (const double*)(w + L.hs_nc);
+    d.lent = (const int*)(w + L.lent);
+    d.nlong = (int)long_entries(hp).size();
     d.cent_ptr = (const int*)(w + L.cent_ptr); d.cent_idx = (const int*)(w + L.cent_idx);
     auto pow2_clamp = [](double x, int lo, int hi) {
         int v = lo;
@@ -446,7 +458,10 @@ template <typename T>
 cudaError_t launch_iteration(cdsdp* h, int form, const cdsdp_opts& o, cudaStream_t st, int use_cond,
                              cudaGraphConditionalHandle hnd, cudaEvent_t ev0, cudaEvent_t ev1) {
     Dev& d = h->dev;
-    const int GE = h->GE, GR = h->GR, PG = std::max(1, std::min((d.p + 3) / 4, 152 * 32));
+    // Algorithm 2's v and lambda: a block per clique where all of them fit the chip
+    // at once and have more entries than a warp takes at a time, else a warp
+    const int whole = d.p <= 152 * 4 && (long long)d.nd > 256LL * d.p;
+    const int GE = h->GE, GR = h->GR, PG = whole ? std::max(1, d.p) : std::max(1, std::min((d.p + 3) / 4, 152 * 32));
     FinishArgs fa;
     fa.eps = o.eps;
     fa.mu = o.rho_mu;
@@ -493,13 +508,13 @@ cudaError_t launch_iteration(cdsdp* h, int form, const cdsdp_opts& o, cudaStream
         if (o.linear_solver == 1) launch_cg(h, o, st);
         else k_gemv<<<GR, RTHREADS, 0, st>>>(d, d.minv, d.g, d.y, 0, h->TPRM);
         k_xupd<<<GE, ETHREADS, 0, st>>>(d, d.t, d.y, d.x, h->Ga, 1);
-        k_vlam_dual<T><<<PG, 128, 0, st>>>(d, fin);
+        k_vlam_dual<T><<<PG, 128, 0, st>>>(d, fin, whole);
         if (d.comp_mode) k_finish_components<<<d.ncomp, 256, 0, st>>>(d, 1, fa);
     } else {  // Algorithm 3; gamma/tau/kappa in sigma21's last block, stopping test in row_update's
         k_hsde_eta<T><<<GE, ETHREADS, 0, st>>>(d, h->Gs);
         k_rows_aw<<<GR, RTHREADS, 0, st>>>(d, d.q, 0.0, 0, d.g, h->TPR);
         k_gemv<<<GR, RTHREADS, 0, st>>>(d, d.kinv, d.g, d.hh, -1, h->TPRM);
-        k_hsde_sigma11<<<GE, ETHREADS, 0, st>>>(d, h->Ga);
+        k_hsde_sigma11<<<GE, ETHREADS, 0, st>>>(d, h->Gx);
         k_hsde_sigma21<<<GR, RTHREADS, 0, st>>>(d, h->TPR, GE);
         if (d.comp_mode) k_hsde_gamma_components<<<dim3(h->hs_parts, d.ncomp), 256, 0, st>>>(d);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -508,7 +523,7 @@ cudaError_t launch_iteration(cdsdp* h, int form, const cdsdp_opts& o, cudaStream
         none.enabled = 0;
         if ((e = launch_projection<T>(h, 2, o, none, st)) != cudaSuccess) return e;
         if (ev1) cudaEventRecord(ev1, st);
-        k_hsde_entry_update<T><<<GE, ETHREADS, 0, st>>>(d, h->Ga);
+        k_hsde_entry_update<T><<<GE, ETHREADS, 0, st>>>(d, h->Gx);
         k_hsde_row_update<<<GR, RTHREADS, 0, st>>>(d, fa);
         if (d.comp_mode) k_finish_hsde_components<<<dim3(h->hs_parts, d.ncomp), 256, 0, st>>>(d, fa);
     }
