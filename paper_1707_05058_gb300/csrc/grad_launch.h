@@ -13,8 +13,7 @@ struct GradArgs {
     const double* lambar; // [nd] adjoint of the multipliers after the iteration
     double* hxbar;        // [nd] out: adjoint of H x
     double* lamprev;      // [nd] out: multiplier adjoint before the affine-step terms
-    double rho, tolrel;
-    int max_sweeps;
+    double rho;
     int slot;             // recorded iteration within the replayed segment
 };
 

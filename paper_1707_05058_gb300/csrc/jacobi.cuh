@@ -760,10 +760,6 @@ __global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4)) k_proj
                     const int ab = packed_ab(f, s), a = ab >> 8, b = ab & 255;
                     cx += (a == b ? ce[e] : 2.0 * ce[e]) * xe[e];
                     const T w = hx[e] - lm[e] * irho;
-                    if (d.wstore) {
-                        const int slot = d.ctl[CTL_ITER];
-                        if (slot < d.wstore_count) reinterpret_cast<T*>(d.wstore)[(size_t)slot * d.nd + off + f] = w;
-                    }
                     jac.put(a, b, w);
                     nrm += (a == b ? T(1) : T(2)) * w * w;
                 }
@@ -790,10 +786,6 @@ __global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4)) k_proj
                     }
                     hx[e] = T(xe);
                     const T w = hx[e] - lam[off + f] * irho;
-                    if (d.wstore) {
-                        const int slot = d.ctl[CTL_ITER];
-                        if (slot < d.wstore_count) reinterpret_cast<T*>(d.wstore)[(size_t)slot * d.nd + off + f] = w;
-                    }
                     jac.put(a, b, w);
                     nrm += (a == b ? T(1) : T(2)) * w * w;
                 }
@@ -805,6 +797,14 @@ __global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4)) k_proj
         if (warm) jac.rotate_into_stored(vc + d.vv_off[k], s, lane);
         jac.run(T(pa.tolrel) * sqrt(nrm), pa.max_sweeps, lane, inv_norm(nrm), UNROLLED ? 0.0f : float(kThetaSolve * pa.tolrel), warm, active);
         if (pa.warm_start) jac.store_basis(vc + d.vv_off[k], s, lane);
+        if (UNROLLED && d.estore) {  // the reverse pass takes the eigenvectors and eigenvalues from here
+            const int slot = d.ctl[CTL_ITER];
+            if (slot < d.estore_count) {
+                T* rec = reinterpret_cast<T*>(d.estore) + 2 * ((size_t)slot * d.nd + off);
+                jac.store_basis(rec, s, lane);
+                jac.eigenvalues_to(rec + s * s, s, lane);
+            }
+        }
         T lm[J::MAXE], xo[J::MAXE];  // old state, on its way during the rebuild
 #pragma unroll
         for (int e = 0; e < J::MAXE; ++e) {

@@ -465,10 +465,6 @@ __global__ void __launch_bounds__(CTAPick<T, S, VARIANT>::threads, CTAPick<T, S,
                         const double xe = d.x[ent[u]];
                         if (own[u]) cx += d.wgt[ent[u]] * d.c[ent[u]] * xe;
                         w = xe - double(v1[u]) * irho;
-                        if (d.wstore) {
-                            const int slot = d.ctl[CTL_ITER];
-                            if (slot < d.wstore_count) reinterpret_cast<T*>(d.wstore)[(size_t)slot * d.nd + off + f] = T(w);
-                        }
                     } else if (FORM == 1) {
                         w = double(v1[u]) - double(v2[u]) * irho;
                     } else if (FORM == 2) {
@@ -500,10 +496,6 @@ __global__ void __launch_bounds__(CTAPick<T, S, VARIANT>::threads, CTAPick<T, S,
                 }
                 if (d.owner[off + f]) cx += d.wgt[ent] * d.c[ent] * xe;
                 w = xe - double(c1[off + f]) * irho;
-                if (d.wstore) {
-                    const int slot = d.ctl[CTL_ITER];
-                    if (slot < d.wstore_count) reinterpret_cast<T*>(d.wstore)[(size_t)slot * d.nd + off + f] = T(w);
-                }
             } else if (FORM == 1) {
                 w = double(c1[off + f]) - double(c2[off + f]) * irho;
             } else if (FORM == 2) {

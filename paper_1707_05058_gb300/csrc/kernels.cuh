@@ -62,10 +62,13 @@ struct Dev {
     const int* vv_off;    // [p+1] offsets into vcache
     const unsigned char* owner;  // [nd] 1 at the first packed position of each pattern entry
     const double* a_valu; // [nnzA] A_ie unweighted, CSR by rows (reverse pass)
-    void* wstore;         // when set, primal projections record W of iteration n at wstore + n * nd
+    // when set, the unrolled projections record the eigendecomposition of iteration
+    // n: per clique its s^2 eigenvector entries (column by column) and s eigenvalues,
+    // 2 packed sizes, at 2 (n nd + packed offset)
+    void* estore;
     const int* lent;      // [nlong] entries in more than kLongList cliques
     int nlong;
-    int wstore_count;     // iterations that fit in wstore
+    int estore_count;     // iterations that fit in estore
     double* part;         // [p * PART_COLS] per-clique partial sums
     double* parte;        // [NBLK_E * PART_COLS] per-block partials, pattern-entry kernels
     double* partr;        // [NBLK_R * PART_COLS] per-block partials, constraint-row kernels

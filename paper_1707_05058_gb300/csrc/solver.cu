@@ -261,7 +261,7 @@ void make_dev(cdsdp* h) {
     d.wgt = (const double*)(w + L.wgt);
     d.a_ptr = (const int*)(w + L.a_ptr); d.a_col = (const int*)(w + L.a_col); d.a_valw = (const double*)(w + L.a_valw);
     d.a_valu = (const double*)(w + L.a_valu);
-    d.wstore = nullptr; d.wstore_count = 0;
+    d.estore = nullptr; d.estore_count = 0;
     d.at_ptr = (const int*)(w + L.at_ptr); d.at_col = (const int*)(w + L.at_col); d.at_val = (const double*)(w + L.at_val);
     d.b = (const double*)(w + L.b); d.minv = (const double*)(w + L.minv); d.kinv = (const double*)(w + L.kinv);
     d.gmap = (const int*)(w + L.gmap); d.pk_off = (const int*)(w + L.pk_off); d.csize = (const int*)(w + L.csize);
@@ -737,7 +737,7 @@ int copy_results(cdsdp* h, cudaStream_t st, double* X, double* y, double* Z, dou
 // ---- differentiation through unrolled Algorithm 1 -------------------------
 
 struct GradLayout {
-    size_t ckpt, wstore, xkbar, lambar, hxbar, lamprev, xbar, u, sbar, ybar, rbar, total;
+    size_t ckpt, estore, xkbar, lambar, hxbar, lamprev, xbar, u, sbar, ybar, rbar, total;
     int nseg;
 };
 
@@ -748,7 +748,7 @@ GradLayout make_grad_layout(const Dev& d, int iters, int ckpt_every, bool fp32) 
     const size_t ts = fp32 ? 4 : 8, nd = d.nd, NE = d.NE, m = d.m;
     G.nseg = (iters + ckpt_every - 1) / ckpt_every;
     G.ckpt = take((size_t)G.nseg * 2 * nd * ts);
-    G.wstore = take((size_t)ckpt_every * nd * ts);
+    G.estore = take((size_t)ckpt_every * 2 * nd * ts);
     G.xkbar = take(nd * 8); G.lambar = take(nd * 8); G.hxbar = take(nd * 8); G.lamprev = take(nd * 8);
     G.xbar = take(NE * 8); G.u = take(NE * 8); G.sbar = take(NE * 8);
     G.ybar = take(m * 8); G.rbar = take(m * 8);
@@ -1570,8 +1570,8 @@ int cdsdp_unrolled_backward(cdsdp* h, const cdsdp_opts* opts, int iters, int ckp
     dd.c = d_c;
     dd.b = d_b;
     dd.max_iter = ckpt_every;
-    dd.wstore = g + G.wstore;
-    dd.wstore_count = ckpt_every;
+    dd.estore = g + G.estore;
+    dd.estore_count = ckpt_every;
     dd.comp_mode = 0;
     const size_t ts = fp32 ? 4 : 8, nd = dd.nd;
     double* xkbar = (double*)(g + G.xkbar);
@@ -1593,14 +1593,14 @@ int cdsdp_unrolled_backward(cdsdp* h, const cdsdp_opts* opts, int iters, int ckp
     const int GN = std::max(1, std::min(NBLK_E, (dd.nd + ETHREADS - 1) / ETHREADS));
     GradArgs ga;
     ga.xkbar = xkbar; ga.lambar = lambar; ga.hxbar = hxbar; ga.lamprev = lamprev;
-    ga.rho = o.rho; ga.tolrel = 0.0; ga.max_sweeps = o.jacobi_max_sweeps;
+    ga.rho = o.rho;
     for (int sg = G.nseg - 1; sg >= 0; --sg) {
         unsigned char* ck = g + G.ckpt + (size_t)sg * 2 * nd * ts;
         CK(cudaMemsetAsync(h->ws + h->L.const_end, 0, h->L.total - h->L.const_end, st));
         CK(cudaMemcpyAsync(dd.ck0, ck, nd * ts, cudaMemcpyDeviceToDevice, st));
         CK(cudaMemcpyAsync(dd.ck1, ck + nd * ts, nd * ts, cudaMemcpyDeviceToDevice, st));
         const int len = std::min(ckpt_every, iters - sg * ckpt_every);
-        rc = run_segment(h, dd, o, len, st);  // replay, recording W of every iteration
+        rc = run_segment(h, dd, o, len, st);  // replay, recording every eigendecomposition
         if (rc != CDSDP_SOLVED) return rc;
         for (int n = len - 1; n >= 0; --n) {
             ga.slot = n;
