@@ -458,7 +458,7 @@ int cdsdp_psd_project(int p, const int* d_off, const int* d_size, int max_size,
  * for both entries) and b (m values) given on the device.  The forward stores
  * the clique state every `ckpt_every` iterations in the caller-owned device
  * buffer d_gws (cdsdp_grad_workspace_bytes); the backward replays each
- * segment from its checkpoint, recording the projection inputs, and runs the
+ * segment from its checkpoint, recording the eigendecompositions, and runs the
  * reverse pass: the Daleckii-Krein adjoint of every clique projection on the
  * GPU (eigenpairs recomputed by the same Jacobi), the linear steps transposed.
  * Warm start is off and the solve never stops early, so the replay repeats

@@ -459,7 +459,8 @@ cudaError_t launch_iteration(cdsdp* h, int form, const cdsdp_opts& o, cudaStream
                              cudaGraphConditionalHandle hnd, cudaEvent_t ev0, cudaEvent_t ev1) {
     Dev& d = h->dev;
     // Algorithm 2's v and lambda: a block per clique where all of them fit the chip
-    // at once and have more entries than a warp takes at a time, else a warp
+    // at once and have more entries than a warp takes at a time (100 cliques of
+    // order 30: 34.6 us with a warp each, 25.8 with a block), else a warp
     const int whole = d.p <= 152 * 4 && (long long)d.nd > 256LL * d.p;
     const int GE = h->GE, GR = h->GR, PG = whole ? std::max(1, d.p) : std::max(1, std::min((d.p + 3) / 4, 152 * 32));
     FinishArgs fa;
