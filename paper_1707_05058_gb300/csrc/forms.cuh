@@ -356,14 +356,14 @@ __global__ void __launch_bounds__(RTHREADS) k_hsde_sigma21(Dev d, int TPR, int n
 // The same update per independent component, each with its own embedding
 // (component mode): gamma_c = zeta_c^T sigma over the component's entries and
 // rows, then tau_c, kappa_c and the new u_y of the component's rows.  Block
-// (i, c) of the grid takes the i-th part of component c's entries; the last of
+// (c, i) of the grid takes the i-th part of component c's entries; the last of
 // a component's blocks to arrive adds the parts in order.  (One block per
 // component read 47,000 entries by itself, 266 us a launch on a batch of eight;
 // with this and the test below split, 48 iterations went from 41.0 to 23.8 ms.)
 __global__ void __launch_bounds__(256) k_hsde_gamma_components(Dev d) {
     __shared__ double sh[32 * 2];
     if (stopped(d)) return;
-    const int c = blockIdx.y, part = blockIdx.x, np = gridDim.x;
+    const int c = blockIdx.x, part = blockIdx.y, np = gridDim.y;
     if (d.comp_done[c]) return;
     double v[2] = {0.0, 0.0};
     const int p0 = d.cent_ptr[c], len = d.cent_ptr[c + 1] - p0;
@@ -583,7 +583,7 @@ __device__ void finish_hsde_block(const Dev& d, const FinishArgs& fa) {
 // tau, kappa and norms of b and c.  A component that passes, proves
 // infeasibility, reaches max_iter or meets a NaN is frozen from the next
 // iteration on; the block that arrives last sets the global state.  Block
-// (i, c) of the grid takes the i-th part of the component's entries (and the
+// (c, i) of the grid takes the i-th part of the component's entries (and the
 // first one its cliques and rows), the last of a component's blocks adds the
 // parts in order and runs the test (181 us a launch with one block per
 // component on a batch of eight).
@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(256) k_finish_hsde_components(Dev d, FinishArg
     __shared__ double sh[32 * 10];
     __shared__ int s_was_done;
     if (stopped(d)) return;
-    const int c = blockIdx.y, part = blockIdx.x, np = gridDim.x;
+    const int c = blockIdx.x, part = blockIdx.y, np = gridDim.y;
     const int it = d.ctl[CTL_ITER] + 1;
     if (threadIdx.x == 0) s_was_done = d.comp_done[c];
     __syncthreads();

@@ -306,14 +306,15 @@ __device__ __forceinline__ bool last_block_single_writer(const Dev& d) {
     return s_last1 != 0;
 }
 
-// The same among the gridDim.x blocks of one component (block (., c) of the
-// grid); the counter returns to zero.
+// The same among the gridDim.y blocks of one component (block (c, .) of the
+// grid: components lie along x, whose limit no problem reaches; y ends at
+// 65,535); the counter returns to zero.
 __device__ __forceinline__ bool last_block_of_component(const Dev& d, int c) {
     __shared__ int s_last2;
     if (threadIdx.x == 0) {
         __threadfence();
         const int ticket = atomicAdd(d.comp_cnt + c, 1);
-        s_last2 = (ticket == (int)gridDim.x - 1) ? 1 : 0;
+        s_last2 = (ticket == (int)gridDim.y - 1) ? 1 : 0;
         if (s_last2) {
             d.comp_cnt[c] = 0;
             __threadfence();

@@ -517,7 +517,7 @@ cudaError_t launch_iteration(cdsdp* h, int form, const cdsdp_opts& o, cudaStream
         k_gemv<<<GR, RTHREADS, 0, st>>>(d, d.kinv, d.g, d.hh, -1, h->TPRM);
         k_hsde_sigma11<<<GE, ETHREADS, 0, st>>>(d, h->Gx);
         k_hsde_sigma21<<<GR, RTHREADS, 0, st>>>(d, h->TPR, GE);
-        if (d.comp_mode) k_hsde_gamma_components<<<dim3(h->hs_parts, d.ncomp), 256, 0, st>>>(d);
+        if (d.comp_mode) k_hsde_gamma_components<<<dim3(d.ncomp, h->hs_parts), 256, 0, st>>>(d);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if (ev0) cudaEventRecord(ev0, st);
         FinishArgs none = fa;
@@ -526,7 +526,7 @@ cudaError_t launch_iteration(cdsdp* h, int form, const cdsdp_opts& o, cudaStream
         if (ev1) cudaEventRecord(ev1, st);
         k_hsde_entry_update<T><<<GE, ETHREADS, 0, st>>>(d, h->Gx);
         k_hsde_row_update<<<GR, RTHREADS, 0, st>>>(d, fa);
-        if (d.comp_mode) k_finish_hsde_components<<<dim3(h->hs_parts, d.ncomp), 256, 0, st>>>(d, fa);
+        if (d.comp_mode) k_finish_hsde_components<<<dim3(d.ncomp, h->hs_parts), 256, 0, st>>>(d, fa);
     }
     return cudaGetLastError();
 }
