@@ -66,18 +66,39 @@ constexpr size_t kMaxWarpSmem = 200 * 1024;  // largest shared block per warp of
 inline size_t align_up(size_t x) { return (x + kCmpAlign - 1) / kCmpAlign * kCmpAlign; }
 
 // Scratch layout (byte offsets, all 256-aligned).  The index section [0, idx_end)
-// is copied from the host image; the rest is written by the kernels.
+// is copied from the host image; [idx_end, base_total) is written by the kernels.
+// The tables of k_cmp_rows follow, from row_begin: they are built and copied
+// only where it runs, for a dense result on a full profile, and a scratch that
+// ends before them is served by k_cmp_step.
 struct CmpLayout {
-    size_t lt_ptr, lt_idx, colptr, prow, pcol, comp, loc, posl, peo_cat, peo_off, woff, lt_pos, lt_loc, first, rowblk,
-        idx_end;
-    size_t T, schur, logdet, flag, total;
-    int smax = 0, ncomp = 0, maxnc = 0;
-    int nrowblk = 0;       // blocks of k_cmp_rows
-    bool profile = false;  // full profile: rows are independent
-    long long welems = 0;
+    size_t lt_ptr, lt_idx, colptr, prow, pcol, comp, loc, posl, peo_cat, peo_off, woff, idx_end;
+    size_t T, schur, logdet, flag, base_total;
+    size_t row_begin, lt_pos, lt_loc, first, rowblk, total;
+    int smax = 0;
+    int nrowblk = 0;  // blocks of k_cmp_rows
 };
 
-CmpLayout cmp_layout(const HostProblem& hp) {
+// Vertices of each component, ascending (local index) and in elimination order,
+// and the offsets of the components' dense blocks.
+struct CmpOrder {
+    std::vector<int> cnt, loc, posl, peo_cat, peo_off;
+    std::vector<long long> woff;
+    int maxnc = 0;
+};
+
+// Offsets of the components' dense blocks, and the largest component.
+void block_offsets(const HostProblem& hp, CmpOrder& o) {
+    const int C = hp.ncomp;
+    o.cnt.assign(C, 0);
+    for (int v = 0; v < hp.n; ++v) ++o.cnt[hp.comp_of_vertex[v]];
+    o.woff.assign(C + 1, 0);
+    for (int c = 0; c < C; ++c) {
+        o.woff[c + 1] = o.woff[c] + (long long)o.cnt[c] * o.cnt[c];
+        o.maxnc = std::max(o.maxnc, o.cnt[c]);
+    }
+}
+
+CmpLayout cmp_layout(const HostProblem& hp, const CmpOrder& ord) {
     CmpLayout L;
     const size_t n = hp.n, NE = hp.prow.size(), nl = hp.lt_idx.size(), C = hp.ncomp;
     size_t o = 0;
@@ -93,27 +114,24 @@ CmpLayout cmp_layout(const HostProblem& hp) {
     L.peo_cat = take(n * 4);
     L.peo_off = take((C + 1) * 4);
     L.woff = take(C * 8);
-    std::vector<int> cnt(C, 0);
-    for (int v = 0; v < hp.n; ++v) ++cnt[hp.comp_of_vertex[v]];
-    for (int nc : cnt) L.nrowblk += (nc + kRowWarps * kRowsPerWarp - 1) / (kRowWarps * kRowsPerWarp);
-    L.lt_pos = take(nl * 4);
-    L.lt_loc = take(nl * 4);
-    L.first = take(n * 4);
-    L.rowblk = take((size_t)L.nrowblk * 8);
     L.idx_end = o;
     L.T = take(nl * 8);
     L.schur = take(n * 8);
     L.logdet = take(C * 8);
     L.flag = take(16);
+    L.base_total = L.row_begin = o;
+    for (int nc : ord.cnt) L.nrowblk += (nc + kRowWarps * kRowsPerWarp - 1) / (kRowWarps * kRowsPerWarp);
+    L.lt_pos = take(nl * 4);
+    L.lt_loc = take(nl * 4);
+    L.first = take(n * 4);
+    L.rowblk = take((size_t)L.nrowblk * 8);
     L.total = o;
-    L.ncomp = (int)C;
     for (int v = 0; v < hp.n; ++v) L.smax = std::max(L.smax, hp.lt_ptr[v + 1] - hp.lt_ptr[v]);
     return L;
 }
 
-// Host image of the index section, and the per-component block offsets.
-void cmp_image(const HostProblem& hp, CmpLayout& L, std::vector<unsigned char>& img,
-               std::vector<long long>& woff_out, int& maxnc) {
+// Host image of the index section.
+void cmp_image(const HostProblem& hp, const CmpLayout& L, CmpOrder& ord, std::vector<unsigned char>& img) {
     const int n = hp.n, C = hp.ncomp;
     img.assign(L.idx_end, 0);
     auto put = [&](size_t off, const void* src, size_t bytes) { if (bytes) std::memcpy(img.data() + off, src, bytes); };
@@ -123,59 +141,63 @@ void cmp_image(const HostProblem& hp, CmpLayout& L, std::vector<unsigned char>& 
     put(L.prow, hp.prow.data(), hp.prow.size() * 4);
     put(L.pcol, hp.pcol.data(), hp.pcol.size() * 4);
     put(L.comp, hp.comp_of_vertex.data(), n * 4);
-    // vertices of each component: ascending (local index) and in elimination order
-    std::vector<int> cnt(C + 1, 0), loc(n), posl(n), peo_cat(n);
-    for (int v = 0; v < n; ++v) loc[v] = cnt[hp.comp_of_vertex[v]]++;
-    std::vector<int> peo_off(C + 1, 0);
-    for (int c = 0; c < C; ++c) peo_off[c + 1] = peo_off[c] + cnt[c];
-    std::vector<int> fill(peo_off.begin(), peo_off.end() - 1);
+    ord.loc.resize(n);
+    ord.posl.resize(n);
+    ord.peo_cat.resize(n);
+    ord.peo_off.assign(C + 1, 0);
+    for (int c = 0; c < C; ++c) ord.peo_off[c + 1] = ord.peo_off[c] + ord.cnt[c];
+    std::vector<int> fill(C, 0);
+    for (int v = 0; v < n; ++v) ord.loc[v] = fill[hp.comp_of_vertex[v]]++;
+    std::fill(fill.begin(), fill.end(), 0);
     for (int k = 0; k < n; ++k) {
         const int v = hp.peo[k], c = hp.comp_of_vertex[v];
-        posl[v] = fill[c] - peo_off[c];
-        peo_cat[fill[c]++] = v;
+        ord.posl[v] = fill[c]++;
+        ord.peo_cat[ord.peo_off[c] + ord.posl[v]] = v;
     }
-    woff_out.assign(C + 1, 0);
-    maxnc = 0;
-    for (int c = 0; c < C; ++c) {
-        woff_out[c + 1] = woff_out[c] + (long long)cnt[c] * cnt[c];
-        maxnc = std::max(maxnc, cnt[c]);
-    }
-    put(L.loc, loc.data(), n * 4);
-    put(L.posl, posl.data(), n * 4);
-    put(L.peo_cat, peo_cat.data(), n * 4);
-    put(L.peo_off, peo_off.data(), (C + 1) * 4);
-    put(L.woff, woff_out.data(), C * 8);
-    // k_cmp_rows: elimination position and local index of every later
-    // neighbour; per position, the first position whose list holds it (itself
-    // when none does); the row blocks, longest chains first
-    std::vector<int> lpos(hp.lt_idx.size()), lloc(hp.lt_idx.size()), first(n), seen(n, 0);
+    put(L.loc, ord.loc.data(), n * 4);
+    put(L.posl, ord.posl.data(), n * 4);
+    put(L.peo_cat, ord.peo_cat.data(), n * 4);
+    put(L.peo_off, ord.peo_off.data(), (C + 1) * 4);
+    put(L.woff, ord.woff.data(), C * 8);
+}
+
+// Whether the pattern has a full profile, and then the image of the tables of
+// k_cmp_rows (scratch offsets row_begin .. total): elimination position and
+// local index of every later neighbour; per position, the first position whose
+// list holds it (itself when none does); the row blocks, longest chains first.
+bool cmp_row_tables(const HostProblem& hp, const CmpLayout& L, const CmpOrder& ord, std::vector<unsigned char>& img) {
+    const int n = hp.n, C = hp.ncomp;
+    const std::vector<int>& peo_off = ord.peo_off;
+    std::vector<int> first(n), seen(n, 0);
     for (int c = 0; c < C; ++c)
         for (int q = peo_off[c]; q < peo_off[c + 1]; ++q) first[q] = q - peo_off[c];
     for (int k = 0; k < n; ++k) {
-        const int v = hp.peo[k], q0 = peo_off[hp.comp_of_vertex[v]];
+        const int v = hp.peo[k], q0 = peo_off[hp.comp_of_vertex[v]], p = ord.posl[v];
         for (int e = hp.lt_ptr[v]; e < hp.lt_ptr[v + 1]; ++e) {
-            const int u = hp.lt_idx[e], qu = q0 + posl[u];
-            lpos[e] = posl[u];
-            lloc[e] = loc[u];
-            first[qu] = std::min(first[qu], posl[v]);
+            const int qu = q0 + ord.posl[hp.lt_idx[e]];
+            first[qu] = std::min(first[qu], p);
             ++seen[qu];
         }
     }
-    L.profile = true;
     for (int c = 0; c < C; ++c)
         for (int q = peo_off[c]; q < peo_off[c + 1]; ++q)
-            if (seen[q] != (q - peo_off[c]) - first[q]) L.profile = false;
+            if (seen[q] != (q - peo_off[c]) - first[q]) return false;
+    img.assign(L.total - L.row_begin, 0);
+    int* lpos = reinterpret_cast<int*>(img.data() + (L.lt_pos - L.row_begin));
+    int* lloc = reinterpret_cast<int*>(img.data() + (L.lt_loc - L.row_begin));
+    for (size_t e = 0; e < hp.lt_idx.size(); ++e) {
+        lpos[e] = ord.posl[hp.lt_idx[e]];
+        lloc[e] = ord.loc[hp.lt_idx[e]];
+    }
+    std::memcpy(img.data() + (L.first - L.row_begin), first.data(), (size_t)n * 4);
     std::vector<std::pair<int, int>> blk;  // (component, first row position)
     for (int c = 0; c < C; ++c)
-        for (int r = 0; r < cnt[c]; r += kRowWarps * kRowsPerWarp) blk.emplace_back(c, r);
+        for (int r = 0; r < ord.cnt[c]; r += kRowWarps * kRowsPerWarp) blk.emplace_back(c, r);
     std::stable_sort(blk.begin(), blk.end(),
                      [](const std::pair<int, int>& a, const std::pair<int, int>& b) { return a.second > b.second; });
-    std::vector<int> flat;
-    for (const auto& b : blk) { flat.push_back(b.first); flat.push_back(b.second); }
-    put(L.lt_pos, lpos.data(), lpos.size() * 4);
-    put(L.lt_loc, lloc.data(), lloc.size() * 4);
-    put(L.first, first.data(), n * 4);
-    put(L.rowblk, flat.data(), flat.size() * 4);
+    int* flat = reinterpret_cast<int*>(img.data() + (L.rowblk - L.row_begin));
+    for (const auto& b : blk) { *flat++ = b.first; *flat++ = b.second; }
+    return true;
 }
 
 // Pattern value of entry (i, j): binary search of max(i, j) among the rows of
@@ -349,7 +371,7 @@ __global__ void __launch_bounds__(kStepThreads) k_cmp_step(int n, int r, const i
 // and two shuffles, 0.4 us a step), not bandwidth: 8 n^2 bytes are written
 // once.  4 lanes a row and 16 rows a block put a chain on nearly every SM at
 // n = 2000 (125 blocks).  Banded n = 2000, w = 10, whole call: 8.73 ms as
-// 1999 dependent launches of k_cmp_step, 1.13 ms with this kernel (0.80 ms of
+// 1999 dependent launches of k_cmp_step, 1.03 ms with this kernel (0.80 ms of
 // it here).  A row past an element's position may read an entry of the dense
 // block that nothing has written: by the profile property it is never used.
 struct RowArgs {
@@ -526,14 +548,11 @@ void completion_release(CmpGraph& g) {
 }
 
 int completion_sizes(const HostProblem& hp, size_t* scratch_bytes, long long* w_elems, long long* w_offsets) {
-    CmpLayout L = cmp_layout(hp);
-    std::vector<unsigned char> img;
-    std::vector<long long> woff;
-    int maxnc = 0;
-    cmp_image(hp, L, img, woff, maxnc);
-    if (scratch_bytes) *scratch_bytes = L.total;
-    if (w_elems) *w_elems = woff[hp.ncomp];
-    if (w_offsets) std::copy(woff.begin(), woff.end(), w_offsets);
+    CmpOrder ord;
+    block_offsets(hp, ord);
+    if (scratch_bytes) *scratch_bytes = cmp_layout(hp, ord).total;
+    if (w_elems) *w_elems = ord.woff[hp.ncomp];
+    if (w_offsets) std::copy(ord.woff.begin(), ord.woff.end(), w_offsets);
     return CDSDP_SOLVED;
 }
 
@@ -541,15 +560,16 @@ int completion_run(const HostProblem& hp, const double* d_X, void* d_scratch, si
                    double* logdet, void* stream, std::string* err, CmpGraph* cache) {
     if (!d_X || !d_scratch) return CDSDP_ERR_ARG;
     if (reinterpret_cast<uintptr_t>(d_scratch) % kCmpAlign) return CDSDP_ERR_ARG;
-    CmpLayout L = cmp_layout(hp);
-    if (scratch_bytes < L.total) return CDSDP_ERR_NOMEM;
+    CmpOrder ord;
+    block_offsets(hp, ord);
+    const CmpLayout L = cmp_layout(hp, ord);
+    if (scratch_bytes < L.base_total) return CDSDP_ERR_NOMEM;
     const int ld = std::max(1, L.smax);
     const size_t per_warp = (size_t)(ld * ld + 2 * ld) * sizeof(double);
     if (per_warp > kMaxWarpSmem) return CDSDP_ERR_UNSUPPORTED;
-    std::vector<unsigned char> img;
-    std::vector<long long> woff;
-    int maxnc = 0;
-    cmp_image(hp, L, img, woff, maxnc);
+    std::vector<unsigned char> img, row_img;
+    cmp_image(hp, L, ord, img);
+    const int maxnc = ord.maxnc;
     cudaStream_t st = (cudaStream_t)stream;
     unsigned char* g = (unsigned char*)d_scratch;
     const int n = hp.n, NE = (int)hp.prow.size(), C = hp.ncomp;
@@ -582,6 +602,8 @@ int completion_run(const HostProblem& hp, const double* d_X, void* d_scratch, si
     k_cmp_factor<<<(n + wpb - 1) / wpb, 32 * wpb, smem, st>>>(n, ld, wpb, lt_ptr, lt_idx, colptr, prow, d_X, T,
                                                                schur, flag);
     CMP_CK(cudaGetLastError());
+    // beside the factor kernel; a logdet alone and other patterns need no row tables
+    const bool rows = d_W && scratch_bytes >= L.total && cmp_row_tables(hp, L, ord, row_img);
     int hflag = 0;
     CMP_CK(cudaMemcpyAsync(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, st));
     CMP_CK(cudaStreamSynchronize(st));
@@ -590,6 +612,7 @@ int completion_run(const HostProblem& hp, const double* d_X, void* d_scratch, si
         return CDSDP_ERR_ARG;
     }
     if (hflag & 1) return CDSDP_NOT_PD;
+    if (rows) CMP_CK(cudaMemcpyAsync(g + L.row_begin, row_img.data(), row_img.size(), cudaMemcpyHostToDevice, st));
     k_cmp_logdet<<<C, 256, 0, st>>>(peo_cat, peo_off, schur, dlog);
     CMP_CK(cudaGetLastError());
     if (d_W) {
@@ -603,7 +626,7 @@ int completion_run(const HostProblem& hp, const double* d_X, void* d_scratch, si
                                                         dwoff, T, d_W);
             return cudaGetLastError();
         };
-        if (L.profile) {  // rows are independent: one launch
+        if (rows) {  // full profile: rows are independent, one launch
             RowArgs ra;
             ra.lt_ptr = lt_ptr;
             ra.lt_pos = (const int*)(g + L.lt_pos);
