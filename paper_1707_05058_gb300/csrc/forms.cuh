@@ -12,7 +12,11 @@ namespace cdsdp_dev {
 // columns 0-3 of the partial table.
 __device__ void finish_dual_block(const Dev& d, const FinishArgs& fa);
 
-template <typename T>
+// B entries of a lane at a time: their loads cannot pass the stores, and one after
+// the other an order-30 clique's 15 a lane took 37 us, eight at a time 25; 40,000
+// cliques of order 2 (three entries for 32 lanes) took 82 us with eight at a time,
+// the chain of one 45 (launch_vlam).
+template <typename T, int B>
 __global__ void __launch_bounds__(128) k_vlam_dual(Dev d, FinishArgs fa, int whole) {
     if (stopped(d)) return;
     __shared__ double sh[4][5];
@@ -22,9 +26,6 @@ __global__ void __launch_bounds__(128) k_vlam_dual(Dev d, FinishArgs fa, int who
     const T* z = reinterpret_cast<const T*>(d.ck0);
     T* v = reinterpret_cast<T*>(d.ck1);
     T* lam = reinterpret_cast<T*>(d.ck2);
-    // Eight of a lane's entries at a time: their loads cannot pass the stores, and
-    // one after the other an order-30 clique's 15 a lane took 37 us, so 25.
-    constexpr int B = 8;
     double acc[4] = {0, 0, 0, 0};
     for (int k = w0; k < d.p; k += nw) {
         if (frozen_clique(d, k)) continue;  // warp-uniform

@@ -454,14 +454,26 @@ void launch_cg(cdsdp* h, const cdsdp_opts& o, cudaStream_t st) {
     k_cg_finish<<<1, CG_THREADS, 0, st>>>(d, 0, h->GR);
 }
 
+// Algorithm 2's v and lambda: a block per clique where all of them fit the chip
+// at once and have more entries than a warp takes at a time (100 cliques of
+// order 30: 34.6 us with a warp each, 25.8 with a block), else a warp.
+int vlam_whole(const Dev& d) { return d.p <= 152 * 4 && (long long)d.nd > 256LL * d.p; }
+
+// Entries in flight per lane: as many as the mean clique has for it.
+template <typename T>
+void launch_vlam(const Dev& d, const FinishArgs& fa, int whole, int grid, cudaStream_t st) {
+    const long long per = d.nd / ((long long)std::max(1, d.p) * (whole ? 128 : 32));
+    if (per < 1) k_vlam_dual<T, 1><<<grid, 128, 0, st>>>(d, fa, whole);
+    else if (per < 2) k_vlam_dual<T, 2><<<grid, 128, 0, st>>>(d, fa, whole);
+    else if (per < 4) k_vlam_dual<T, 4><<<grid, 128, 0, st>>>(d, fa, whole);
+    else k_vlam_dual<T, 8><<<grid, 128, 0, st>>>(d, fa, whole);
+}
+
 template <typename T>
 cudaError_t launch_iteration(cdsdp* h, int form, const cdsdp_opts& o, cudaStream_t st, int use_cond,
                              cudaGraphConditionalHandle hnd, cudaEvent_t ev0, cudaEvent_t ev1) {
     Dev& d = h->dev;
-    // Algorithm 2's v and lambda: a block per clique where all of them fit the chip
-    // at once and have more entries than a warp takes at a time (100 cliques of
-    // order 30: 34.6 us with a warp each, 25.8 with a block), else a warp
-    const int whole = d.p <= 152 * 4 && (long long)d.nd > 256LL * d.p;
+    const int whole = vlam_whole(d);
     const int GE = h->GE, GR = h->GR, PG = whole ? std::max(1, d.p) : std::max(1, std::min((d.p + 3) / 4, 152 * 32));
     FinishArgs fa;
     fa.eps = o.eps;
@@ -509,7 +521,7 @@ cudaError_t launch_iteration(cdsdp* h, int form, const cdsdp_opts& o, cudaStream
         if (o.linear_solver == 1) launch_cg(h, o, st);
         else k_gemv<<<GR, RTHREADS, 0, st>>>(d, d.minv, d.g, d.y, 0, h->TPRM);
         k_xupd<<<GE, ETHREADS, 0, st>>>(d, d.t, d.y, d.x, h->Ga, 1);
-        k_vlam_dual<T><<<PG, 128, 0, st>>>(d, fin, whole);
+        launch_vlam<T>(d, fin, whole, PG, st);
         if (d.comp_mode) k_finish_components<<<d.ncomp, 256, 0, st>>>(d, 1, fa);
     } else {  // Algorithm 3; gamma/tau/kappa in sigma21's last block, stopping test in row_update's
         k_hsde_eta<T><<<GE, ETHREADS, 0, st>>>(d, h->Gs);
