@@ -151,7 +151,10 @@ __global__ void __launch_bounds__(ETHREADS) k_xupd(Dev d, const double* __restri
 // ---- constraint-row kernels ------------------------------------------------
 
 // out_i = (A W v)_i + delta b_i (delta / rho_i when delta_rho); Appendix A
-// item (ii): A D^-1 bhat - b.
+// item (ii): A D^-1 bhat - b.  SHORT: rows with about one term a lane, one at a
+// time (60,000 rows of one nonzero: 47 us with the empty slots of four, 38
+// without).
+template <bool SHORT>
 __global__ void __launch_bounds__(RTHREADS) k_rows_aw(Dev d, const double* __restrict__ v, double delta,
                                                       int delta_rho, double* __restrict__ out, int TPR) {
     __shared__ double sh[RTHREADS / 32];
@@ -166,8 +169,12 @@ __global__ void __launch_bounds__(RTHREADS) k_rows_aw(Dev d, const double* __res
             const int q0 = d.a_ptr[i], q1 = d.a_ptr[i + 1];
             // long rows: more in flight (409 rows of 25,710: 67 us one term at a time,
             // 48 four, 39 eight; 3,600 rows of 900: 45, 40 and 46 us)
-            s = q1 - q0 > 8 * TPR ? sparse_dot<8, true>(d.a_valw, d.a_col, v, q0 + tig, q1, TPR)
-                                  : sparse_dot<4, true>(d.a_valw, d.a_col, v, q0 + tig, q1, TPR);
+            if constexpr (SHORT) {
+                s = sparse_dot<1, true>(d.a_valw, d.a_col, v, q0 + tig, q1, TPR);
+            } else {
+                s = q1 - q0 > 8 * TPR ? sparse_dot<8, true>(d.a_valw, d.a_col, v, q0 + tig, q1, TPR)
+                                      : sparse_dot<4, true>(d.a_valw, d.a_col, v, q0 + tig, q1, TPR);
+            }
         }
         s = row_group_sum(s, TPR, sh);
         if (live && tig == 0) out[i] = s + (delta_rho ? delta / rho_row(d, i) : delta) * d.b[i];

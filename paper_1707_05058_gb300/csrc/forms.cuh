@@ -295,7 +295,8 @@ __global__ void __launch_bounds__(ETHREADS) k_hsde_eta(Dev d, int G) {
 }
 
 // sigma_11 = P^-1 eta - P^-1 A^T (I + A P^-1 A^T)^-1 A P^-1 eta (Eq. MatrixInvFlops);
-// partial <c, sigma_11> in parte[block][2].
+// partial <c, sigma_11> in parte[block][2].  SHORT: as in k_rows_aw, for columns of A.
+template <bool SHORT>
 __global__ void __launch_bounds__(ETHREADS) k_hsde_sigma11(Dev d, int G) {
     __shared__ double sh[32];
     if (stopped(d)) return;
@@ -307,7 +308,7 @@ __global__ void __launch_bounds__(ETHREADS) k_hsde_sigma11(Dev d, int G) {
         const int e = gid + it * ng;
         double s = 0.0;
         if (e < d.NE) {
-            s = sparse_dot<4, false>(d.at_val, d.at_col, d.hh, d.at_ptr[e] + lig, d.at_ptr[e + 1], G);
+            s = sparse_dot<SHORT ? 1 : 4, false>(d.at_val, d.at_col, d.hh, d.at_ptr[e] + lig, d.at_ptr[e + 1], G);
         }
         s = group_sum(s, G);
         if (e < d.NE && lig == 0 && !frozen_entry(d, e)) {
@@ -324,6 +325,7 @@ __global__ void __launch_bounds__(ETHREADS) k_hsde_sigma11(Dev d, int G) {
 // in partr[block][2]; A sigma_11 kept for the primal residual.
 __device__ void hsde_gamma_block(const Dev& d, int nbe, int nbr);
 
+template <bool SHORT>
 __global__ void __launch_bounds__(RTHREADS) k_hsde_sigma21(Dev d, int TPR, int nbe) {
     __shared__ double sh[RTHREADS / 32];
     __shared__ double sh2[32];
@@ -336,7 +338,7 @@ __global__ void __launch_bounds__(RTHREADS) k_hsde_sigma21(Dev d, int TPR, int n
         double s = 0.0;
         if (i < d.m) {
             const int q1 = d.a_ptr[i + 1];
-            s = sparse_dot<4, true>(d.a_valw, d.a_col, d.s11, d.a_ptr[i] + tig, q1, TPR);
+            s = sparse_dot<SHORT ? 1 : 4, true>(d.a_valw, d.a_col, d.s11, d.a_ptr[i] + tig, q1, TPR);
         }
         s = row_group_sum(s, TPR, sh);
         if (i < d.m && tig == 0 && !frozen_row(d, i)) {
@@ -442,7 +444,7 @@ __device__ void hsde_gamma_block(const Dev& d, int nbe, int nbr) {
 // u_x <- sigma_11 - gamma zeta_hat_x; A^T u_y (u_y is formed with gamma, once per
 // row rather than once per nonzero here);
 // partials: |A^T u_y + H^T v_z - tau c|^2 (parte col 0) and <c, u_x> (col 1).
-template <typename T>
+template <typename T, bool SHORT>
 __global__ void __launch_bounds__(ETHREADS) k_hsde_entry_update(Dev d, int G) {
     __shared__ double sh[64];
     if (stopped(d)) return;
@@ -452,7 +454,7 @@ __global__ void __launch_bounds__(ETHREADS) k_hsde_entry_update(Dev d, int G) {
     const int nloop = (d.NE + ng - 1) / ng;
     double p[2] = {0.0, 0.0};
     auto gather = [&](int e, int l, int step, double& a, double& hv) {
-        a = sparse_dot<4, false>(d.at_val, d.at_col, d.y, d.at_ptr[e] + l, d.at_ptr[e + 1], step);
+        a = sparse_dot<SHORT ? 1 : 4, false>(d.at_val, d.at_col, d.y, d.at_ptr[e] + l, d.at_ptr[e + 1], step);
         const int j1 = d.sc_ptr[e + 1];
         for (int j = d.sc_ptr[e] + l; j < j1; j += step) hv += double(vz[d.sc_idx[j]]);
     };

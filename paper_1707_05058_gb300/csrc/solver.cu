@@ -63,6 +63,7 @@ struct cdsdp {
     // per entry for scatters (Gs) and A^T rows (Ga), threads per A row (TPR)
     // and per row of the cached inverse (TPRM)
     int GE = 1, GR = 1, Gs = 1, Ga = 1, Gx = 1, TPR = 32, TPRM = 32;
+    bool short_rows = false, short_cols = false;  // rows / columns of A with about one nonzero a lane
     int hs_parts = 1;   // blocks per component of Algorithm 3's component reductions
     int TPR_auto = 32;  // TPR from the row lengths (opts.row_threads = 0)
     // Algorithm 1: compute x = t - D^-1 A^T y in its own kernel (coalesced
@@ -311,6 +312,8 @@ void make_dev(cdsdp* h) {
     h->Ga = pow2_clamp(std::max(avg_at, avg_sc) / 3.0, 1, 32);
     h->Gx = pow2_clamp(avg_at / 6.0, 1, 32);  // lanes per A^T row in the separate x-update
     h->TPR = h->TPR_auto = pow2_clamp(avg_a / 4.0, 32, RTHREADS);
+    h->short_rows = avg_a <= 32.0;
+    h->short_cols = avg_at <= 2.0;  // one lane each
     // The separate kernel forms each x_e once (in float64, whose throughput is
     // low on this GPU); inside the gather it is formed once per clique holding e.
     h->x_split_auto = true;
@@ -454,6 +457,12 @@ void launch_cg(cdsdp* h, const cdsdp_opts& o, cudaStream_t st) {
     k_cg_finish<<<1, CG_THREADS, 0, st>>>(d, 0, h->GR);
 }
 
+// g = A W v + delta b
+void launch_rows(const cdsdp* h, const Dev& d, const double* v, double delta, int delta_rho, cudaStream_t st) {
+    if (h->short_rows) k_rows_aw<true><<<h->GR, RTHREADS, 0, st>>>(d, v, delta, delta_rho, d.g, h->TPR);
+    else k_rows_aw<false><<<h->GR, RTHREADS, 0, st>>>(d, v, delta, delta_rho, d.g, h->TPR);
+}
+
 // Algorithm 2's v and lambda: a block per clique where all of them fit the chip
 // at once and have more entries than a warp takes at a time (100 cliques of
 // order 30: 34.6 us with a warp each, 25.8 with a block), else a warp.
@@ -501,7 +510,7 @@ cudaError_t launch_iteration(cdsdp* h, int form, const cdsdp_opts& o, cudaStream
     cudaError_t e;
     if (form == 0) {  // Algorithm 1; the projection computes x on the fly and its last block the stopping test
         launch_scatter<T>(h, d, (const T*)d.ck0, (const T*)d.ck1, -1.0, 1.0, 1.0, 1, 1, d.dinv, d.t, 1, st);
-        k_rows_aw<<<GR, RTHREADS, 0, st>>>(d, d.t, -1.0, 0, d.g, h->TPR);
+        launch_rows(h, d, d.t, -1.0, 0, st);
         if (o.linear_solver == 1) launch_cg(h, o, st);
         else k_gemv<<<GR, RTHREADS, 0, st>>>(d, d.minv, d.g, d.y, 0, h->TPRM);
         if (h->x_split) k_xupd<<<GE, ETHREADS, 0, st>>>(d, d.t, d.y, d.x, h->Gx, 0);
@@ -517,7 +526,7 @@ cudaError_t launch_iteration(cdsdp* h, int form, const cdsdp_opts& o, cudaStream
         if ((e = launch_projection<T>(h, 1, o, none, st)) != cudaSuccess) return e;
         if (ev1) cudaEventRecord(ev1, st);
         launch_scatter<T>(h, d, (const T*)d.ck0, (const T*)d.ck2, 1.0, -1.0, 1.0, 0, 1, d.dinv, d.t, 1, st);
-        k_rows_aw<<<GR, RTHREADS, 0, st>>>(d, d.t, 1.0, 1, d.g, h->TPR);
+        launch_rows(h, d, d.t, 1.0, 1, st);
         if (o.linear_solver == 1) launch_cg(h, o, st);
         else k_gemv<<<GR, RTHREADS, 0, st>>>(d, d.minv, d.g, d.y, 0, h->TPRM);
         k_xupd<<<GE, ETHREADS, 0, st>>>(d, d.t, d.y, d.x, h->Ga, 1);
@@ -525,10 +534,12 @@ cudaError_t launch_iteration(cdsdp* h, int form, const cdsdp_opts& o, cudaStream
         if (d.comp_mode) k_finish_components<<<d.ncomp, 256, 0, st>>>(d, 1, fa);
     } else {  // Algorithm 3; gamma/tau/kappa in sigma21's last block, stopping test in row_update's
         k_hsde_eta<T><<<GE, ETHREADS, 0, st>>>(d, h->Gs);
-        k_rows_aw<<<GR, RTHREADS, 0, st>>>(d, d.q, 0.0, 0, d.g, h->TPR);
+        launch_rows(h, d, d.q, 0.0, 0, st);
         k_gemv<<<GR, RTHREADS, 0, st>>>(d, d.kinv, d.g, d.hh, -1, h->TPRM);
-        k_hsde_sigma11<<<GE, ETHREADS, 0, st>>>(d, h->Gx);
-        k_hsde_sigma21<<<GR, RTHREADS, 0, st>>>(d, h->TPR, GE);
+        if (h->short_cols) k_hsde_sigma11<true><<<GE, ETHREADS, 0, st>>>(d, h->Gx);
+        else k_hsde_sigma11<false><<<GE, ETHREADS, 0, st>>>(d, h->Gx);
+        if (h->short_rows) k_hsde_sigma21<true><<<GR, RTHREADS, 0, st>>>(d, h->TPR, GE);
+        else k_hsde_sigma21<false><<<GR, RTHREADS, 0, st>>>(d, h->TPR, GE);
         if (d.comp_mode) k_hsde_gamma_components<<<dim3(d.ncomp, h->hs_parts), 256, 0, st>>>(d);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if (ev0) cudaEventRecord(ev0, st);
@@ -536,7 +547,8 @@ cudaError_t launch_iteration(cdsdp* h, int form, const cdsdp_opts& o, cudaStream
         none.enabled = 0;
         if ((e = launch_projection<T>(h, 2, o, none, st)) != cudaSuccess) return e;
         if (ev1) cudaEventRecord(ev1, st);
-        k_hsde_entry_update<T><<<GE, ETHREADS, 0, st>>>(d, h->Gx);
+        if (h->short_cols) k_hsde_entry_update<T, true><<<GE, ETHREADS, 0, st>>>(d, h->Gx);
+        else k_hsde_entry_update<T, false><<<GE, ETHREADS, 0, st>>>(d, h->Gx);
         k_hsde_row_update<<<GR, RTHREADS, 0, st>>>(d, fa);
         if (d.comp_mode) k_finish_hsde_components<<<dim3(d.ncomp, h->hs_parts), 256, 0, st>>>(d, fa);
     }
