@@ -323,10 +323,10 @@ __global__ void __launch_bounds__(ETHREADS) k_hsde_sigma11(Dev d, int G) {
 
 // sigma_21 = nu_21 - A sigma_11 (Eq. AppendixEqSigma2); partial <b, sigma_21>
 // in partr[block][2]; A sigma_11 kept for the primal residual.
-__device__ void hsde_gamma_block(const Dev& d, int nbe, int nbr);
+__device__ void hsde_gamma_block(const Dev& d, int nbe, int nbr, int uy);
 
 template <bool SHORT>
-__global__ void __launch_bounds__(RTHREADS) k_hsde_sigma21(Dev d, int TPR, int nbe) {
+__global__ void __launch_bounds__(RTHREADS) k_hsde_sigma21(Dev d, int TPR, int nbe, int uy) {
     __shared__ double sh[RTHREADS / 32];
     __shared__ double sh2[32];
     if (stopped(d)) return;
@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(RTHREADS) k_hsde_sigma21(Dev d, int TPR, int n
     block_sum<1>(bs, sh2);
     if (threadIdx.x == 0) d.partr[blockIdx.x * PART_COLS + 2] = bs[0];
     if (d.comp_mode) return;  // k_hsde_gamma_components runs next, one block per component
-    if (last_block_single_writer(d)) hsde_gamma_block(d, nbe, gridDim.x);
+    if (last_block_single_writer(d)) hsde_gamma_block(d, nbe, gridDim.x, uy);
 }
 
 // The same update per independent component, each with its own embedding
@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(RTHREADS) k_hsde_sigma21(Dev d, int TPR, int n
 // a component's blocks to arrive adds the parts in order.  (One block per
 // component read 47,000 entries by itself, 266 us a launch on a batch of eight;
 // with this and the test below split, 48 iterations went from 41.0 to 23.8 ms.)
-__global__ void __launch_bounds__(256) k_hsde_gamma_components(Dev d) {
+__global__ void __launch_bounds__(256) k_hsde_gamma_components(Dev d, int uy) {
     __shared__ double sh[32 * 2];
     if (stopped(d)) return;
     const int c = blockIdx.x, part = blockIdx.y, np = gridDim.y;
@@ -408,6 +408,7 @@ __global__ void __launch_bounds__(256) k_hsde_gamma_components(Dev d) {
         d.hs_kappa[c] = kappa - tauhat + tn;
         s_gamma = gamma;
     }
+    if (!uy) return;
     __syncthreads();
     for (int j = d.crow_ptr[c] + threadIdx.x; j < d.crow_ptr[c + 1]; j += blockDim.x) {
         const int i = d.crow_idx[j];
@@ -417,9 +418,9 @@ __global__ void __launch_bounds__(256) k_hsde_gamma_components(Dev d) {
 
 // gamma = zeta^T sigma, u_hat_2 = omega_2 + zeta^T u_hat_1 = omega_2 + gamma (1 - zeta^T zeta_hat)
 // (Eqs. MatrixInverseResult, FirstBlockElimination); tau <- max(0, u_hat_tau - kappa),
-// kappa <- kappa - u_hat_tau + tau (Eqs. HsdeStep2-3 on the R_+ component); then
-// u_y <- sigma_21 - gamma zeta_hat_y.
-__device__ void hsde_gamma_block(const Dev& d, int nbe, int nbr) {
+// kappa <- kappa - u_hat_tau + tau (Eqs. HsdeStep2-3 on the R_+ component); then,
+// with uy, u_y <- sigma_21 - gamma zeta_hat_y.
+__device__ void hsde_gamma_block(const Dev& d, int nbe, int nbr, int uy) {
     __shared__ double sh[32];
     const double cs = sum_col(d.parte, nbe, 2, sh);
     const double bs = sum_col(d.partr, nbr, 2, sh);
@@ -436,13 +437,17 @@ __device__ void hsde_gamma_block(const Dev& d, int nbe, int nbr) {
         d.ctl[CTL_COUNTER] = 0;
         sh[0] = gamma;
     }
+    if (!uy) return;
     __syncthreads();
     const double gamma = sh[0];
     for (int i = threadIdx.x; i < d.m; i += blockDim.x) d.y[i] = __ldcg(d.s21 + i) - gamma * d.zhy[i];
 }
 
-// u_x <- sigma_11 - gamma zeta_hat_x; A^T u_y (u_y is formed with gamma, once per
-// row rather than once per nonzero here);
+// u_x <- sigma_11 - gamma zeta_hat_x; A^T u_y.  u_y is formed with gamma, by the
+// block that finds it: once per row rather than once per nonzero.  With SHORT
+// columns it is formed here and by k_hsde_row_update instead, since one block
+// over all rows takes 1.3 us a thousand (20,000 rows of one nonzero: 174 us an
+// iteration with it, 151 without);
 // partials: |A^T u_y + H^T v_z - tau c|^2 (parte col 0) and <c, u_x> (col 1).
 template <typename T, bool SHORT>
 __global__ void __launch_bounds__(ETHREADS) k_hsde_entry_update(Dev d, int G) {
@@ -454,7 +459,15 @@ __global__ void __launch_bounds__(ETHREADS) k_hsde_entry_update(Dev d, int G) {
     const int nloop = (d.NE + ng - 1) / ng;
     double p[2] = {0.0, 0.0};
     auto gather = [&](int e, int l, int step, double& a, double& hv) {
-        a = sparse_dot<SHORT ? 1 : 4, false>(d.at_val, d.at_col, d.y, d.at_ptr[e] + l, d.at_ptr[e + 1], step);
+        if constexpr (SHORT) {
+            const double gamma = hs_gamma_c(d, comp_e(d, e));
+            for (int q = d.at_ptr[e] + l; q < d.at_ptr[e + 1]; q += step) {
+                const int i = d.at_col[q];
+                a += d.at_val[q] * (d.s21[i] - gamma * d.zhy[i]);
+            }
+        } else {
+            a = sparse_dot<4, false>(d.at_val, d.at_col, d.y, d.at_ptr[e] + l, d.at_ptr[e + 1], step);
+        }
         const int j1 = d.sc_ptr[e + 1];
         for (int j = d.sc_ptr[e] + l; j < j1; j += step) hv += double(vz[d.sc_idx[j]]);
     };
@@ -498,11 +511,11 @@ __global__ void __launch_bounds__(ETHREADS) k_hsde_entry_update(Dev d, int G) {
     }
 }
 
-// A u_x = A sigma_11 - gamma A zeta_hat_x;
+// A u_x = A sigma_11 - gamma A zeta_hat_x; with form_uy u_y <- sigma_21 - gamma zeta_hat_y;
 // partials |A u_x - tau b|^2 (partr col 0) and <b, u_y> (col 1).
 __device__ void finish_hsde_block(const Dev& d, const FinishArgs& fa);
 
-__global__ void __launch_bounds__(RTHREADS) k_hsde_row_update(Dev d, FinishArgs fa) {
+__global__ void __launch_bounds__(RTHREADS) k_hsde_row_update(Dev d, FinishArgs fa, int form_uy) {
     __shared__ double sh[64];
     if (stopped(d)) return;
     double p[2] = {0.0, 0.0};
@@ -510,7 +523,8 @@ __global__ void __launch_bounds__(RTHREADS) k_hsde_row_update(Dev d, FinishArgs 
         if (frozen_row(d, i)) continue;
         const int c = comp_r(d, i);
         const double gamma = hs_gamma_c(d, c), tau = hs_tau_c(d, c);
-        const double uy = d.y[i];
+        const double uy = form_uy ? d.s21[i] - gamma * d.zhy[i] : d.y[i];
+        if (form_uy) d.y[i] = uy;
         const double r = d.as11[i] - gamma * d.azhx[i] - tau * d.b[i];
         p[0] += r * r;
         p[1] += d.b[i] * uy;
