@@ -949,8 +949,13 @@ __global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4)) k_proj
 // with nu_12 = u_s + v_z, nu_22 = u_t.  Partial sums for eps_c (Eq.
 // HSDEconsensusResidual): |u_s - H u_x|^2, |u_s|^2, |H u_x|^2, |v_z - u_t|^2,
 // |v_z|^2, |u_t|^2, where u_x = sigma_11 - gamma zeta_hat_x.
+// Registers bound how many warps an SM holds, and with many cliques the time: two
+// blocks an SM at float orders up to 4, 20 and 24, and an epilogue of one entry at
+// a time where it would take the registers of the sweeps (8,000 cliques: order 7
+// 137 -> 124 us an iteration, order 20 524 -> 478, order 21 681 -> 571, order 24
+// 719 -> 654).
 template <typename T, int S>
-__global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4)) k_project_hsde(Dev d, const int4* __restrict__ list, int nlist, ProjArgs pa) {
+__global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4), sizeof(T) == 4 && (S <= 4 || S == 20 || S == 24) ? 2 : 1) k_project_hsde(Dev d, const int4* __restrict__ list, int nlist, ProjArgs pa) {
     constexpr int LW = proj_lanes(S), G = 32 / LW;  // lanes per clique, cliques per warp
     using J = BLJacobi<T, S, LW>;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1011,7 +1016,8 @@ __global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4)) k_proj
         if (pa.warm_start) jac.store_basis(vc + d.vv_off[k], s, lane);
         jac.project(lane);
         double p[6] = {0, 0, 0, 0, 0, 0};
-#pragma unroll 4
+constexpr int EU = (S <= 8 || S == 20 || S == 24) ? 1 : 4;
+#pragma unroll EU
         for (int f = lane; f < npk; f += LW) {
             const int ab = packed_ab(f, s), a = ab >> 8, b = ab & 255;
             const int ent = __ldg(d.gmap + off + f);
