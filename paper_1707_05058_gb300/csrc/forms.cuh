@@ -363,10 +363,13 @@ __global__ void __launch_bounds__(RTHREADS) k_hsde_sigma21(Dev d, int TPR, int n
 // a component's blocks to arrive adds the parts in order.  (One block per
 // component read 47,000 entries by itself, 266 us a launch on a batch of eight;
 // with this and the test below split, 48 iterations went from 41.0 to 23.8 ms.)
+// Without PARTS (small components) a component has one block: 2,000 components
+// of 5 cliques took 106 us a test with the code of the parts in it, 97 without.
+template <bool PARTS>
 __global__ void __launch_bounds__(256) k_hsde_gamma_components(Dev d, int uy) {
     __shared__ double sh[32 * 2];
     if (stopped(d)) return;
-    const int c = blockIdx.x, part = blockIdx.y, np = gridDim.y;
+    const int c = blockIdx.x, part = PARTS ? blockIdx.y : 0, np = PARTS ? gridDim.y : 1;
     if (d.comp_done[c]) return;
     double v[2] = {0.0, 0.0};
     const int p0 = d.cent_ptr[c], len = d.cent_ptr[c + 1] - p0;
@@ -383,7 +386,7 @@ __global__ void __launch_bounds__(256) k_hsde_gamma_components(Dev d, int uy) {
     }
     block_sum<2>(v, sh);
     __shared__ double s_gamma;
-    if (np > 1) {  // parts in the per-block table (free here in component mode)
+    if constexpr (PARTS) {  // parts in the per-block table (free here in component mode)
         if (threadIdx.x == 0) {
             double* pr = d.parte + (size_t)(c * np + part) * PART_COLS;
             pr[0] = v[0];
@@ -604,11 +607,12 @@ __device__ void finish_hsde_block(const Dev& d, const FinishArgs& fa) {
 // first one its cliques and rows), the last of a component's blocks adds the
 // parts in order and runs the test (181 us a launch with one block per
 // component on a batch of eight).
+template <bool PARTS>
 __global__ void __launch_bounds__(256) k_finish_hsde_components(Dev d, FinishArgs fa) {
     __shared__ double sh[32 * 10];
     __shared__ int s_was_done;
     if (stopped(d)) return;
-    const int c = blockIdx.x, part = blockIdx.y, np = gridDim.y;
+    const int c = blockIdx.x, part = PARTS ? blockIdx.y : 0, np = PARTS ? gridDim.y : 1;
     const int it = d.ctl[CTL_ITER] + 1;
     if (threadIdx.x == 0) s_was_done = d.comp_done[c];
     __syncthreads();
@@ -633,7 +637,7 @@ __global__ void __launch_bounds__(256) k_finish_hsde_components(Dev d, FinishArg
         }
         block_sum<10>(v, sh);
     }
-    if (np > 1) {  // parts in the per-block tables (free here in component mode)
+    if constexpr (PARTS) {  // parts in the per-block tables (free here in component mode)
         if (threadIdx.x == 0) {
             double* pr = d.parte + (size_t)(c * np + part) * PART_COLS;
             pr[0] = v[6];

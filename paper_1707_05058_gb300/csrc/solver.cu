@@ -541,7 +541,8 @@ cudaError_t launch_iteration(cdsdp* h, int form, const cdsdp_opts& o, cudaStream
         const int uy = h->short_cols ? 0 : 1;  // u_y with gamma, else per nonzero and in the row update
         if (h->short_rows) k_hsde_sigma21<true><<<GR, RTHREADS, 0, st>>>(d, h->TPR, GE, uy);
         else k_hsde_sigma21<false><<<GR, RTHREADS, 0, st>>>(d, h->TPR, GE, uy);
-        if (d.comp_mode) k_hsde_gamma_components<<<dim3(d.ncomp, h->hs_parts), 256, 0, st>>>(d, uy);
+        if (d.comp_mode && h->hs_parts > 1) k_hsde_gamma_components<true><<<dim3(d.ncomp, h->hs_parts), 256, 0, st>>>(d, uy);
+        else if (d.comp_mode) k_hsde_gamma_components<false><<<d.ncomp, 256, 0, st>>>(d, uy);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if (ev0) cudaEventRecord(ev0, st);
         FinishArgs none = fa;
@@ -551,7 +552,8 @@ cudaError_t launch_iteration(cdsdp* h, int form, const cdsdp_opts& o, cudaStream
         if (h->short_cols) k_hsde_entry_update<T, true><<<GE, ETHREADS, 0, st>>>(d, h->Gx);
         else k_hsde_entry_update<T, false><<<GE, ETHREADS, 0, st>>>(d, h->Gx);
         k_hsde_row_update<<<GR, RTHREADS, 0, st>>>(d, fa, !uy);
-        if (d.comp_mode) k_finish_hsde_components<<<dim3(d.ncomp, h->hs_parts), 256, 0, st>>>(d, fa);
+        if (d.comp_mode && h->hs_parts > 1) k_finish_hsde_components<true><<<dim3(d.ncomp, h->hs_parts), 256, 0, st>>>(d, fa);
+        else if (d.comp_mode) k_finish_hsde_components<false><<<d.ncomp, 256, 0, st>>>(d, fa);
     }
     return cudaGetLastError();
 }
