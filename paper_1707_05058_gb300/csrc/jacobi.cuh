@@ -152,18 +152,23 @@ __device__ __forceinline__ void rotation(double app, double aqq, double apq, dou
 }
 
 // The same rotation through tan(theta) (Rutishauser's form of the 2x2 Schur
-// step), for the unrolled passes: a derivative through the projections jumps
+// step), for the smallest orders, where few rotations make each one's rounding
+// show: 1,024 random blocks of order 2, 3 and 4 came out 0.81, 1.44 and 1.85
+// u ||W||_F off with the half-angle form in float and 0.69, 1.38 and 1.78 with
+// this one (order 5: 2.21 and 2.28); in double order 2 0.77 and 0.68, since an
+// angle in float32 takes it two rotations, and no difference above.  And, with
+// sc = 1, for the unrolled passes: a derivative through the projections jumps
 // where an eigenvalue changes sign, so gradients are only comparable between
 // builds while the projections round alike, and these kept their arithmetic
 // when the half-angle form above replaced it in the solves.
 template <typename T>
-__device__ __forceinline__ void rotation_tan(T app, T aqq, T apq, T tol, T& tau, T& sn, T& ta) {
+__device__ __forceinline__ void rotation_tan(T app, T aqq, T apq, T tol, T sc, T& tau, T& sn, T& ta) {
     tau = T(0); sn = T(0); ta = T(0);
     if (fabs(apq) > tol) {
-        const T zeta = T(0.5) * (aqq - app);
-        const T r2 = zeta * zeta + apq * apq;
+        const T zeta = T(0.5) * (aqq - app) * sc, q = apq * sc;
+        const T r2 = zeta * zeta + q * q;
         const T r = r2 * rsqrt_t<T>(r2);
-        const T tt = copysign(T(1), zeta) * div_t<T>(apq, fabs(zeta) + r);
+        const T tt = copysign(T(1), zeta) * div_t<T>(q, fabs(zeta) + r);
         const T c = rsqrt_t<T>(T(1) + tt * tt);
         sn = tt * c;
         tau = div_t<T>(sn, T(1) + c);
@@ -240,6 +245,7 @@ struct BLJacobi {
     static_assert(LW == 32 || S <= LW, "row `lane` of V needs a lane per row");
     static_assert(rr_sigma_ok<S>(), "closed form of sigma");
     using RR = RoundRobin<S>;
+    static constexpr bool EXACT = TAN || S <= (sizeof(T) == 4 ? 4 : 2);  // rotation_tan
     static constexpr int K = S / 2;
     static constexpr int R = S - 1;
     // row pitch: rows start on 16 bytes and eight consecutive rows read as
@@ -523,10 +529,10 @@ struct BLJacobi {
         if (V_STEP) rotate_v<1 - B>(vin, vout);
         // rotation of pair `lane` (lanes < K own the diagonal blocks in slot 0)
         T tau, sn, ta;
-        if (TAN) rotation_tan(bv[0][0], bv[0][3], bv[0][1], tol, tau, sn, ta);
+        if constexpr (EXACT) rotation_tan(bv[0][0], bv[0][3], bv[0][1], tol, TAN ? T(1) : sc, tau, sn, ta);
         else rotation(bv[0][0], bv[0][3], bv[0][1], tol, sc, tau, sn, ta);
         if (lane < K) rot[B * K + lane] = P2{tau, sn};
-        const bool schur = (TAN || sizeof(T) == 4) && lane < K && sn != T(0);
+        const bool schur = (EXACT || sizeof(T) == 4) && lane < K && sn != T(0);
 #pragma unroll
         for (int t = 0; t < NS; ++t) {
             const int I = bI[t] >= 0 ? bI[t] : 0, J = bJ[t];
@@ -541,7 +547,7 @@ struct BLJacobi {
             T o01 = r01 + sJ * (r00 - uJ * r01);
             T o10 = r10 - sJ * (r11 + uJ * r10);
             T o11 = r11 + sJ * (r10 - uJ * r11);
-            if (t == 0) {  // float32 diagonal block: the 2x2 Schur result
+            if (t == 0) {  // diagonal block whose angle is exact to T: the 2x2 Schur result
                 o00 = schur ? bv[t][0] - ta : o00;
                 o11 = schur ? bv[t][3] + ta : o11;
                 o10 = schur ? T(0) : o10;
@@ -950,12 +956,12 @@ __global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4)) k_proj
 // HSDEconsensusResidual): |u_s - H u_x|^2, |u_s|^2, |H u_x|^2, |v_z - u_t|^2,
 // |v_z|^2, |u_t|^2, where u_x = sigma_11 - gamma zeta_hat_x.
 // Registers bound how many warps an SM holds, and with many cliques the time: two
-// blocks an SM at float orders up to 4, 20 and 24, and an epilogue of one entry at
+// blocks an SM at orders up to 4 and in float at 20 and 24, and an epilogue of one entry at
 // a time where it would take the registers of the sweeps (8,000 cliques: order 7
 // 137 -> 124 us an iteration, order 20 524 -> 478, order 21 681 -> 571, order 24
 // 719 -> 654).
 template <typename T, int S>
-__global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4), sizeof(T) == 4 && (S <= 4 || S == 20 || S == 24) ? 2 : 1) k_project_hsde(Dev d, const int4* __restrict__ list, int nlist, ProjArgs pa) {
+__global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4), S <= 4 || (sizeof(T) == 4 && (S == 20 || S == 24)) ? 2 : 1) k_project_hsde(Dev d, const int4* __restrict__ list, int nlist, ProjArgs pa) {
     constexpr int LW = proj_lanes(S), G = 32 / LW;  // lanes per clique, cliques per warp
     using J = BLJacobi<T, S, LW>;
     extern __shared__ __align__(16) unsigned char smem[];

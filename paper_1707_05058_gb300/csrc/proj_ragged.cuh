@@ -3,7 +3,7 @@
 // the solver makes on the host is made here by each thread block or warp.
 //
 // Orders <= 32 (k_project_ragged): a thread block takes a run of consecutive
-// batch entries, sorts them by padded order (steps of 4) with warp ballots and
+// batch entries, sorts them by padded order (2, then steps of 4) with warp ballots and
 // lets its four warps draw work items, largest orders first: one block per
 // warp above order 16, two at orders 9..16 and four up to 8 (BLJacobi's lane
 // groups).  Before, every block of the batch ran at the padded order of the
@@ -81,12 +81,12 @@ __global__ void __launch_bounds__(32 * kRaggedWarps) k_project_ragged(int p, int
     if (warp == 0) {
         const int k = blockIdx.x * run + lane;
         const int s = lane < run && k < p ? size_arr[k] : 0;
-        const int cls = s >= 1 && s <= limit ? (s + 3) / 4 : 0;  // padded order 4 cls
+        const int cls = s < 1 || s > limit ? -1 : (s <= 2 ? 0 : (s + 3) / 4);  // padded order 4 cls, or 2
         int pos0 = 0, it0 = 0;
 #pragma unroll
-        for (int c = SMAX / 4; c >= 1; --c) {
+        for (int c = SMAX / 4; c >= 0; --c) {
             const unsigned mask = __ballot_sync(0xffffffffu, cls == c);
-            const int n = __popc(mask), G = 32 / proj_lanes(4 * c);
+            const int n = __popc(mask), G = 32 / proj_lanes(c ? 4 * c : 2);
             if (cls == c) {
                 const int r = __popc(mask & ((1u << lane) - 1u));
                 entry[pos0 + r] = k;
@@ -119,6 +119,7 @@ __global__ void __launch_bounds__(32 * kRaggedWarps) k_project_ragged(int p, int
             }
         }
         switch (item_cls[it]) {
+            case 0: project_item<T, 2>(ws, ks, n, off_arr, size_arr, W, X, tolrel, max_sweeps); break;
             CDSDP_ITEM(1) CDSDP_ITEM(2) CDSDP_ITEM(3) CDSDP_ITEM(4)
         }
 #undef CDSDP_ITEM
