@@ -564,11 +564,52 @@ struct BLJacobi {
         T* tmp = X; X = Y; Y = tmp;
     }
 
+    // fro = ||W||_F and sc = 1 / ||W||_F (0 for a zero block: nothing to rotate
+    // there) from its square; sc only brings entries to order one, so in double a
+    // float32 root serves, without the hundreds of cycles of a float64 root and
+    // division.  Entries whose squares leave the range of T are scaled by the
+    // largest one first (X holds the block, or V^T W V, in both triangles): a block
+    // of entries near 1e-24 would otherwise read as a zero block.
+    __device__ __forceinline__ void norm(T nrm2, bool active, int lane, T& fro, T& sc) const {
+        if (TAN) {
+            fro = sqrt(nrm2);
+            sc = T(1);
+            return;
+        }
+        constexpr T lo = sizeof(T) == 4 ? T(1e-30) : T(1e-290), hi = sizeof(T) == 4 ? T(1e37) : T(1e290);
+        if (sizeof(T) == 8 && nrm2 > T(1e-30) && nrm2 < T(1e30)) {
+            sc = T(rsqrt_ftz(float(nrm2)));
+            fro = nrm2 * sc;
+        } else {
+            fro = sqrt(nrm2);
+            sc = nrm2 > T(0) ? T(1) / fro : T(0);
+        }
+        const bool out = active && !(nrm2 >= lo && nrm2 <= hi);
+        if (!__any_sync(0xffffffffu, out)) return;
+        T m = T(0), s = T(0);
+#pragma unroll 1
+        for (int i = lane; i < S * S; i += LW) m = fmax(m, fabs(X[(i / S) * LDA + i % S]));
+        for (int o = LW / 2; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+        // into the middle of the range in two steps, each a power of two away from overflow
+        const T up = m < T(1) ? T(sizeof(T) == 4 ? 1.329227995784916e36 : 1e250) : T(1);
+        const T dn = T(1) / (m * up);
+#pragma unroll 1
+        for (int i = lane; i < S * S; i += LW) {
+            const T x = X[(i / S) * LDA + i % S] * up * dn;
+            s += x * x;
+        }
+        for (int o = LW / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (!out || !(s > T(0)) || !(m <= T(sizeof(T) == 4 ? 3.4e38 : 1.7e308))) return;  // zero, NaN, infinite
+        const T root = sqrt(s);
+        fro = root * m;
+        sc = fmin(dn / root * up, T(sizeof(T) == 4 ? 3.4e38 : 1.7e308));
+    }
+
     // Diagonalise; returns the number of sweeps run.  Afterwards X holds the
     // (nearly) diagonal matrix and v the eigenvector row.  With v_preset the
     // sweeps start from the basis already in v (see rotate_into_stored);
     // otherwise from the identity.  A sweep runs only while some off-diagonal
-    // entry exceeds tol.  sc = 1 / ||W||_F.
+    // entry exceeds tol = tolrel ||W||_F; nrm2 = ||W||_F^2 as summed.
     //
     // theta > 0 lets the sweeps end earlier, for callers that rebuild with
     // project(): that takes the remaining off-diagonal part to first order, and
@@ -587,8 +628,11 @@ struct BLJacobi {
     // rotation skipped (threshold +inf): its storage order returns to the
     // identity after each sweep and its matrix and V stay as they were, so each
     // clique's result is the one it gets alone.
-    __device__ int run(T tol, int max_sweeps, int lane, T sc, float theta = 0.0f, bool v_preset = false,
+    __device__ int run(double tolrel, T nrm2, int max_sweeps, int lane, float theta = 0.0f, bool v_preset = false,
                        bool active = true) {
+        T fro, sc;
+        norm(nrm2, active, lane, fro, sc);
+        const T tol = T(tolrel) * fro;
         const T noise = tol * T(2 * S);  // 4 S u ||W||_F when tol = 2 u ||W||_F
         if (!v_preset) {
 #pragma unroll
@@ -686,10 +730,6 @@ struct BLJacobi {
     __device__ __forceinline__ static double gamma_across(double hi, double d) { return hi / d; }
     __device__ __forceinline__ T projected(int a, int b) const { return Y[b * LDA + a]; }
 };
-
-// 1 / ||W||_F for run(): 0 for a zero block (nothing to rotate there)
-template <typename T>
-__device__ __forceinline__ T inv_norm(T nrm2) { return nrm2 > T(0) ? T(1) / sqrt(nrm2) : T(0); }
 
 // ---------------------------------------------------------------------------
 // Algorithm 1, projection and multiplier step for every clique in `list`:
@@ -801,7 +841,7 @@ __global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4)) k_proj
         const double cxk = group_sum(cx, LW);
         __syncwarp();
         if (warm) jac.rotate_into_stored(vc + d.vv_off[k], s, lane);
-        jac.run(T(pa.tolrel) * sqrt(nrm), pa.max_sweeps, lane, inv_norm(nrm), UNROLLED ? 0.0f : float(kThetaSolve * pa.tolrel), warm, active);
+        jac.run(pa.tolrel, nrm, pa.max_sweeps, lane, UNROLLED ? 0.0f : float(kThetaSolve * pa.tolrel), warm, active);
         if (pa.warm_start) jac.store_basis(vc + d.vv_off[k], s, lane);
         if (UNROLLED && d.estore) {  // the reverse pass takes the eigenvectors and eigenvalues from here
             const int slot = d.ctl[CTL_ITER];
@@ -916,7 +956,7 @@ __global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4)) k_proj
         nrm = group_sum(nrm, LW);
         __syncwarp();
         if (warm) jac.rotate_into_stored(vc + d.vv_off[k], s, lane);
-        jac.run(T(pa.tolrel) * sqrt(nrm), pa.max_sweeps, lane, inv_norm(nrm), float(kThetaSolve * pa.tolrel), warm, active);
+        jac.run(pa.tolrel, nrm, pa.max_sweeps, lane, float(kThetaSolve * pa.tolrel), warm, active);
         if (pa.warm_start) jac.store_basis(vc + d.vv_off[k], s, lane);
         jac.project(lane);
         T p0 = 0;  // in the clique state's precision; float64 across cliques
@@ -1018,7 +1058,7 @@ __global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4), S <= 4
         nrm = group_sum(nrm, LW);
         __syncwarp();
         if (warm) jac.rotate_into_stored(vc + d.vv_off[k], s, lane);
-        jac.run(T(pa.tolrel) * sqrt(nrm), pa.max_sweeps, lane, inv_norm(nrm), float(kThetaSolve * pa.tolrel), warm, active);
+        jac.run(pa.tolrel, nrm, pa.max_sweeps, lane, float(kThetaSolve * pa.tolrel), warm, active);
         if (pa.warm_start) jac.store_basis(vc + d.vv_off[k], s, lane);
         jac.project(lane);
         double p[6] = {0, 0, 0, 0, 0, 0};
@@ -1098,7 +1138,7 @@ __global__ void __launch_bounds__(128) k_project_standalone(int p, const int* __
         nrm = warp_sum(nrm);
         __syncwarp();
         // eigenvalues or vectors asked for: diagonalise to the threshold
-        jac.run(T(tolrel) * sqrt(nrm), max_sweeps, lane, inv_norm(nrm), eig || Vout ? 0.0f : float(kThetaSolve * tolrel));
+        jac.run(tolrel, nrm, max_sweeps, lane, eig || Vout ? 0.0f : float(kThetaSolve * tolrel));
         if (eig) jac.eigenvalues_to(eig + voff[k], s, lane);
         if (Vout && lane < s) {
 #pragma unroll

@@ -59,7 +59,7 @@ __device__ __noinline__ void project_item(int smem_at, const int* ks, int count,
     }
     nrm = group_sum(nrm, LW);
     __syncwarp();
-    jac.run(T(tolrel) * sqrt(nrm), max_sweeps, lane, inv_norm(nrm), float(kThetaSolve * tolrel), false, active);
+    jac.run(tolrel, nrm, max_sweeps, lane, float(kThetaSolve * tolrel), false, active);
     jac.project(lane);
     for (int f = lane; f < npk; f += LW) {
         const int ab = packed_ab(f, s), a = ab >> 8, b = ab & 255;

@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(32 * kViolWarps) k_psd_violation(int p, const 
             }
             nrm = warp_sum(nrm);
             __syncwarp();
-            jac.run(T(tolrel) * sqrt(nrm), max_sweeps, lane, inv_norm(nrm));
+            jac.run(tolrel, nrm, max_sweeps, lane);
             double l = (lane < s) ? double(jac.X[lane * J::LDA + lane]) : 0.0;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) l = fmin(l, __shfl_xor_sync(0xffffffffu, l, o));
