@@ -245,6 +245,8 @@ struct BLJacobi {
     static_assert(LW == 32 || S <= LW, "row `lane` of V needs a lane per row");
     static_assert(rr_sigma_ok<S>(), "closed form of sigma");
     using RR = RoundRobin<S>;
+    // order 2: one rotation leaves an exact zero, so the diagonal alone is P(W)
+    static constexpr bool DIAG = TAN || S == 2;
     static constexpr bool EXACT = TAN || S <= (sizeof(T) == 4 ? 4 : 2);  // rotation_tan
     static constexpr int K = S / 2;
     static constexpr int R = S - 1;
@@ -322,8 +324,8 @@ struct BLJacobi {
         X[b * LDA + a] = w;
     }
 
-    // Largest |off-diagonal entry| of the lower triangle in X and, with sc =
-    // 1 / ||W||_F, the sum over pairs sc a_ij^2 / (|a_ii| + |a_jj|) (see run();
+    // Largest |off-diagonal entry| of the lower triangle in X and, unless DIAG, with
+    // sc = 1 / ||W||_F the sum over pairs sc a_ij^2 / (|a_ii| + |a_jj|) (see run();
     // same in all lanes of the group).
     __device__ __forceinline__ void off_diagonal(int lane, T sc, T& off, float& second) const {
         T m = T(0);
@@ -341,14 +343,16 @@ struct BLJacobi {
                 const T x = fabs(p[i * LDA + j]);
                 if (t == 0 && lane < K && e != 1) continue;  // of a diagonal block the lower entry only
                 m = fmax(m, x);
-                const float y = float(x * sc);
-                x2 += y * y * rcp_ftz(fmaxf(lr[i] + lc[j], 1.0e-30f));
+                if constexpr (!DIAG) {
+                    const float y = float(x * sc);
+                    x2 += y * y * rcp_ftz(fmaxf(lr[i] + lc[j], 1.0e-30f));
+                }
             }
         }
 #pragma unroll
         for (int o = LW / 2; o > 0; o >>= 1) {  // within the group
             m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-            x2 += __shfl_xor_sync(0xffffffffu, x2, o);
+            if constexpr (!DIAG) x2 += __shfl_xor_sync(0xffffffffu, x2, o);
         }
         off = m;
         second = x2;
@@ -647,7 +651,7 @@ struct BLJacobi {
             T off;
             float second;
             off_diagonal(lane, sc, off, second);
-            if (go && (sw >= max_sweeps || off <= tol || (!TAN && second <= theta) || (off <= noise && off > T(0.5) * prev)))
+            if (go && (sw >= max_sweeps || off <= tol || (!DIAG && second <= theta) || (off <= noise && off > T(0.5) * prev)))
                 go = false;  // converged, or stagnated at the rounding-noise level
             if (!__any_sync(0xffffffffu, go)) break;
             prev = off;
@@ -679,7 +683,7 @@ struct BLJacobi {
     // 0 between others of one sign, and max(l_i, l_j) / (|l_i| + |l_j|) across.
     // Left in Y, entry (a, b) at Y[b LDA + a] (projected()).
     __device__ __forceinline__ void project(int lane) {
-        if (TAN) {  // V max(L, 0) V^T
+        if (DIAG) {  // V max(L, 0) V^T
             T w[S];
 #pragma unroll
             for (int i = 0; i < S; ++i) {
@@ -727,7 +731,13 @@ struct BLJacobi {
     __device__ __forceinline__ static float gamma_across(float hi, float d) {
         return d > 1.0e-37f ? hi * rcp_ftz(d) : 1.0f;
     }
-    __device__ __forceinline__ static double gamma_across(double hi, double d) { return hi / d; }
+    // F is at most about 1e-8 ||W||_F here, so 1e-14 of the quotient is enough
+    __device__ __forceinline__ static double gamma_across(double hi, double d) {
+        const float f = float(d);
+        if (!(f > 1.0e-30f && f < 1.0e30f)) return hi / d;
+        const double y = double(rcp_ftz(f));
+        return hi * fma(y, fma(-d, y, 1.0), y);
+    }
     __device__ __forceinline__ T projected(int a, int b) const { return Y[b * LDA + a]; }
 };
 
