@@ -406,6 +406,7 @@ __global__ void __launch_bounds__(CTAPick<T, S, VARIANT>::threads, CTAPick<T, S,
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ double shr[32 * 6];
     if (FORM != 3 && stopped(d)) return;
+    if (FORM == 3) batch_begin();
     J jac;
     jac.bind(smem);
     const int tid = threadIdx.x;
@@ -666,7 +667,10 @@ __global__ void __launch_bounds__(CTAPick<T, S, VARIANT>::threads, CTAPick<T, S,
         __syncthreads();
         }
     }
-    if (FORM == 3) return;
+    if (FORM == 3) {
+        batch_end();
+        return;
+    }
     if (d.comp_mode) return;
     if (tid == 0) {
         double* pr = d.part + (size_t)(pa.row_off + blockIdx.x) * PART_COLS;

@@ -152,6 +152,7 @@ struct ProjArgs {
     int x_ready;         // Algorithm 1: x was computed by a separate kernel this
                          // iteration (read it) instead of inside the gather
     int min_size;        // standalone launches: smaller orders are left to other kernels
+    int overlap;         // standalone launches: beside the batch's previous kernel (launch_beside)
     int unrolled;        // inside an unrolled pass (derivatives are taken): see BLJacobi
     int cta_variant;     // thread-block projections, float32 orders 36..64: 0 = V in
                          // shared memory (CTAJacobiMid), 1 = V in registers (CTAJacobiReg)
@@ -259,6 +260,13 @@ __device__ __forceinline__ double sparse_dot(const double* __restrict__ val, con
     }
     return s;
 }
+
+// The kernels of one standalone batch work on different blocks and run beside each
+// other (launch_beside): each lets the next one start once its own blocks have,
+// and ends only after the one before it has ended, so that whatever follows the
+// last one on the stream follows all of them.
+__device__ __forceinline__ void batch_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void batch_end() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll

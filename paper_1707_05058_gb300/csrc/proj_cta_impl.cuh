@@ -31,9 +31,8 @@ cudaError_t launch_cta_v(const Dev& d, const int4* list, int nlist, const ProjAr
     ProjArgs pa = pa_in;
     pa.tolrel = jacobi_tolrel(S, sizeof(T) == 4);
     if (FORM == 3) pa.max_sweeps = max_sweeps;
-    k_project_cta<T, S, FORM, VARIANT><<<proj_cta_grid(nlist), Pick::threads, smem, st>>>(d, list, nlist, pa, fa, off,
-                                                                                         size, (const T*)W, (T*)X);
-    return cudaGetLastError();
+    return launch_beside(FORM == 3 && pa.overlap, k_project_cta<T, S, FORM, VARIANT>, proj_cta_grid(nlist),
+                         Pick::threads, smem, st, d, list, nlist, pa, fa, off, size, (const T*)W, (T*)X);
 }
 
 // pa.cta_variant = 1 selects variant 1 (V in registers) for float32 orders
@@ -79,11 +78,12 @@ cudaError_t CTA_SUFFIX(launch_proj_cta)(int S, int form, const Dev& d, const int
 
 #ifdef CTA_STANDALONE
 cudaError_t CTA_SUFFIX(launch_proj_cta_standalone)(int S, int p, const int* off, const int* size, const void* W,
-                                                   void* X, int max_sweeps, cudaStream_t st) {
+                                                   void* X, int max_sweeps, bool overlap, cudaStream_t st) {
     Dev d{};
     ProjArgs pa{};
     FinishArgs fa{};
     pa.restart = 1;
+    pa.overlap = overlap ? 1 : 0;
     pa.min_size = S == 128 ? 97 : (S == 96 ? 65 : kMaxWarpOrder + 1);
     switch (S) {
 #define CTA_CASE(N) \

@@ -45,6 +45,25 @@ inline ProjShape proj_shape(int nlist, int max_warps) {
     return {wpb, grid};
 }
 
+// A kernel of a batch whose others run beside it: with `overlap` it may start
+// once every block of the kernel before it on the stream has started; both call
+// batch_begin() and batch_end() (kernels.cuh).
+template <typename... K, typename... A>
+inline cudaError_t launch_beside(bool overlap, void (*kernel)(K...), int grid, int block, size_t smem, cudaStream_t st,
+                                 A... args) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 inline int proj_class_of(int s) {
     for (int c = 0; c < kNumProjClasses; ++c)
         if (s <= kProjClasses[c]) return c;
@@ -74,7 +93,7 @@ CDSDP_DECLARE_PROJ(f64_large)
     cudaError_t launch_proj_cta_##SUF(int S, int form, const Dev& d, const int4* list, int nlist,               \
                                       const ProjArgs& pa, const FinishArgs& fa, cudaStream_t st);                \
     cudaError_t launch_proj_cta_standalone_##SUF(int S, int p, const int* off, const int* size, const void* W, \
-                                                 void* X, int max_sweeps, cudaStream_t st);
+                                                 void* X, int max_sweeps, bool overlap, cudaStream_t st);
 CDSDP_DECLARE_CTA(f32a)
 CDSDP_DECLARE_CTA(f32b)
 CDSDP_DECLARE_CTA(f32c)
@@ -85,9 +104,9 @@ CDSDP_DECLARE_CTA(f64b)
 // Standalone projection of a batch with device-side orders (proj_ragged.cu):
 // entries of order 1..min(limit, 32), and float entries of order 33..min(limit, 64).
 cudaError_t launch_project_ragged(bool fp32, int p, int limit, const int* off, const int* size, const void* W, void* X,
-                                  int max_sweeps, cudaStream_t st);
+                                  int max_sweeps, bool overlap, cudaStream_t st);
 cudaError_t launch_project_cta_ragged(int p, int limit, const int* off, const int* size, const void* W, void* X,
-                                      int max_sweeps, cudaStream_t st);
+                                      int max_sweeps, bool overlap, cudaStream_t st);
 
 inline cudaError_t launch_proj_cta(bool fp32, int form, int cls, const Dev& d, const int4* list, int nlist,
                                    const ProjArgs& pa, const FinishArgs& fa, cudaStream_t st) {
@@ -101,11 +120,11 @@ inline cudaError_t launch_proj_cta(bool fp32, int form, int cls, const Dev& d, c
 }
 // Float orders above 64 (a class skips orders at or below the one before it), double orders 33..64.
 inline cudaError_t launch_proj_cta_standalone(bool fp32, int cls, int p, const int* off, const int* size,
-                                              const void* W, void* X, int max_sweeps, cudaStream_t st) {
+                                              const void* W, void* X, int max_sweeps, bool overlap, cudaStream_t st) {
     const int S = kProjClasses[cls];
-    if (fp32) return launch_proj_cta_standalone_f32c(S, p, off, size, W, X, max_sweeps, st);
-    return S <= 48 ? launch_proj_cta_standalone_f64a(S, p, off, size, W, X, max_sweeps, st)
-                   : launch_proj_cta_standalone_f64b(S, p, off, size, W, X, max_sweeps, st);
+    if (fp32) return launch_proj_cta_standalone_f32c(S, p, off, size, W, X, max_sweeps, overlap, st);
+    return S <= 48 ? launch_proj_cta_standalone_f64a(S, p, off, size, W, X, max_sweeps, overlap, st)
+                   : launch_proj_cta_standalone_f64b(S, p, off, size, W, X, max_sweeps, overlap, st);
 }
 
 inline cudaError_t launch_proj_f32(int form, int cls, const Dev& d, const int4* list, int nlist, const ProjArgs& pa,
@@ -141,9 +160,10 @@ inline cudaError_t launch_proj_standalone_f32(int cls, int p, const int* off, co
                    : launch_proj_standalone_f32_large(cls, p, off, size, W, X, eig, voff, V, vvoff, tolrel, max_sweeps, st);
     cudaError_t e = cudaSuccess;
     for (int c = cls; e == cudaSuccess && kProjClasses[c] > 64; --c)
-        e = launch_proj_cta_standalone(true, c, p, off, size, W, X, max_sweeps, st);
-    if (e == cudaSuccess && limit > kMaxWarpOrder) e = launch_project_cta_ragged(p, limit, off, size, W, X, max_sweeps, st);
-    if (e == cudaSuccess) e = launch_project_ragged(true, p, limit, off, size, W, X, max_sweeps, st);
+        e = launch_proj_cta_standalone(true, c, p, off, size, W, X, max_sweeps, c < cls, st);
+    if (e == cudaSuccess && limit > kMaxWarpOrder)
+        e = launch_project_cta_ragged(p, limit, off, size, W, X, max_sweeps, limit > 64, st);
+    if (e == cudaSuccess) e = launch_project_ragged(true, p, limit, off, size, W, X, max_sweeps, limit > kMaxWarpOrder, st);
     return e;
 }
 inline cudaError_t launch_proj_standalone_f64(int cls, int p, const int* off, const int* size, const void* W, void* X,
@@ -155,8 +175,8 @@ inline cudaError_t launch_proj_standalone_f64(int cls, int p, const int* off, co
                    ? launch_proj_standalone_f64_small(cls, p, off, size, W, X, eig, voff, V, vvoff, tolrel, max_sweeps, st)
                    : launch_proj_standalone_f64_large(cls, p, off, size, W, X, eig, voff, V, vvoff, tolrel, max_sweeps, st);
     cudaError_t e = cudaSuccess;
-    if (limit > kMaxWarpOrder) e = launch_proj_cta_standalone(false, cls, p, off, size, W, X, max_sweeps, st);
-    if (e == cudaSuccess) e = launch_project_ragged(false, p, limit, off, size, W, X, max_sweeps, st);
+    if (limit > kMaxWarpOrder) e = launch_proj_cta_standalone(false, cls, p, off, size, W, X, max_sweeps, false, st);
+    if (e == cudaSuccess) e = launch_project_ragged(false, p, limit, off, size, W, X, max_sweeps, limit > kMaxWarpOrder, st);
     return e;
 }
 

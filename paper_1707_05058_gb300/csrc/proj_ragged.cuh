@@ -77,6 +77,7 @@ __global__ void __launch_bounds__(32 * kRaggedWarps) k_project_ragged(int p, int
                                                                       T* X, double tolrel, int max_sweeps) {
     __shared__ int entry[32], item_cls[32], item_pos[32], item_n[32];
     __shared__ int n_items, next;
+    batch_begin();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (warp == 0) {
         const int k = blockIdx.x * run + lane;
@@ -124,11 +125,12 @@ __global__ void __launch_bounds__(32 * kRaggedWarps) k_project_ragged(int p, int
         }
 #undef CDSDP_ITEM
     }
+    batch_end();
 }
 
 template <typename T, int SMAX>
 cudaError_t launch_ragged(int p, int limit, const int* off, const int* size, const void* W, void* X, double tolrel,
-                          int max_sweeps, cudaStream_t st) {
+                          int max_sweeps, bool overlap, cudaStream_t st) {
     // entries per thread block: two thread blocks per SM where the batch
     // reaches that far (fewer leaves SMs idle, more leaves nothing to sort)
     const int run = std::max(1, std::min(32, (p + 2 * 152 - 1) / (2 * 152)));
@@ -136,9 +138,8 @@ cudaError_t launch_ragged(int p, int limit, const int* off, const int* size, con
     cudaError_t e = cudaFuncSetAttribute(k_project_ragged<T, SMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    k_project_ragged<T, SMAX><<<(p + run - 1) / run, 32 * kRaggedWarps, smem, st>>>(
-        p, run, limit, off, size, (const T*)W, (T*)X, tolrel, max_sweeps);
-    return cudaGetLastError();
+    return launch_beside(overlap, k_project_ragged<T, SMAX>, (p + run - 1) / run, 32 * kRaggedWarps, smem, st, p, run,
+                         limit, off, size, (const T*)W, (T*)X, tolrel, max_sweeps);
 }
 
 // ---- orders 33..64 -------------------------------------------------------------
@@ -184,6 +185,7 @@ __global__ void __launch_bounds__(kRaggedCtaThreads, 3) k_project_cta_ragged(int
                                                                              const float* W, float* X, double tolrel,
                                                                              int max_sweeps) {
     __shared__ double shr[32];
+    batch_begin();
     for (int k = blockIdx.x; k < p; k += gridDim.x) {
         const int s = size_arr[k];
         if (s <= kMaxWarpOrder || s > limit) continue;  // block-uniform
@@ -200,6 +202,7 @@ __global__ void __launch_bounds__(kRaggedCtaThreads, 3) k_project_cta_ragged(int
             case 16: project_block<64>(shr, s, w, x, tolrel, max_sweeps); break;
         }
     }
+    batch_end();
 }
 
 }  // namespace cdsdp_dev
