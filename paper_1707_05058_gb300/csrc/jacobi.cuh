@@ -154,10 +154,27 @@ __device__ __forceinline__ void rotation(double app, double aqq, double apq, dou
 // The same rotation through tan(theta) (Rutishauser's form of the 2x2 Schur
 // step), for the smallest orders, where few rotations make each one's rounding
 // show: 1,024 random blocks of order 2, 3 and 4 came out 0.81, 1.44 and 1.85
-// u ||W||_F off with the half-angle form in float and 0.69, 1.38 and 1.78 with
-// this one (order 5: 2.21 and 2.28); in double order 2 0.77 and 0.68, since an
-// angle in float32 takes it two rotations, and no difference above.  And, with
-// sc = 1, for the unrolled passes: a derivative through the projections jumps
+// u ||W||_F off with the half-angle form in float and 0.69, 1.38 and 1.78 through
+// the tangent (order 5: 2.21 and 2.28); in double order 2 0.77 and 0.68, since an
+// angle in float32 takes it two rotations, and no difference above.
+// float: three special functions on the chain and no branch; the entries are of
+// order one with sc, and 1/(1 + c) is found as in rotation().
+__device__ __forceinline__ void rotation_small(float app, float aqq, float apq, float tol, float sc, float& tau,
+                                               float& sn, float& ta) {
+    const float zeta = (aqq - app) * (0.5f * sc), q = apq * sc;
+    const float r2 = zeta * zeta + q * q;
+    const float t = copysignf(1.0f, zeta) * q * rcp_ftz(fabsf(zeta) + r2 * rsqrt_ftz(r2));
+    const float c = rsqrt_ftz(1.0f + t * t);
+    const float d = 1.0f + c;
+    float y = (0.1577689f * d - 0.8772993f) * d + 1.623585f;
+    y += y * (1.0f - d * y);
+    const bool on = fabsf(apq) > tol;
+    const float s = t * c;
+    sn = on ? s : 0.0f;
+    tau = on ? s * y : 0.0f;
+    ta = on ? t * apq : 0.0f;
+}
+// And, with sc = 1, for the unrolled passes: a derivative through the projections jumps
 // where an eigenvalue changes sign, so gradients are only comparable between
 // builds while the projections round alike, and these kept their arithmetic
 // when the half-angle form above replaced it in the solves.
@@ -247,7 +264,7 @@ struct BLJacobi {
     using RR = RoundRobin<S>;
     // order 2: one rotation leaves an exact zero, so the diagonal alone is P(W)
     static constexpr bool DIAG = TAN || S == 2;
-    static constexpr bool EXACT = TAN || S <= (sizeof(T) == 4 ? 4 : 2);  // rotation_tan
+    static constexpr bool EXACT = TAN || S <= (sizeof(T) == 4 ? 4 : 2);  // through tan(theta)
     static constexpr int K = S / 2;
     static constexpr int R = S - 1;
     // row pitch: rows start on 16 bytes and eight consecutive rows read as
@@ -533,7 +550,8 @@ struct BLJacobi {
         if (V_STEP) rotate_v<1 - B>(vin, vout);
         // rotation of pair `lane` (lanes < K own the diagonal blocks in slot 0)
         T tau, sn, ta;
-        if constexpr (EXACT) rotation_tan(bv[0][0], bv[0][3], bv[0][1], tol, TAN ? T(1) : sc, tau, sn, ta);
+        if constexpr (EXACT && !TAN && sizeof(T) == 4) rotation_small(bv[0][0], bv[0][3], bv[0][1], tol, sc, tau, sn, ta);
+        else if constexpr (EXACT) rotation_tan(bv[0][0], bv[0][3], bv[0][1], tol, TAN ? T(1) : sc, tau, sn, ta);
         else rotation(bv[0][0], bv[0][3], bv[0][1], tol, sc, tau, sn, ta);
         if (lane < K) rot[B * K + lane] = P2{tau, sn};
         const bool schur = (EXACT || sizeof(T) == 4) && lane < K && sn != T(0);

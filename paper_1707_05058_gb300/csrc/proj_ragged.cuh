@@ -3,7 +3,7 @@
 // the solver makes on the host is made here by each thread block or warp.
 //
 // Orders <= 32 (k_project_ragged): a thread block takes a run of consecutive
-// batch entries, sorts them by padded order (2, then steps of 4) with warp ballots and
+// batch entries, sorts them by padded order (steps of 4) with warp ballots and
 // lets its four warps draw work items, largest orders first: one block per
 // warp above order 16, two at orders 9..16 and four up to 8 (BLJacobi's lane
 // groups).  Before, every block of the batch ran at the padded order of the
@@ -82,10 +82,11 @@ __global__ void __launch_bounds__(32 * kRaggedWarps) k_project_ragged(int p, int
     if (warp == 0) {
         const int k = blockIdx.x * run + lane;
         const int s = lane < run && k < p ? size_arr[k] : 0;
-        const int cls = s < 1 || s > limit ? -1 : (s <= 2 ? 0 : (s + 3) / 4);  // padded order 4 cls, or 2
+        // padded order 4 cls; in double order 2 by itself (0), whose rotation is exact (jacobi.cuh)
+        const int cls = s < 1 || s > limit ? -1 : (sizeof(T) == 8 && s <= 2 ? 0 : (s + 3) / 4);
         int pos0 = 0, it0 = 0;
 #pragma unroll
-        for (int c = SMAX / 4; c >= 0; --c) {
+        for (int c = SMAX / 4; c >= (sizeof(T) == 8 ? 0 : 1); --c) {
             const unsigned mask = __ballot_sync(0xffffffffu, cls == c);
             const int n = __popc(mask), G = 32 / proj_lanes(c ? 4 * c : 2);
             if (cls == c) {
@@ -120,7 +121,7 @@ __global__ void __launch_bounds__(32 * kRaggedWarps) k_project_ragged(int p, int
             }
         }
         switch (item_cls[it]) {
-            case 0: project_item<T, 2>(ws, ks, n, off_arr, size_arr, W, X, tolrel, max_sweeps); break;
+            case 0: if constexpr (sizeof(T) == 8) project_item<T, 2>(ws, ks, n, off_arr, size_arr, W, X, tolrel, max_sweeps); break;
             CDSDP_ITEM(1) CDSDP_ITEM(2) CDSDP_ITEM(3) CDSDP_ITEM(4)
         }
 #undef CDSDP_ITEM
