@@ -460,7 +460,7 @@ int cdsdp_psd_project(int p, const int* d_off, const int* d_size, int max_size,
  * buffer d_gws (cdsdp_grad_workspace_bytes); the backward replays each
  * segment from its checkpoint, recording the eigendecompositions, and runs the
  * reverse pass: the Daleckii-Krein adjoint of every clique projection on the
- * GPU (eigenpairs recomputed by the same Jacobi), the linear steps transposed.
+ * GPU (with the eigenpairs that the replay recorded), the linear steps transposed.
  * Warm start is off and the solve never stops early, so the replay repeats
  * the forward bit for bit.  Only opts->rho, precision and jacobi_max_sweeps
  * are used.  Cliques of order > 32 return CDSDP_ERR_UNSUPPORTED; ckpt_every

@@ -33,7 +33,7 @@
 // floor and stops.
 // In a solve the sweeps end before that: what is rebuilt is P(W) to first order
 // in the remaining off-diagonal part (project()), and a sweep is left out once
-// the second-order remainder is bounded by a quarter of tol (run()).
+// an estimate of what that leaves out is at most a quarter of tol (run()).
 // Warm start (ADMM iterates move little between iterations): each clique keeps
 // its eigenvectors V from the previous iteration; the new block W is first
 // rotated into that basis (A = V^T W V, two warp-level products) and the
@@ -634,12 +634,15 @@ struct BLJacobi {
     // entry exceeds tol = tolrel ||W||_F; nrm2 = ||W||_F^2 as summed.
     //
     // theta > 0 lets the sweeps end earlier, for callers that rebuild with
-    // project(): that takes the remaining off-diagonal part to first order, and
-    // what it leaves out is of second order.  With A = diag(l) + F the bound
-    // sum over i < j of F_ij^2 / (|l_i| + |l_j|) was never below the error of
-    // that expansion in float64 emulations (random blocks of order 5..100, and
-    // the blocks of banded, block-arrow and batched solves; it was 1.02 to 5
-    // times the error in half of them), so the sweeps end once it is at most
+    // project(): that takes the remaining off-diagonal part to first order.  With
+    // A = diag(l) + F the second-order term of P(A) is sum over k of F_ik F_kj
+    // f[l_i, l_k, l_j], f = max(., 0), whose divided difference is at most
+    // 1 / sqrt((|l_i| + |l_k|)(|l_k| + |l_j|)): with G_ij = |F_ij| / sqrt(|l_i| +
+    // |l_j|) the term is at most |G|_F^2 = 2 sum over i < j of F_ij^2 / (|l_i| +
+    // |l_j|).  That bounds this term only; of the whole error the sum was an
+    // estimate from above in float64 replays (never below it on random blocks of
+    // order 5..100 and on the blocks of banded, block-arrow and batched solves,
+    // 1.02 to 5 times it in half of them).  The sweeps end once the sum is at most
     // theta ||W||_F.  In a solve whose clique blocks move little between
     // iterations this takes one sweep or none from the previous iteration's
     // eigenvectors, where reaching tol takes two or three.

@@ -5,9 +5,9 @@
 // round-robin permutation sigma after every round), the 2x2 symmetric Schur
 // step and rotations in Rutishauser's form (tau = s / (1 + c)), warm start from
 // the clique's previous eigenvectors, stagnation stop at the rounding-noise
-// floor.  The arithmetic of every rotation and of every updated entry of A is
-// that of CTAJacobiMid; what changes is where the data live and how a round
-// is synchronised.
+// floor.  Every updated entry of A is formed as in CTAJacobiMid, the rotations
+// by rotation() of jacobi.cuh (half-angle form); what else changes is where the
+// data live and how a round is synchronised.
 //
 //  * A (lower triangle, physical layout of CTAJacobiMid: even storage indices
 //    first, then odd ones) is double-buffered in shared memory; each thread

@@ -9,8 +9,8 @@
 //    swizzle), one mbarrier per stage with the transaction byte count, and after
 //    them the tile of C as one more stage;
 //  * thread 0 of warp 1 issues tcgen05.mma kind::f16 (M = 128, K = 16):
-//    three products per K step into two float32 accumulators in tensor memory
-//    (hi hi; hi lo + lo hi), and frees a stage with tcgen05.commit on that stage's "empty" mbarrier;
+//    two a K step, A_hi [B_hi; B_lo] into two float32 accumulators in tensor
+//    memory (hi hi; hi lo) and A_lo B_hi into the second, and frees a stage with tcgen05.commit on that stage's "empty" mbarrier;
 //  * the warps read the accumulator back (tcgen05.ld 32x32b, one row per
 //    thread, the columns split between the two groups of four warps), apply
 //    D = alpha acc + beta C, split D into its (hi, lo) pair and lay the tile and

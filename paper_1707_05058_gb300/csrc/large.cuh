@@ -25,7 +25,7 @@
 // B_lo + A_lo B_hi), both sums accumulated in float32, each in its own columns of
 // tensor memory.  Every operand is a power of X_0 or a polynomial of it with
 // eigenvalues below 4, so 2^12 x stays below the float16 range, and an entry
-// keeps its 22 bits down to 1.5e-8 (an absolute 2^-37 below that).
+// keeps its 22 bits down to 1.5e-8 (an absolute 2^-48 below that).
 // Every such matrix is stored as its (hi, lo) pair, row-major, block k at a
 // 256-byte aligned offset with row pitch S_k = ceil(s_k / 128) * 128 (zero
 // padding stays zero under odd polynomials); W itself and P stay float32.
