@@ -516,7 +516,7 @@ def _completion(cdsdp, workloads, torch, stream):
         vc, _ = P.components()
         sizes = np.bincount(vc)
         out.update({"n": int(prob.n), "components": int(P.info["ncomp"]), "dense_doubles": int(we),
-                    "step_launches": int(sizes.max()) - 1})
+                    "recurrence_steps": int(sizes.max()) - 1})
         res[key] = out
     return res
 
