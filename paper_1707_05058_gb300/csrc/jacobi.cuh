@@ -587,33 +587,50 @@ struct BLJacobi {
     }
 
     // fro = ||W||_F and sc = 1 / ||W||_F (0 for a zero block: nothing to rotate
-    // there) from its square; sc only brings entries to order one, so in double a
-    // float32 root serves, without the hundreds of cycles of a float64 root and
-    // division.  Entries whose squares leave the range of T are scaled by the
-    // largest one first (X holds the block, or V^T W V, in both triangles): a block
-    // of entries near 1e-24 would otherwise read as a zero block.
-    __device__ __forceinline__ void norm(T nrm2, bool active, int lane, T& fro, T& sc) const {
+    // there) from its square; sc only brings entries to order one.
+    // float: a block whose squares leave the type's range takes a fixed scale, at
+    // which its entries' squares are normal numbers, the lower end of the norm for
+    // the threshold (0 below 1e-18, 3e18 above that), and no theta, so that it is
+    // swept to single entries: read as a zero block, one of entries near 1e-24 came
+    // back unprojected.
+    // double: a float32 root serves for sc, without the hundreds of cycles of a
+    // float64 root and division.  Blocks beyond 1e-145 and 1e145 are scaled by
+    // their largest entry (X holds the block in both triangles) where WIDE is set:
+    // the standalone kernels; in the solves its registers cost k_project_dual<double,
+    // 16> 3% in spills.
+    template <bool WIDE>
+    __device__ __forceinline__ void norm(T nrm2, bool active, int lane, T& fro, T& sc, float& theta) const {
         if (TAN) {
             fro = sqrt(nrm2);
             sc = T(1);
             return;
         }
-        constexpr T lo = sizeof(T) == 4 ? T(1e-30) : T(1e-290), hi = sizeof(T) == 4 ? T(1e37) : T(1e290);
-        if (sizeof(T) == 8 && nrm2 > T(1e-30) && nrm2 < T(1e30)) {
+        if constexpr (sizeof(T) == 4) {
+            fro = sqrt(nrm2);
+            sc = 1.0f / fro;
+            if (!(nrm2 >= 1.0e-36f && nrm2 <= 1.0e37f)) {
+                fro = nrm2 < 1.0f ? 0.0f : 3.0e18f;
+                sc = nrm2 < 1.0f ? 1.0e30f : 1.0e-30f;
+                theta = -1.0f;
+            }
+            return;
+        }
+        if (nrm2 > T(1e-30) && nrm2 < T(1e30)) {
             sc = T(rsqrt_ftz(float(nrm2)));
             fro = nrm2 * sc;
         } else {
             fro = sqrt(nrm2);
             sc = nrm2 > T(0) ? T(1) / fro : T(0);
         }
-        const bool out = active && !(nrm2 >= lo && nrm2 <= hi);
+        if (!WIDE) return;
+        const bool out = active && !(nrm2 >= T(1e-290) && nrm2 <= T(1e290));
         if (!__any_sync(0xffffffffu, out)) return;
         T m = T(0), s = T(0);
 #pragma unroll 1
         for (int i = lane; i < S * S; i += LW) m = fmax(m, fabs(X[(i / S) * LDA + i % S]));
         for (int o = LW / 2; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-        // into the middle of the range in two steps, each a power of two away from overflow
-        const T up = m < T(1) ? T(sizeof(T) == 4 ? 1.329227995784916e36 : 1e250) : T(1);
+        // tiny entries are brought up by a constant first, so that 1 / m is finite
+        const T up = m < T(1) ? T(1e250) : T(1);
         const T dn = T(1) / (m * up);
 #pragma unroll 1
         for (int i = lane; i < S * S; i += LW) {
@@ -621,10 +638,10 @@ struct BLJacobi {
             s += x * x;
         }
         for (int o = LW / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (!out || !(s > T(0)) || !(m <= T(sizeof(T) == 4 ? 3.4e38 : 1.7e308))) return;  // zero, NaN, infinite
+        if (!out || !(s > T(0)) || !(m <= T(1.7e308))) return;  // zero, NaN, infinite
         const T root = sqrt(s);
         fro = root * m;
-        sc = fmin(dn / root * up, T(sizeof(T) == 4 ? 3.4e38 : 1.7e308));
+        sc = fmin(dn / root * up, T(1.7e308));
     }
 
     // Diagonalise; returns the number of sweeps run.  Afterwards X holds the
@@ -653,10 +670,11 @@ struct BLJacobi {
     // rotation skipped (threshold +inf): its storage order returns to the
     // identity after each sweep and its matrix and V stay as they were, so each
     // clique's result is the one it gets alone.
+    template <bool WIDE = true>
     __device__ int run(double tolrel, T nrm2, int max_sweeps, int lane, float theta = 0.0f, bool v_preset = false,
                        bool active = true) {
         T fro, sc;
-        norm(nrm2, active, lane, fro, sc);
+        norm<WIDE>(nrm2, active, lane, fro, sc, theta);
         const T tol = T(tolrel) * fro;
         const T noise = tol * T(2 * S);  // 4 S u ||W||_F when tol = 2 u ||W||_F
         if (!v_preset) {
@@ -872,7 +890,7 @@ __global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4)) k_proj
         const double cxk = group_sum(cx, LW);
         __syncwarp();
         if (warm) jac.rotate_into_stored(vc + d.vv_off[k], s, lane);
-        jac.run(pa.tolrel, nrm, pa.max_sweeps, lane, UNROLLED ? 0.0f : float(kThetaSolve * pa.tolrel), warm, active);
+        jac.template run<false>(pa.tolrel, nrm, pa.max_sweeps, lane, UNROLLED ? 0.0f : float(kThetaSolve * pa.tolrel), warm, active);
         if (pa.warm_start) jac.store_basis(vc + d.vv_off[k], s, lane);
         if (UNROLLED && d.estore) {  // the reverse pass takes the eigenvectors and eigenvalues from here
             const int slot = d.ctl[CTL_ITER];
@@ -987,7 +1005,7 @@ __global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4)) k_proj
         nrm = group_sum(nrm, LW);
         __syncwarp();
         if (warm) jac.rotate_into_stored(vc + d.vv_off[k], s, lane);
-        jac.run(pa.tolrel, nrm, pa.max_sweeps, lane, float(kThetaSolve * pa.tolrel), warm, active);
+        jac.template run<false>(pa.tolrel, nrm, pa.max_sweeps, lane, float(kThetaSolve * pa.tolrel), warm, active);
         if (pa.warm_start) jac.store_basis(vc + d.vv_off[k], s, lane);
         jac.project(lane);
         T p0 = 0;  // in the clique state's precision; float64 across cliques
@@ -1089,7 +1107,7 @@ __global__ void __launch_bounds__(32 * proj_max_warps(S, sizeof(T) == 4), S <= 4
         nrm = group_sum(nrm, LW);
         __syncwarp();
         if (warm) jac.rotate_into_stored(vc + d.vv_off[k], s, lane);
-        jac.run(pa.tolrel, nrm, pa.max_sweeps, lane, float(kThetaSolve * pa.tolrel), warm, active);
+        jac.template run<false>(pa.tolrel, nrm, pa.max_sweeps, lane, float(kThetaSolve * pa.tolrel), warm, active);
         if (pa.warm_start) jac.store_basis(vc + d.vv_off[k], s, lane);
         jac.project(lane);
         double p[6] = {0, 0, 0, 0, 0, 0};
